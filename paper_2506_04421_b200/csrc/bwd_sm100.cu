@@ -38,6 +38,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <cstddef>
+
 #include "hmar_common.h"
 #include "launchers.h"
 #include "ptx_sm100.cuh"
@@ -80,12 +82,13 @@ struct __align__(1024) SharedStorage {
     uint64_t dq_full, dq_empty, acc_full, acc_empty;
     BwdWork work[WORK_CACHE];               // the head's work list (its first WORK_CACHE tiles)
     uint32_t tmem_base;
-    int abort_flag;
+    uint32_t gave_up;                       // offset of the barrier whose wait ran out (0: none did)
     // The block's items: n_chunks runs of consecutive items; run c starts at item chunk_item[c] and holds the
     // block's items number chunk_first[c] .. chunk_first[c + 1] - 1.
     int chunk_item[MAX_CHUNKS], chunk_first[MAX_CHUNKS + 1];
     int n_chunks;
 };
+#define AT(field) (base + (uint32_t)offsetof(SharedStorage, field))     // shared-memory address
 
 __device__ __forceinline__ void report_timeout(int* status, int where) {
     if (status != nullptr) {
@@ -222,19 +225,25 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                    const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do,
                    const __grid_constant__ CUtensorMap map_dq, const BwdArgs args) {
-    extern __shared__ uint8_t smem_raw[];
-    SharedStorage& sm = *reinterpret_cast<SharedStorage*>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    // aligned by its declaration, so that every shared-memory address is a constant of the code (one added at run time
+    // costs a register in every role and about 5 % of the code); checked below
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    SharedStorage& sm = *reinterpret_cast<SharedStorage*>(smem_raw);
+    const uint32_t base = smem_u32(&sm);
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
 
     if (args.status != nullptr && *reinterpret_cast<volatile int*>(args.status) != 0) return;
+    if ((base & 1023u) != 0) {
+        if (threadIdx.x == 0) report_timeout(args.status, 0x3FF);
+        return;
+    }
 
     const int L = args.L;
     const int n_work = args.n_work;
 
     if (threadIdx.x == 0) {
-        sm.abort_flag = 0;
+        sm.gave_up = 0;
         for (int b = 0; b < 2; ++b) {
             mbar_init(&sm.k_full[b], 1);
             mbar_init(&sm.k_free[b], 1);
@@ -301,7 +310,11 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         while (n < sm.chunk_first[run] && run > 0) --run;
         return sm.chunk_item[run] + (n - sm.chunk_first[run]);
     };
-    volatile int* abort_flag = &sm.abort_flag;
+    auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
+        if (warp_wait(bar, parity)) return true;
+        if (lane == 0) sm.gave_up = bar - base;
+        return false;
+    };
 
     auto get_work = [&](int g) -> BwdWork {
         const int t = g % n_work;
@@ -338,12 +351,12 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 const int n_steps = steps_of(w);
                 if (item >= 2) {
                     // the buffer held K of the item before the previous one, read by its dQ products
-                    ok = __all_sync(0xffffffffu, mbar_wait(&sm.k_free[item & 1], ((item >> 1) & 1) ^ 1, abort_flag));
-                    if (!ok) { if (lane == 0) report_timeout(args.status, 0x1000); break; }
+                    ok = wait(AT(k_free) + (item & 1) * 8, ((item >> 1) & 1) ^ 1);
+                    if (!ok) break;
                 }
                 if (leader) {
-                    mbar_arrive_expect_tx(&sm.k_full[item & 1], TILE_BYTES);
-                    tma_load_4d(sm.k[item & 1], &map_k, &sm.k_full[item & 1], 0, w.row_begin, head, batch);
+                    bar_expect_tx(AT(k_full) + (item & 1) * 8, TILE_BYTES);
+                    tma_load_4d_at(AT(k) + (item & 1) * TILE_BYTES, &map_k, AT(k_full) + (item & 1) * 8, 0, w.row_begin, head, batch);
                     // the V rows are read by the drain warps a few steps from now: bring them into L2
                     tma_prefetch_4d(&map_v, 0, w.row_begin, head, batch);
                 }
@@ -352,13 +365,13 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     const int slot = gs % NSTAGE;
                     const int q0 = w.q_begin + i * BQ;
                     if (gs >= NSTAGE) {
-                        ok = __all_sync(0xffffffffu, mbar_wait(&sm.q_empty[slot], ((gs / NSTAGE) & 1) ^ 1, abort_flag));
-                        if (!ok) { if (lane == 0) report_timeout(args.status, 0x1100 + i); break; }
+                        ok = wait(AT(q_empty) + (slot) * 8, ((gs / NSTAGE) & 1) ^ 1);
+                        if (!ok) break;
                     }
                     if (leader) {
-                        mbar_arrive_expect_tx(&sm.qdo_full[slot], 2 * TILE_BYTES);
-                        tma_load_4d(sm.q[slot], &map_q, &sm.qdo_full[slot], 0, q0, head, batch);
-                        tma_load_4d(sm.dout[slot], &map_do, &sm.qdo_full[slot], 0, q0, head, batch);
+                        bar_expect_tx(AT(qdo_full) + (slot) * 8, 2 * TILE_BYTES);
+                        tma_load_4d_at(AT(q) + slot * TILE_BYTES, &map_q, AT(qdo_full) + (slot) * 8, 0, q0, head, batch);
+                        tma_load_4d_at(AT(dout) + slot * TILE_BYTES, &map_do, AT(qdo_full) + (slot) * 8, 0, q0, head, batch);
                     }
                     __syncwarp();
                 }
@@ -383,9 +396,8 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 for (int i = 0; i < n_steps; ++i, ++gs) {
                     const int aslot = gs % AUX_STAGES;
                     if (gs >= AUX_STAGES) {
-                        ok = __all_sync(0xffffffffu,
-                                        mbar_wait(&sm.aux_empty[aslot], ((gs / AUX_STAGES) & 1) ^ 1, abort_flag));
-                        if (!ok) { if (lane == 0) report_timeout(args.status, 0x1700 + i); break; }
+                        ok = wait(AT(aux_empty) + (aslot) * 8, ((gs / AUX_STAGES) & 1) ^ 1);
+                        if (!ok) break;
                     }
                     const int q0 = w.q_begin + i * BQ;
                     // all loads first, then the stores: stores to shared memory in between would serialise them
@@ -403,7 +415,7 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         sm.lse2[aslot][t * 32 + lane] = lv[t] * -1.4426950408889634f;
                         sm.delta[aslot][t * 32 + lane] = -dv[t];
                     }
-                    mbar_arrive(&sm.aux_full[aslot]);
+                    bar_arrive(AT(aux_full) + (aslot) * 8);
                 }
             }
         } else if (warp == MMA_WARP) {
@@ -417,27 +429,23 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             //   Y_i = dV,dK of half 1 of step i, then S^T,dP^T of half 1 of step i+1, then dQ_i
             // each preceded by one look at the barriers it depends on (two at a time, both usually complete).
             const bool leader = elect_one();
-            const uint64_t k_mn0 = smem_desc_sw128(smem_u32(sm.k[0]), 1024);    // K as MN-major B of dQ
+            const uint64_t k_mn0 = smem_desc_sw128(AT(k), 1024);    // K as MN-major B of dQ
             // the ring slots and the dS buffers are 16 KB apart: descriptor of slot s = base + s * 1024
-            const uint64_t q_kd0 = smem_desc_sw128(smem_u32(sm.q[0]), 16), do_kd0 = smem_desc_sw128(smem_u32(sm.dout[0]), 16);
-            const uint64_t q_mn0 = smem_desc_sw128(smem_u32(sm.q[0]), 1024), do_mn0 = smem_desc_sw128(smem_u32(sm.dout[0]), 1024);
-            const uint64_t ds_mn0 = smem_desc_sw128(smem_u32(sm.ds[0][0]), TILE_BYTES);
+            const uint64_t q_kd0 = smem_desc_sw128(AT(q), 16), do_kd0 = smem_desc_sw128(AT(dout), 16);
+            const uint64_t q_mn0 = smem_desc_sw128(AT(q), 1024), do_mn0 = smem_desc_sw128(AT(dout), 1024);
+            const uint64_t ds_mn0 = smem_desc_sw128(AT(ds), TILE_BYTES);
             constexpr uint32_t idesc_acc = idesc_bf16_f32(BKV, D, false, true);    // A from TMEM, B MN-major
             constexpr uint32_t idesc_dq = idesc_bf16_f32(BQ, D, true, true);
             bool ok = true;
             int gs = 0;                                         // steps issued so far (ring slot, dQ parity)
             int ng[2] = {0, 0};                                 // gradient halves issued so far, per half
             // waits for barrier a and, if have_b, barrier b; the two first looks overlap
-            auto wait2 = [&](uint64_t* a, uint32_t pa, uint64_t* b, uint32_t pb, bool have_b, int code) -> bool {
-                const bool ra = mbar_try_wait(a, pa);
-                const bool rb = !have_b || mbar_try_wait(b, pb);
-                if (__all_sync(0xffffffffu, ra && rb)) return true;
+            auto wait2 = [&](uint32_t a, uint32_t pa, uint32_t b, uint32_t pb, bool have_b) -> bool {
+                bool ra, rb;
+                warp_try_wait2(a, pa, have_b ? b : a, have_b ? pb : pa, ra, rb);
                 // a barrier seen complete is not looked at again: a look is a shared-memory round trip behind the
                 // compute warps' stores, on the critical path of the step
-                const bool done = (ra || mbar_wait(a, pa, abort_flag)) && (rb || mbar_wait(b, pb, abort_flag));
-                if (__all_sync(0xffffffffu, done)) return true;
-                if (lane == 0) report_timeout(args.status, code);
-                return false;
+                return (ra || wait(a, pa)) && (!have_b || rb || wait(b, pb));
             };
             // S^T_h = K Q_h^T,  dP^T_h = V dO_h^T : n query columns of half h, Q / dO tile in ring slot `slot`
             auto scores = [&](int h, int n, int slot) {
@@ -449,7 +457,7 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 #pragma unroll
                 for (int ks = 0; ks < D / 16; ++ks)
                     mma_ts(tmem + COL_DPT + h * HQ, tmem + COL_V + ks * 8, dd + ks * 2, idesc, ks > 0);
-                tc_commit(&sm.s_full[h]);
+                commit_at(AT(s_full) + (h) * 8);
             };
             // dV += P_h^T dO_h,  dK += dS_h^T Q_h : n query columns of half h
             auto grads = [&](int h, int n, int slot, bool first) {
@@ -465,25 +473,20 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         mma_ts(tmem + COL_DK, tmem + COL_DPT + h * HQ + ks * 8, qd + ks * 128, idesc_acc, !first || (ks > 0));
             };
 
-            auto wait1 = [&](uint64_t* a, uint32_t pa, int code) -> bool {
-                if (__all_sync(0xffffffffu, mbar_wait(a, pa, abort_flag))) return true;
-                if (lane == 0) report_timeout(args.status, code);
-                return false;
-            };
             // The steps of all items form one sequence: while the compute warpgroups work on a step, the
             // tensor core gets the next step's S^T, dP^T even when that step belongs to the next item (whose
             // K, V rows the drain warps have put into TMEM by then).
             int run = 0;
             if (n_items > 0) {
                 const BwdWork w0 = get_work(item_at(0, run));
-                ok = wait2(&sm.kv_tmem, 0, &sm.qdo_full[0], 0, true, 0x1200);
+                ok = wait2(AT(kv_tmem), 0, AT(qdo_full) + (0) * 8, 0, true);
                 if (ok) {
                     tc_fence_after();
                     if (leader) {
                         scores(0, half_cols(w0, 0, 0), 0);
                         const int n1 = half_cols(w0, 0, 1);
                         if (n1 > 0) scores(1, n1, 0);
-                        if (steps_of(w0) == 1 && 1 < n_items) tc_commit(&sm.kv_free);
+                        if (steps_of(w0) == 1 && 1 < n_items) commit_at(AT(kv_free));
                     }
                     __syncwarp();
                 }
@@ -506,15 +509,15 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     // the next step is the last one that reads its item's K, V rows in TMEM, and another item follows
                     const bool frees_kv = more ? (i + 2 == n_steps && next_item) : (cross && n_steps_next == 1 && item + 2 < n_items);
                     // ---- burst X: needs P^T, dS^T of half 0 and the next step's Q / dO tile
-                    ok = wait2(&sm.p_full[0], ng[0] & 1, &sm.qdo_full[slot_next], ((gs + 1) / NSTAGE) & 1, any_next, 0x1400 + i);
+                    ok = wait2(AT(p_full) + (0) * 8, ng[0] & 1, AT(qdo_full) + (slot_next) * 8, ((gs + 1) / NSTAGE) & 1, any_next);
                     if (!ok) break;
                     ++ng[0];
                     if (cross) {                                // K, V of the next item in TMEM
-                        ok = wait1(&sm.kv_tmem, (item + 1) & 1, 0x1200);
+                        ok = wait(AT(kv_tmem), (item + 1) & 1);
                         if (!ok) break;
                     }
                     if (i == 0 && item > 0) {                   // dK, dV of the previous item read out
-                        ok = wait1(&sm.acc_empty, (item - 1) & 1, 0x1B00);
+                        ok = wait(AT(acc_empty), (item - 1) & 1);
                         if (!ok) break;
                     }
                     tc_fence_after();
@@ -526,33 +529,33 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     // ---- burst Y: needs P^T, dS^T of half 1 (if the step has one) and dQ of the previous
                     // step drained from TMEM
                     if (n1 > 0) {
-                        ok = wait2(&sm.p_full[1], ng[1] & 1, &sm.dq_empty, (gs - 1) & 1, gs > 0, 0x1800 + i);
+                        ok = wait2(AT(p_full) + (1) * 8, ng[1] & 1, AT(dq_empty), (gs - 1) & 1, gs > 0);
                         ++ng[1];
                     } else if (gs > 0) {
-                        ok = wait2(&sm.dq_empty, (gs - 1) & 1, nullptr, 0, false, 0x1800 + i);
+                        ok = wait(AT(dq_empty), (gs - 1) & 1);
                     }
                     if (!ok) break;
                     if (i == 0) {                               // K of this item in shared memory (B operand of dQ)
-                        ok = wait1(&sm.k_full[item & 1], (item >> 1) & 1, 0x1C00);
+                        ok = wait(AT(k_full) + (item & 1) * 8, (item >> 1) & 1);
                         if (!ok) break;
                     }
                     tc_fence_after();
                     if (leader) {
                         if (n1 > 0) grads(1, n1, slot, false);
-                        tc_commit(&sm.q_empty[slot]);           // Q_i, dO_i are not read again
-                        if (!more) tc_commit(&sm.acc_full);     // dK, dV of the item are complete
+                        commit_at(AT(q_empty) + (slot) * 8);           // Q_i, dO_i are not read again
+                        if (!more) commit_at(AT(acc_full));     // dK, dV of the item are complete
                         // the next scores of half 1 go first: the compute warpgroup is waiting for them, dQ_i
                         // is not needed before the drain warps get to it
                         if (m1 > 0) scores(1, m1, slot_next);
-                        if (frees_kv) tc_commit(&sm.kv_free);
+                        if (frees_kv) commit_at(AT(kv_free));
                         // dQ_i = dS K over both halves: A = dS (queries x keys) read as an MN-major operand.  When
                         // the step has no second half its rows are stale data and are never drained.
                         const uint64_t dsd = ds_mn0 + (gs & 1) * 2048;
 #pragma unroll
                         for (int ks = 0; ks < BKV / 16; ++ks)
                             mma_ss(tmem + COL_DQ, dsd + ks * 128, k_mn + ks * 128, idesc_dq, ks > 0);
-                        tc_commit(&sm.dq_full);
-                        if (!more) tc_commit(&sm.k_free[item & 1]);
+                        commit_at(AT(dq_full));
+                        if (!more) commit_at(AT(k_free) + (item & 1) * 8);
                     }
                     __syncwarp();
                 }
@@ -575,11 +578,6 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         uint32_t buf[32];
         bool ok = true;
         int gs = 0;
-        auto wait1 = [&](uint64_t* a, uint32_t pa, int code) -> bool {
-            if (__all_sync(0xffffffffu, mbar_wait(a, pa, abort_flag))) return true;
-            if (lane == 0) report_timeout(args.status, code);
-            return false;
-        };
         // K and V rows of item gc (the block's item number `item`) to TMEM, one key row per thread: the A
         // operands of S^T = K Q^T and dP^T = V dO^T.  The V row comes straight from global memory and waits
         // in registers until the previous item's last scores have been computed; the K row is read from the
@@ -603,16 +601,16 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 buf[4 * c] = val.x; buf[4 * c + 1] = val.y; buf[4 * c + 2] = val.z; buf[4 * c + 3] = val.w;
             }
             if (wait_free) {
-                if (!wait1(&sm.kv_free, (item - 1) & 1, 0x1900)) return false;
+                if (!wait(AT(kv_free), (item - 1) & 1)) return false;
                 tc_fence_after();
             }
             tmem_st32(lane_base + COL_V, buf);
-            if (!wait1(&sm.k_full[item & 1], (item >> 1) & 1, 0x1980)) return false;
+            if (!wait(AT(k_full) + (item & 1) * 8, (item >> 1) & 1)) return false;
             load_swizzled_row(sm.k[item & 1], r, buf);
             tmem_st32(lane_base + COL_K, buf);
             tmem_st_wait();
             tc_fence_before();
-            mbar_arrive(&sm.kv_tmem);
+            bar_arrive(AT(kv_tmem));
             return true;
         };
         int run = 0;
@@ -638,7 +636,7 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 }
                 if (!more) {
                     // ---- end of the item: dK and dV, one key row per thread, scaled and rounded to bf16
-                    ok = wait1(&sm.acc_full, item & 1, 0x1A00);
+                    ok = wait(AT(acc_full), item & 1);
                     if (!ok) break;
                     tc_fence_after();
 #pragma unroll
@@ -647,7 +645,7 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         tmem_ld_wait();
                         if (part == 3) {
                             tc_fence_before();
-                            mbar_arrive(&sm.acc_empty);         // the next item's products may overwrite dK / dV
+                            bar_arrive(AT(acc_empty));         // the next item's products may overwrite dK / dV
                         }
                         if (r < w.row_count) {
                             const float mul = part < 2 ? args.softmax_scale : 1.f;
@@ -674,11 +672,8 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         }
                     }
                 }
-                if (!__all_sync(0xffffffffu, mbar_wait(&sm.dq_full, gs & 1, abort_flag))) {
-                    if (lane == 0) report_timeout(args.status, 0x1600 + i);
-                    ok = false;
-                    break;
-                }
+                ok = wait(AT(dq_full), gs & 1);
+                if (!ok) break;
                 tc_fence_after();
                 const int q0 = w.q_begin + i * BQ;
                 const bool row_in = r < min(BQ, w.q_end - q0);
@@ -688,7 +683,7 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     tmem_ld_wait();
                     if (c == 1) {
                         tc_fence_before();
-                        mbar_arrive(&sm.dq_empty);
+                        bar_arrive(AT(dq_empty));
                     }
                     // the previous piece must have been read out of the staging buffer
                     if (lane == 0) bulk_wait_read_all();
@@ -749,12 +744,12 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 const int cbase = h * HQ;                   // first query column of this half inside the step
 
                 const int aslot = gs % AUX_STAGES;
-                ok = __all_sync(0xffffffffu, mbar_wait(&sm.aux_full[aslot], (gs / AUX_STAGES) & 1, abort_flag));
-                if (!ok) { if (lane == 0) report_timeout(args.status, 0x1500 + i); break; }
+                ok = wait(AT(aux_full) + (aslot) * 8, (gs / AUX_STAGES) & 1);
+                if (!ok) break;
 
                 if (n_cols > 0) {
-                    ok = __all_sync(0xffffffffu, mbar_wait(&sm.s_full[h], nsh & 1, abort_flag));
-                    if (!ok) { if (lane == 0) report_timeout(args.status, 0x1580 + i); break; }
+                    ok = wait(AT(s_full) + (h) * 8, nsh & 1);
+                    if (!ok) break;
                     ++nsh;
                     tc_fence_after();
                     // tiles whose rows all see every column skip the mask code
@@ -779,9 +774,9 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     tmem_st_wait();
                     tc_fence_before();
                     fence_proxy_async_smem();
-                    mbar_arrive(&sm.p_full[h]);
+                    bar_arrive(AT(p_full) + (h) * 8);
                 }
-                mbar_arrive(&sm.aux_empty[aslot]);      // this thread is done with the step's lse / delta
+                bar_arrive(AT(aux_empty) + (aslot) * 8);      // this thread is done with the step's lse / delta
             }
         }
     }
@@ -792,6 +787,7 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         tc_fence_after();
         tmem_dealloc(tmem, TMEM_COLS);
     }
+    if (threadIdx.x == 0 && sm.gave_up != 0) report_timeout(args.status, (int)sm.gave_up);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -879,7 +875,7 @@ template <bool STRIDED>
 static cudaError_t launch_bwd_tc_layout(const CUtensorMap& q, const CUtensorMap& k, const CUtensorMap& v, const CUtensorMap& dout_map,
                                         const CUtensorMap& dq_acc_map, const BwdArgs& args, const __nv_bfloat16* out,
                                         const __nv_bfloat16* dout, __nv_bfloat16* dq, int BH, cudaStream_t stream) {
-    const size_t smem = sizeof(SharedStorage) + 1024;
+    const size_t smem = sizeof(SharedStorage);
     cudaError_t e = cudaFuncSetAttribute(hmar_bwd_tc_kernel<false, STRIDED, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(hmar_bwd_tc_kernel<true, STRIDED, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
