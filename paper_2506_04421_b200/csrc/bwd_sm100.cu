@@ -143,7 +143,10 @@ __device__ __forceinline__ void load_swizzled_row(const uint8_t* tile, int r, ui
 // holds another tile's keys; its P^T and dS^T only reach rows of dV and dK that are never written, but in
 // dQ = dS K it would be summed over, so the copy of dS in shared memory gets zeros there.
 // MODE 0: all rows see all columns.
-template <int MODE>
+// ROLLED: the two halves of the rows are iterations of a loop and not two copies of the code.  Less code, but the compiler
+// no longer mixes one half's stores with the next half's loads: the instantiation for partial and packed tiles is bound
+// by instruction fetch and gains (L = 680: 332 -> 295 us), the one for full tiles loses (L = 2240: 832 -> 849 us).
+template <int MODE, bool ROLLED>
 __device__ __forceinline__ void softmax_grad_half(uint32_t lane_base, int cbase, const float* neg_lse2, const float* neg_delta,
                                                   float sl2, const int (&c_lo)[4], const int (&c_hi)[4], uint8_t* ds_tile,
                                                   int quarter, int lane) {
@@ -157,8 +160,9 @@ __device__ __forceinline__ void softmax_grad_half(uint32_t lane_base, int cbase,
         nde[k] = *reinterpret_cast<const uint64_t*>(neg_delta + cbase + 8 * k + 2 * tq);
     }
     const uint64_t sl2_2 = f32x2(sl2, sl2);
-#pragma unroll
+#pragma unroll (ROLLED ? 1 : 2)
     for (int hl = 0; hl < 2; ++hl) {                    // lanes 0-15, then 16-31 of the warp's quarter
+        const int lo2[2] = {hl ? c_lo[2] : c_lo[0], hl ? c_lo[3] : c_lo[1]}, hi2[2] = {hl ? c_hi[2] : c_hi[0], hl ? c_hi[3] : c_hi[1]};
         const uint32_t taddr = lane_base + ((uint32_t)(hl * 16) << 16);
         uint32_t s_buf[32], dp_buf[32];
         tmem_ld_16x256b_x8(taddr + COL_ST + cbase, s_buf);
@@ -176,9 +180,9 @@ __device__ __forceinline__ void softmax_grad_half(uint32_t lane_base, int cbase,
                                   sl2_2, nls[k]), x0, x1);
                 float p0 = ex2(x0), p1 = ex2(x1);
                 if (MODE == 2) {
-                    const int c = cbase + 8 * k + 2 * tq, i = hl * 2 + rs;
-                    p0 = (c >= c_lo[i] && c < c_hi[i]) ? p0 : 0.f;
-                    p1 = (c + 1 >= c_lo[i] && c + 1 < c_hi[i]) ? p1 : 0.f;
+                    const int c = cbase + 8 * k + 2 * tq;
+                    p0 = (c >= lo2[rs] && c < hi2[rs]) ? p0 : 0.f;
+                    p1 = (c + 1 >= lo2[rs] && c + 1 < hi2[rs]) ? p1 : 0.f;
                 }
                 float d0, d1;
                 f32x2_split(fmul2(f32x2(p0, p1),
@@ -188,7 +192,7 @@ __device__ __forceinline__ void softmax_grad_half(uint32_t lane_base, int cbase,
                 ds_pack[2 * k + rs] = pack_bf16(d0, d1);
                 // 8-row groups are 1024 bytes apart; 16-byte piece k of a row sits at position k ^ (row & 7)
                 *reinterpret_cast<uint32_t*>(ds_row + rs * 1024 + ((k ^ tr) << 4)) =
-                    (MODE == 1 && c_hi[hl * 2 + rs] <= 0) ? 0u : ds_pack[2 * k + rs];
+                    (MODE == 1 && hi2[rs] <= 0) ? 0u : ds_pack[2 * k + rs];
             }
         }
         tmem_st_16x128b_x8(taddr + COL_ST + cbase, p_pack);
@@ -761,14 +765,14 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                             c_hi[r4] = min(qhi[r4] - q0, n_valid);
                         }
                         if (rows_only)
-                            softmax_grad_half<1>(lane_base, cbase, sm.lse2[aslot], sm.delta[aslot], sl2, c_lo, c_hi,
+                            softmax_grad_half<1, ONE_MASK>(lane_base, cbase, sm.lse2[aslot], sm.delta[aslot], sl2, c_lo, c_hi,
                                                  sm.ds[gs & 1][h], quarter, lane);
                         else
-                            softmax_grad_half<2>(lane_base, cbase, sm.lse2[aslot], sm.delta[aslot], sl2, c_lo, c_hi,
+                            softmax_grad_half<2, ONE_MASK>(lane_base, cbase, sm.lse2[aslot], sm.delta[aslot], sl2, c_lo, c_hi,
                                                  sm.ds[gs & 1][h], quarter, lane);
                     } else {
                         const int none[4] = {0, 0, 0, 0};
-                        softmax_grad_half<0>(lane_base, cbase, sm.lse2[aslot], sm.delta[aslot], sl2, none, none,
+                        softmax_grad_half<0, ONE_MASK>(lane_base, cbase, sm.lse2[aslot], sm.delta[aslot], sl2, none, none,
                                                  sm.ds[gs & 1][h], quarter, lane);
                     }
                     tmem_st_wait();
