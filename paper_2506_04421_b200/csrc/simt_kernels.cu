@@ -1,9 +1,14 @@
-// Plain SIMT kernels for HMAR's Markovian masked attention: the fp32 debug build, and the bf16
-// fall-back used while debugging the tensor-core kernels.  All arithmetic is fp32 FMA; inputs and
-// outputs are float or bf16.  Two threads share one row, each owning half of the head dimensions.  These
-// kernels are templated on the head dimension (32, 64, 128); the tensor-core kernels exist for 64 only.
+// Plain SIMT kernels for HMAR's Markovian masked attention: the fp32 debug build, the path of head dimensions 32 and 128,
+// and the bf16 fall-back used while debugging the tensor-core kernels.  All arithmetic is fp32 FMA; inputs and outputs
+// are float or bf16.
 //
-// Mask (paper Sec. 4.1, Fig. attn-mask): a query of scale k sees keys [start[k-1], start[k+1]).
+// A block of 128 threads owns a tile of up to 64 rows of ONE scale, so all of its rows see the same contiguous range of
+// the other operand (mask: paper Sec. 4.1, Fig. attn-mask) and no element needs a mask but the ragged end of that range.
+// It walks the range 64 rows at a time, as small dense products from shared memory with 8 x 4 results per thread: 12
+// 16-byte shared-memory loads feed 128 FMAs, which leaves the FMA pipe as the bound (a warp's loads take half of the
+// shared-memory cycles its FMAs last).  One row per thread pair, an operand of every FMA from shared memory, was bound
+// by those loads: B2 H16 L680 D64, forward + backward, 954 us, against 70 us of FMAs.
+// Tiles of the last (largest) scale come first in the grid.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include "hmar_common.h"
@@ -12,275 +17,318 @@
 namespace hmar {
 namespace {
 
-constexpr int ROWS = 64;           // rows per block (128 threads)
-constexpr int KT = 32;             // partner rows staged in shared memory per step
+constexpr int TR = 64;             // rows of a tile, on either side
+constexpr int THREADS = 128;       // thread t: rows 8 (t / 16) .. + 7, columns t % 16 + {0, 16, 32, 48} of a 64 x 64 product
 
 __device__ __forceinline__ float to_f(float x) { return x; }
 __device__ __forceinline__ float to_f(__nv_bfloat16 x) { return __bfloat162float(x); }
 __device__ __forceinline__ void from_f(float* p, float x) { *p = x; }
 __device__ __forceinline__ void from_f(__nv_bfloat16* p, float x) { *p = __float2bfloat16_rn(x); }
 
-// Key/value rows of one head may come in two segments (previous scale, then current scale) for the
-// inference step; the training kernels use a single segment.
-template <typename T, int D>
-struct KvView {
-    const T* k0; const T* v0; int n0;
-    const T* k1; const T* v1;
-    __device__ __forceinline__ const T* krow(int j) const {
-        return j < n0 ? k0 + (size_t)j * D : k1 + (size_t)(j - n0) * D;
-    }
-    __device__ __forceinline__ const T* vrow(int j) const {
-        return j < n0 ? v0 + (size_t)j * D : v1 + (size_t)(j - n0) * D;
-    }
-};
+// Four consecutive elements as float.
+__device__ __forceinline__ float4 load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
+    const uint2 v = *reinterpret_cast<const uint2*>(p);
+    return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
+                       __uint_as_float(v.y & 0xffff0000u));
+}
 
+// Rows in shared memory are padded by four floats: 16-byte loads of eight consecutive rows then hit 32 distinct banks.
+template <int D> struct RowTile { float v[TR][D + 4]; };
+struct SquareTile { float v[TR][TR + 4]; };
+
+// dst rows [0, TR) = src rows [0, n) as float; the rest zeros.
 template <typename T, int D>
-__device__ __forceinline__ void stage_rows(float (*dst)[D], const T* src_base, int first, int count) {
-    // dst[r][:] = row (first + r) for r < count; 128 threads, coalesced along D
-    for (int idx = threadIdx.x; idx < count * D; idx += blockDim.x) {
-        int r = idx / D, d = idx % D;
-        dst[r][d] = to_f(src_base[(size_t)(first + r) * D + d]);
+__device__ __forceinline__ void stage(RowTile<D>& dst, const T* src, int n) {
+#pragma unroll 8
+    for (int idx = threadIdx.x; idx < TR * (D / 4); idx += THREADS) {
+        const int r = idx / (D / 4), c = idx % (D / 4) * 4;
+        *reinterpret_cast<float4*>(&dst.v[r][c]) = r < n ? load4(src + (size_t)r * D + c) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
 
-// ---------------------------------------------------------------------------------------------
-// Forward and inference step.  dense != 0: every query row sees all n_kv keys (inference step).
-template <typename T, int D>
-__global__ void __launch_bounds__(128)
-simt_fwd_kernel(const T* __restrict__ q, const T* __restrict__ k0, const T* __restrict__ v0,
-                const T* __restrict__ k1, const T* __restrict__ v1,
-                T* __restrict__ out, float* __restrict__ lse,
-                ScaleTable st, int n_q, int n0, int n1, int dense, float scale) {
-    constexpr int DH = D / 2;          // dimensions per thread
-    __shared__ float sK[KT][D];
-    __shared__ float sV[KT][D];
-    const int bh = blockIdx.y;
-    const int row0 = blockIdx.x * ROWS;
-    const int half = threadIdx.x & 1;
-    const int row_raw = row0 + (threadIdx.x >> 1);
-    const bool row_ok = row_raw < n_q;
-    const int row = row_ok ? row_raw : n_q - 1;
-    const int last_row = min(row0 + ROWS, n_q) - 1;
-
-    KvView<T, D> kv{k0 + (size_t)bh * n0 * D, v0 + (size_t)bh * n0 * D, n0,
-                 k1 ? k1 + (size_t)bh * n1 * D : nullptr, v1 ? v1 + (size_t)bh * n1 * D : nullptr};
-
-    int lo, hi, blk_lo, blk_hi;
-    if (dense) {
-        lo = blk_lo = 0;
-        hi = blk_hi = n0 + n1;
-    } else {
-        int s = scale_of_row(st, row);
-        lo = st.start[first_key_scale(st.window, s)];
-        hi = st.start[last_key_scale(st.window, s) + 1];
-        int sf = scale_of_row(st, row0), sl = scale_of_row(st, last_row);
-        blk_lo = st.start[first_key_scale(st.window, sf)];
-        blk_hi = st.start[last_key_scale(st.window, sl) + 1];
-    }
-
-    float qr[DH], o[DH];
-    const T* qp = q + ((size_t)bh * n_q + row) * D + half * DH;
+// acc[i][j] = sum_d a[r0 + i][d] b[tx + 16 j][d]
+template <int D>
+__device__ __forceinline__ void product_nt(const RowTile<D>& a, const RowTile<D>& b, int r0, int tx, float (&acc)[8][4]) {
 #pragma unroll
-    for (int d = 0; d < DH; ++d) { qr[d] = to_f(qp[d]); o[d] = 0.f; }
-    float m = -INFINITY, l = 0.f;
-
-    for (int t = blk_lo; t < blk_hi; t += KT) {
-        const int cnt = min(KT, blk_hi - t);
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < cnt * D; idx += blockDim.x) {
-            int r = idx / D, d = idx % D;
-            sK[r][d] = to_f(kv.krow(t + r)[d]);
-            sV[r][d] = to_f(kv.vrow(t + r)[d]);
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+#pragma unroll 2
+    for (int d = 0; d < D; d += 4) {
+        float4 bv[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) bv[j] = *reinterpret_cast<const float4*>(&b.v[tx + 16 * j][d]);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float4 av = *reinterpret_cast<const float4*>(&a.v[r0 + i][d]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                acc[i][j] = fmaf(av.w, bv[j].w, fmaf(av.z, bv[j].z, fmaf(av.y, bv[j].y, fmaf(av.x, bv[j].x, acc[i][j]))));
         }
-        __syncthreads();
-        for (int r = 0; r < cnt; ++r) {
-            float s = 0.f;
+    }
+}
+
+// A thread's columns of a [TR x D] result: D / 16 of them, in groups of W consecutive ones that are 16 W apart.
+template <int D> struct Cols {
+    static constexpr int W = D >= 64 ? 4 : 2, GROUPS = D / (16 * W), N = D / 16;
+};
+
+// acc[i][.] += sum_k p[r0 + i][k] b[k][columns of the thread], k < n (a multiple of 4)
+template <int D>
+__device__ __forceinline__ void product_nn(const SquareTile& p, const RowTile<D>& b, int r0, int tx, int n, float (&acc)[8][Cols<D>::N]) {
+    constexpr int W = Cols<D>::W, G = Cols<D>::GROUPS;
+#pragma unroll 2
+    for (int k = 0; k < n; k += 4) {
+        float4 pv[8];
 #pragma unroll
-            for (int d = 0; d < DH; ++d) s = fmaf(qr[d], sK[r][half * DH + d], s);
-            s += __shfl_xor_sync(0xffffffffu, s, 1);
-            s *= scale;
-            const int j = t + r;
-            if (j >= lo && j < hi) {
-                float m_new = fmaxf(m, s);
-                float corr = expf(m - m_new);      // exp(-inf) = 0 on the first key
-                float p = expf(s - m_new);
-                l = l * corr + p;
+        for (int i = 0; i < 8; ++i) pv[i] = *reinterpret_cast<const float4*>(&p.v[r0 + i][k]);
 #pragma unroll
-                for (int d = 0; d < DH; ++d) o[d] = fmaf(o[d], corr, p * sV[r][half * DH + d]);
-                m = m_new;
+        for (int kk = 0; kk < 4; ++kk) {
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                float bv[W];
+                const float* src = &b.v[k + kk][g * 16 * W + tx * W];
+                if (W == 4) {
+                    const float4 x = *reinterpret_cast<const float4*>(src);
+                    bv[0] = x.x; bv[1] = x.y; bv[W - 2] = x.z; bv[W - 1] = x.w;
+                } else {
+                    const float2 x = *reinterpret_cast<const float2*>(src);
+                    bv[0] = x.x; bv[1] = x.y;
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float w = kk == 0 ? pv[i].x : kk == 1 ? pv[i].y : kk == 2 ? pv[i].z : pv[i].w;
+#pragma unroll
+                    for (int e = 0; e < W; ++e) acc[i][g * W + e] = fmaf(w, bv[e], acc[i][g * W + e]);
+                }
             }
         }
     }
-    if (row_ok) {
-        const float inv = 1.f / l;
-        T* op = out + ((size_t)bh * n_q + row) * D + half * DH;
+}
+
+// dst[r][d] = acc * mul for the thread's rows below n
+template <typename T, int D>
+__device__ __forceinline__ void store_rows(T* dst, const float (&acc)[8][Cols<D>::N], const float (&mul)[8], int r0, int tx, int n) {
+    constexpr int W = Cols<D>::W, G = Cols<D>::GROUPS;
 #pragma unroll
-        for (int d = 0; d < DH; ++d) from_f(op + d, o[d] * inv);
-        if (lse != nullptr && half == 0) lse[(size_t)bh * n_q + row] = m + logf(l);
+    for (int i = 0; i < 8; ++i) {
+        if (r0 + i >= n) break;
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+#pragma unroll
+            for (int e = 0; e < W; ++e) from_f(dst + (size_t)(r0 + i) * D + g * 16 * W + tx * W + e, acc[i][g * W + e] * mul[i]);
+    }
+}
+
+// Tile number `t` of a head: rows [row0, row0 + n) of scale s.  Tiles of the last scale come first.
+struct TileRows { int s, row0, n; };
+__device__ __forceinline__ TileRows tile_rows(const ScaleTable& st, int t) {
+    int s = st.n_scales - 1;
+    while (true) {
+        const int rows = st.start[s + 1] - st.start[s], tiles = (rows + TR - 1) / TR;
+        if (t < tiles || s == 0) return {s, st.start[s] + t * TR, min(TR, rows - t * TR)};
+        t -= tiles;
+        --s;
     }
 }
 
 // ---------------------------------------------------------------------------------------------
-// delta_i = sum_d dO_id * O_id
+// Forward and inference step.  The keys are rows [lo, hi) of one sequence, or (inference step: st has one scale, the
+// queries) n0 rows of the previous scale followed by n1 of the current one.
+template <int D> struct FwdSmem { RowTile<D> q, k, v; SquareTile p; };
+
 template <typename T, int D>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(THREADS)
+simt_fwd_kernel(const T* __restrict__ q, const T* __restrict__ k0, const T* __restrict__ v0,
+                const T* __restrict__ k1, const T* __restrict__ v1,
+                T* __restrict__ out, float* __restrict__ lse,
+                const __grid_constant__ ScaleTable st, int n_q, int n0, int n1, int dense, float scale) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    FwdSmem<D>& sm = *reinterpret_cast<FwdSmem<D>*>(smem_raw);
+    const int bh = blockIdx.y;
+    const TileRows tile = tile_rows(st, blockIdx.x);
+    const int tx = threadIdx.x & 15, r0 = (threadIdx.x >> 4) * 8;
+    const bool live = (threadIdx.x >> 5) * 16 < tile.n;     // the warp has rows of the tile
+    const int lo = dense ? 0 : st.start[first_key_scale(st.window, tile.s)];
+    const int hi = dense ? n0 + n1 : st.start[last_key_scale(st.window, tile.s) + 1];
+    const T* kh = k0 + (size_t)bh * n0 * D;
+    const T* vh = v0 + (size_t)bh * n0 * D;
+
+    stage(sm.q, q + ((size_t)bh * n_q + tile.row0) * D, tile.n);
+    float o[8][Cols<D>::N], m[8], l[8];                     // l: this thread's columns only, summed over the row at the end
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        m[i] = -INFINITY;
+        l[i] = 0.f;
+#pragma unroll
+        for (int e = 0; e < Cols<D>::N; ++e) o[i][e] = 0.f;
+    }
+    for (int t = lo; t < hi;) {
+        // the tile does not cross from one segment into the other
+        const bool second = dense && t >= n0;
+        const int n = min(TR, (dense && !second ? n0 : hi) - t);
+        const T* ks = second ? k1 + ((size_t)bh * n1 + (t - n0)) * D : kh + (size_t)t * D;
+        const T* vs = second ? v1 + ((size_t)bh * n1 + (t - n0)) * D : vh + (size_t)t * D;
+        __syncthreads();
+        stage(sm.k, ks, n);
+        stage(sm.v, vs, n);
+        __syncthreads();
+        if (live) {
+            float s[8][4];
+            product_nt(sm.q, sm.k, r0, tx, s);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                float mx = -INFINITY;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    s[i][j] = tx + 16 * j < n ? s[i][j] * scale : -INFINITY;
+                    mx = fmaxf(mx, s[i][j]);
+                }
+#pragma unroll
+                for (int w = 8; w > 0; w >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, w));
+                const float m_new = fmaxf(m[i], mx), corr = expf(m[i] - m_new);      // exp(-inf) = 0 on the first tile
+                m[i] = m_new;
+                l[i] *= corr;
+#pragma unroll
+                for (int e = 0; e < Cols<D>::N; ++e) o[i][e] *= corr;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float p = expf(s[i][j] - m_new);
+                    l[i] += p;
+                    sm.p.v[r0 + i][tx + 16 * j] = p;
+                }
+            }
+            __syncwarp();                     // a row of P is written and read by the same 16 lanes
+            product_nn(sm.p, sm.v, r0, tx, (n + 3) & ~3, o);
+        }
+        t += n;
+    }
+    if (!live) return;
+    float inv[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+#pragma unroll
+        for (int w = 8; w > 0; w >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], w);
+        inv[i] = 1.f / l[i];
+        if (lse != nullptr && tx == 0 && r0 + i < tile.n) lse[(size_t)bh * n_q + tile.row0 + r0 + i] = m[i] + logf(l[i]);
+    }
+    store_rows<T, D>(out + ((size_t)bh * n_q + tile.row0) * D, o, inv, r0, tx, tile.n);
+}
+
+// ---------------------------------------------------------------------------------------------
+// delta_i = sum_d dO_id * O_id, two threads per row
+template <typename T, int D>
+__global__ void __launch_bounds__(THREADS)
 simt_delta_kernel(const T* __restrict__ out, const T* __restrict__ dout, float* __restrict__ delta,
                   size_t n_rows) {
     constexpr int DH = D / 2;          // dimensions per thread
-    const size_t row = (size_t)blockIdx.x * ROWS + (threadIdx.x >> 1);
+    const size_t row = (size_t)blockIdx.x * (THREADS / 2) + (threadIdx.x >> 1);
     const int half = threadIdx.x & 1;
     float acc = 0.f;
     if (row < n_rows) {
         const T* a = out + row * D + half * DH;
         const T* b = dout + row * D + half * DH;
 #pragma unroll
-        for (int d = 0; d < DH; ++d) acc = fmaf(to_f(a[d]), to_f(b[d]), acc);
+        for (int d = 0; d < DH; d += 4) {
+            const float4 x = load4(a + d), y = load4(b + d);
+            acc = fmaf(x.w, y.w, fmaf(x.z, y.z, fmaf(x.y, y.y, fmaf(x.x, y.x, acc))));
+        }
     }
     acc += __shfl_xor_sync(0xffffffffu, acc, 1);
     if (row < n_rows && half == 0) delta[row] = acc;
 }
 
 // ---------------------------------------------------------------------------------------------
-// dQ: one thread pair per query row, loop over the row's keys.
+// Backward: the first half of the grid owns key tiles (dK, dV over the queries that see them), the second half query
+// tiles (dQ over their keys); one launch, so that both halves fill the chip together.  Each result has one owner that
+// adds in a fixed order: the gradients are bit-reproducible.
+template <int D> struct BwdSmem { RowTile<D> a, b, x, y; SquareTile p; float lse[TR], delta[TR]; };
+
 template <typename T, int D>
-__global__ void __launch_bounds__(128)
-simt_dq_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
-               const T* __restrict__ dout, const float* __restrict__ lse,
-               const float* __restrict__ delta, T* __restrict__ dq,
-               ScaleTable st, int L, float scale) {
-    constexpr int DH = D / 2;          // dimensions per thread
-    __shared__ float sK[KT][D];
-    __shared__ float sV[KT][D];
-    const int bh = blockIdx.y;
-    const int row0 = blockIdx.x * ROWS;
-    const int half = threadIdx.x & 1;
-    const int row_raw = row0 + (threadIdx.x >> 1);
-    const bool row_ok = row_raw < L;
-    const int row = row_ok ? row_raw : L - 1;
-    const int last_row = min(row0 + ROWS, L) - 1;
-    const int s_row = scale_of_row(st, row);
-    const int lo = st.start[first_key_scale(st.window, s_row)], hi = st.start[last_key_scale(st.window, s_row) + 1];
-    const int sf = scale_of_row(st, row0), sl = scale_of_row(st, last_row);
-    const int blk_lo = st.start[first_key_scale(st.window, sf)], blk_hi = st.start[last_key_scale(st.window, sl) + 1];
-    const size_t head = (size_t)bh * L;
+__global__ void __launch_bounds__(THREADS)
+simt_bwd_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
+                const T* __restrict__ dout, const float* __restrict__ lse, const float* __restrict__ delta,
+                T* __restrict__ dq, T* __restrict__ dk, T* __restrict__ dv,
+                const __grid_constant__ ScaleTable st, int L, int n_tiles, float scale) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    BwdSmem<D>& sm = *reinterpret_cast<BwdSmem<D>*>(smem_raw);
+    const size_t head = (size_t)blockIdx.y * L;
+    const bool keys = (int)blockIdx.x < n_tiles;            // the block owns a key tile
+    const TileRows tile = tile_rows(st, keys ? blockIdx.x : blockIdx.x - n_tiles);
+    const int tx = threadIdx.x & 15, r0 = (threadIdx.x >> 4) * 8;
+    const bool live = (threadIdx.x >> 5) * 16 < tile.n;     // the warp has rows of the tile
+    // Own rows a, b against partner rows x, y: keys own K, V and walk Q, dO; queries own Q, dO and walk K, V.
+    const T* own_a = keys ? k : q;
+    const T* own_b = keys ? v : dout;
+    const T* far_x = keys ? q : k;
+    const T* far_y = keys ? dout : v;
+    // (under HMAR_WINDOW_PREV the keys of the last scale have no queries: lo = hi, and zeros are stored)
+    const int lo = st.start[keys ? first_query_scale(st.window, tile.s) : first_key_scale(st.window, tile.s)];
+    const int hi = st.start[(keys ? last_query_scale(st.window, tile.s, st.n_scales) : last_key_scale(st.window, tile.s)) + 1];
 
-    float qr[DH], gr[DH], acc[DH];
+    stage(sm.a, own_a + (head + tile.row0) * D, tile.n);
+    stage(sm.b, own_b + (head + tile.row0) * D, tile.n);
+    float row_lse[8], row_delta[8];
 #pragma unroll
-    for (int d = 0; d < DH; ++d) {
-        qr[d] = to_f(q[(head + row) * D + half * DH + d]);
-        gr[d] = to_f(dout[(head + row) * D + half * DH + d]);
-        acc[d] = 0.f;
+    for (int i = 0; i < 8; ++i) {
+        const bool in = !keys && r0 + i < tile.n;
+        row_lse[i] = in ? lse[head + tile.row0 + r0 + i] : 0.f;
+        row_delta[i] = in ? delta[head + tile.row0 + r0 + i] : 0.f;
     }
-    const float lse_i = lse[head + row], delta_i = delta[head + row];
+    constexpr int N = Cols<D>::N;
+    float acc1[8][N], acc2[8][N];                           // dK and dV, or dQ and nothing
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int e = 0; e < N; ++e) acc1[i][e] = acc2[i][e] = 0.f;
 
-    for (int t = blk_lo; t < blk_hi; t += KT) {
-        const int cnt = min(KT, blk_hi - t);
+    for (int t = lo; t < hi; t += TR) {
+        const int n = min(TR, hi - t);
         __syncthreads();
-        stage_rows(sK, k + head * D, t, cnt);
-        stage_rows(sV, v + head * D, t, cnt);
-        __syncthreads();
-        for (int r = 0; r < cnt; ++r) {
-            float s = 0.f, dp = 0.f;
-#pragma unroll
-            for (int d = 0; d < DH; ++d) {
-                s = fmaf(qr[d], sK[r][half * DH + d], s);
-                dp = fmaf(gr[d], sV[r][half * DH + d], dp);
-            }
-            s += __shfl_xor_sync(0xffffffffu, s, 1);
-            dp += __shfl_xor_sync(0xffffffffu, dp, 1);
-            const int j = t + r;
-            if (j >= lo && j < hi) {
-                float p = expf(s * scale - lse_i);
-                float ds = p * (dp - delta_i);
-#pragma unroll
-                for (int d = 0; d < DH; ++d) acc[d] = fmaf(ds, sK[r][half * DH + d], acc[d]);
-            }
-        }
-    }
-    if (row_ok) {
-        T* op = dq + (head + row) * D + half * DH;
-#pragma unroll
-        for (int d = 0; d < DH; ++d) from_f(op + d, acc[d] * scale);
-    }
-}
-
-// ---------------------------------------------------------------------------------------------
-// dK, dV: one thread pair per key row, loop over the queries that see it.
-template <typename T, int D>
-__global__ void __launch_bounds__(128)
-simt_dkdv_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
-                 const T* __restrict__ dout, const float* __restrict__ lse,
-                 const float* __restrict__ delta, T* __restrict__ dk, T* __restrict__ dv,
-                 ScaleTable st, int L, float scale) {
-    constexpr int DH = D / 2;          // dimensions per thread
-    __shared__ float sQ[KT][D];
-    __shared__ float sG[KT][D];
-    __shared__ float sLse[KT];
-    __shared__ float sDelta[KT];
-    const int bh = blockIdx.y;
-    const int row0 = blockIdx.x * ROWS;
-    const int half = threadIdx.x & 1;
-    const int row_raw = row0 + (threadIdx.x >> 1);
-    const bool row_ok = row_raw < L;
-    const int row = row_ok ? row_raw : L - 1;
-    const int last_row = min(row0 + ROWS, L) - 1;
-    const int K = st.n_scales;
-    const int s_row = scale_of_row(st, row);
-    // (under HMAR_WINDOW_PREV the keys of the last scale have no queries: lo = hi = L, and dK = dV = 0 is stored)
-    const int lo = st.start[first_query_scale(st.window, s_row)], hi = max(lo, st.start[last_query_scale(st.window, s_row, K) + 1]);
-    const int blk_lo = st.start[first_query_scale(st.window, scale_of_row(st, row0))];
-    const int blk_hi = max(blk_lo, st.start[last_query_scale(st.window, scale_of_row(st, last_row), K) + 1]);
-    const size_t head = (size_t)bh * L;
-
-    float kr[DH], vr[DH], ak[DH], av[DH];
-#pragma unroll
-    for (int d = 0; d < DH; ++d) {
-        kr[d] = to_f(k[(head + row) * D + half * DH + d]);
-        vr[d] = to_f(v[(head + row) * D + half * DH + d]);
-        ak[d] = 0.f;
-        av[d] = 0.f;
-    }
-
-    for (int t = blk_lo; t < blk_hi; t += KT) {
-        const int cnt = min(KT, blk_hi - t);
-        __syncthreads();
-        stage_rows(sQ, q + head * D, t, cnt);
-        stage_rows(sG, dout + head * D, t, cnt);
-        if (threadIdx.x < cnt) {
-            sLse[threadIdx.x] = lse[head + t + threadIdx.x];
-            sDelta[threadIdx.x] = delta[head + t + threadIdx.x];
+        stage(sm.x, far_x + (head + t) * D, n);
+        stage(sm.y, far_y + (head + t) * D, n);
+        if (keys && threadIdx.x < TR) {
+            sm.lse[threadIdx.x] = threadIdx.x < n ? lse[head + t + threadIdx.x] : 0.f;
+            sm.delta[threadIdx.x] = threadIdx.x < n ? delta[head + t + threadIdx.x] : 0.f;
         }
         __syncthreads();
-        for (int r = 0; r < cnt; ++r) {
-            float s = 0.f, dp = 0.f;
+        if (!live) continue;
+        float s[8][4], dp[8][4];
+        product_nt(sm.a, sm.x, r0, tx, s);
 #pragma unroll
-            for (int d = 0; d < DH; ++d) {
-                s = fmaf(kr[d], sQ[r][half * DH + d], s);
-                dp = fmaf(vr[d], sG[r][half * DH + d], dp);
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int c = tx + 16 * j;
+                s[i][j] = c < n ? expf(s[i][j] * scale - (keys ? sm.lse[c] : row_lse[i])) : 0.f;
             }
-            s += __shfl_xor_sync(0xffffffffu, s, 1);
-            dp += __shfl_xor_sync(0xffffffffu, dp, 1);
-            const int i = t + r;
-            if (i >= lo && i < hi) {
-                float p = expf(s * scale - sLse[r]);
-                float ds = p * (dp - sDelta[r]);
+        if (keys) {
 #pragma unroll
-                for (int d = 0; d < DH; ++d) {
-                    av[d] = fmaf(p, sG[r][half * DH + d], av[d]);
-                    ak[d] = fmaf(ds, sQ[r][half * DH + d], ak[d]);
-                }
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) sm.p.v[r0 + i][tx + 16 * j] = s[i][j];
+            __syncwarp();                     // a row of P is written and read by the same 16 lanes
+            product_nn(sm.p, sm.y, r0, tx, (n + 3) & ~3, acc2);
+            __syncwarp();
+        }
+        product_nt(sm.b, sm.y, r0, tx, dp);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int c = tx + 16 * j;
+                sm.p.v[r0 + i][c] = s[i][j] * (dp[i][j] - (keys ? sm.delta[c] : row_delta[i]));
             }
-        }
+        __syncwarp();
+        product_nn(sm.p, sm.x, r0, tx, (n + 3) & ~3, acc1);
     }
-    if (row_ok) {
-        T* pk = dk + (head + row) * D + half * DH;
-        T* pv = dv + (head + row) * D + half * DH;
+    if (!live) return;
+    float mul[8], one[8];
 #pragma unroll
-        for (int d = 0; d < DH; ++d) {
-            from_f(pk + d, ak[d] * scale);
-            from_f(pv + d, av[d]);
-        }
-    }
+    for (int i = 0; i < 8; ++i) { mul[i] = scale; one[i] = 1.f; }
+    store_rows<T, D>((keys ? dk : dq) + (head + tile.row0) * D, acc1, mul, r0, tx, tile.n);
+    if (keys) store_rows<T, D>(dv + (head + tile.row0) * D, acc2, one, r0, tx, tile.n);
 }
 
 }  // namespace
@@ -288,14 +336,28 @@ simt_dkdv_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
 // ---------------------------------------------------------------------------------------------
 // Launchers
 
+static int count_tiles(const ScaleTable& st) {
+    int n = 0;
+    for (int s = 0; s < st.n_scales; ++s) n += (st.start[s + 1] - st.start[s] + TR - 1) / TR;
+    return n;
+}
+
+template <typename T, int D>
+static cudaError_t simt_fwd_any(const T* q, const T* k0, const T* v0, const T* k1, const T* v1, T* out, float* lse, int BH,
+                                const ScaleTable& st, int n_q, int n0, int n1, int dense, float scale, cudaStream_t stream) {
+    const cudaError_t e = cudaFuncSetAttribute(simt_fwd_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FwdSmem<D>));
+    if (e != cudaSuccess) return e;
+    simt_fwd_kernel<T, D><<<dim3(count_tiles(st), BH), THREADS, sizeof(FwdSmem<D>), stream>>>(q, k0, v0, k1, v1, out, lse, st, n_q, n0, n1,
+                                                                                             dense, scale);
+    count_launch(1);
+    return cudaGetLastError();
+}
+
 template <typename T, int D>
 static cudaError_t simt_fwd_d(const T* q, const T* k, const T* v, T* out, float* lse, int BH,
                               const ScaleTable& st, float scale, cudaStream_t stream) {
     const int L = st.start[st.n_scales];
-    dim3 grid((L + ROWS - 1) / ROWS, BH);
-    simt_fwd_kernel<T, D><<<grid, 128, 0, stream>>>(q, k, v, nullptr, nullptr, out, lse, st, L, L, 0, 0, scale);
-    count_launch(1);
-    return cudaGetLastError();
+    return simt_fwd_any<T, D>(q, k, v, nullptr, nullptr, out, lse, BH, st, L, L, 0, 0, scale, stream);
 }
 
 template <typename T, int D>
@@ -303,15 +365,11 @@ static cudaError_t simt_scale_step_d(const T* q, const T* k_prev, const T* v_pre
                                      T* out, float* lse, int BH, int n_prev, int n_cur, float scale,
                                      cudaStream_t stream) {
     ScaleTable st{};
-    dim3 grid((n_cur + ROWS - 1) / ROWS, BH);
+    st.n_scales = 1;
+    st.start[1] = n_cur;
     if (n_prev > 0)
-        simt_fwd_kernel<T, D><<<grid, 128, 0, stream>>>(q, k_prev, v_prev, k_cur, v_cur, out, lse, st,
-                                                     n_cur, n_prev, n_cur, 1, scale);
-    else
-        simt_fwd_kernel<T, D><<<grid, 128, 0, stream>>>(q, k_cur, v_cur, nullptr, nullptr, out, lse, st,
-                                                     n_cur, n_cur, 0, 1, scale);
-    count_launch(1);
-    return cudaGetLastError();
+        return simt_fwd_any<T, D>(q, k_prev, v_prev, k_cur, v_cur, out, lse, BH, st, n_cur, n_prev, n_cur, 1, scale, stream);
+    return simt_fwd_any<T, D>(q, k_cur, v_cur, nullptr, nullptr, out, lse, BH, st, n_cur, n_cur, 0, 1, scale, stream);
 }
 
 template <typename T, int D>
@@ -320,11 +378,13 @@ static cudaError_t simt_bwd_d(const T* q, const T* k, const T* v, const T* out, 
                               cudaStream_t stream) {
     const int L = st.start[st.n_scales];
     const size_t n_rows = (size_t)BH * L;
-    simt_delta_kernel<T, D><<<(unsigned)((n_rows + ROWS - 1) / ROWS), 128, 0, stream>>>(out, dout, delta, n_rows);
-    dim3 grid((L + ROWS - 1) / ROWS, BH);
-    simt_dq_kernel<T, D><<<grid, 128, 0, stream>>>(q, k, v, dout, lse, delta, dq, st, L, scale);
-    simt_dkdv_kernel<T, D><<<grid, 128, 0, stream>>>(q, k, v, dout, lse, delta, dk, dv, st, L, scale);
-    count_launch(3);
+    const cudaError_t e = cudaFuncSetAttribute(simt_bwd_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BwdSmem<D>));
+    if (e != cudaSuccess) return e;
+    simt_delta_kernel<T, D><<<(unsigned)((n_rows + THREADS / 2 - 1) / (THREADS / 2)), THREADS, 0, stream>>>(out, dout, delta, n_rows);
+    const int n_tiles = count_tiles(st);
+    simt_bwd_kernel<T, D><<<dim3(2 * n_tiles, BH), THREADS, sizeof(BwdSmem<D>), stream>>>(q, k, v, dout, lse, delta, dq, dk, dv, st, L,
+                                                                                         n_tiles, scale);
+    count_launch(2);
     return cudaGetLastError();
 }
 
