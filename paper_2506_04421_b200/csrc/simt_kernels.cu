@@ -47,24 +47,33 @@ __device__ __forceinline__ void stage(RowTile<D>& dst, const T* src, int n) {
     }
 }
 
-// acc[i][j] = sum_d a[r0 + i][d] b[tx + 16 j][d]
+// acc[i][j] = sum_d a[r0 + i][d] b[tx + 16 j][d].  Sums of eight products are added up: one chain over all of d doubles
+// the rounding error of large logits (LSE at |logits| = 30, D = 64: 1.1e-5 against 0.6e-5), and an addition per eight
+// FMAs costs less than that.
 template <int D>
 __device__ __forceinline__ void product_nt(const RowTile<D>& a, const RowTile<D>& b, int r0, int tx, float (&acc)[8][4]) {
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-#pragma unroll 2
-    for (int d = 0; d < D; d += 4) {
-        float4 bv[4];
+#pragma unroll 1
+    for (int d = 0; d < D; d += 8) {
+        float4 b0[4], b1[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) bv[j] = *reinterpret_cast<const float4*>(&b.v[tx + 16 * j][d]);
+        for (int j = 0; j < 4; ++j) {
+            b0[j] = *reinterpret_cast<const float4*>(&b.v[tx + 16 * j][d]);
+            b1[j] = *reinterpret_cast<const float4*>(&b.v[tx + 16 * j][d + 4]);
+        }
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            const float4 av = *reinterpret_cast<const float4*>(&a.v[r0 + i][d]);
+            const float4 a0 = *reinterpret_cast<const float4*>(&a.v[r0 + i][d]);
+            const float4 a1 = *reinterpret_cast<const float4*>(&a.v[r0 + i][d + 4]);
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-                acc[i][j] = fmaf(av.w, bv[j].w, fmaf(av.z, bv[j].z, fmaf(av.y, bv[j].y, fmaf(av.x, bv[j].x, acc[i][j]))));
+            for (int j = 0; j < 4; ++j) {
+                float t = fmaf(a0.w, b0[j].w, fmaf(a0.z, b0[j].z, fmaf(a0.y, b0[j].y, a0.x * b0[j].x)));
+                t = fmaf(a1.w, b1[j].w, fmaf(a1.z, b1[j].z, fmaf(a1.y, b1[j].y, fmaf(a1.x, b1[j].x, t))));
+                acc[i][j] += t;
+            }
         }
     }
 }
