@@ -880,12 +880,6 @@ static cudaError_t launch_bwd_tc_layout(const CUtensorMap& q, const CUtensorMap&
                                         const CUtensorMap& dq_acc_map, const BwdArgs& args, const __nv_bfloat16* out,
                                         const __nv_bfloat16* dout, __nv_bfloat16* dq, int BH, cudaStream_t stream) {
     const size_t smem = sizeof(SharedStorage);
-    cudaError_t e = cudaFuncSetAttribute(hmar_bwd_tc_kernel<false, STRIDED, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(hmar_bwd_tc_kernel<true, STRIDED, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(hmar_bwd_tc_kernel<false, STRIDED, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     const size_t n_rows = (size_t)BH * args.L;
     {
         KernelTimer timer("hmar_bwd_delta_kernel", stream);
@@ -905,12 +899,14 @@ static cudaError_t launch_bwd_tc_layout(const CUtensorMap& q, const CUtensorMap&
             a.split = 8;
             while (a.split > 0 && ((long long)BH * a.split + grid - 1) / grid > MAX_CHUNKS) a.split >>= 1;
         }
-        if (a.split > 0)
-            hmar_bwd_tc_kernel<true, STRIDED, false><<<grid, NUM_THREADS, smem, stream>>>(q, k, v, dout_map, dq_acc_map, a);
-        else if (args.plain_permille < kOneMaskBelowPermille)
-            hmar_bwd_tc_kernel<false, STRIDED, true><<<grid, NUM_THREADS, smem, stream>>>(q, k, v, dout_map, dq_acc_map, a);
-        else
-            hmar_bwd_tc_kernel<false, STRIDED, false><<<grid, NUM_THREADS, smem, stream>>>(q, k, v, dout_map, dq_acc_map, a);
+        static SmemOptIn opt_in[3];
+        auto kernel = hmar_bwd_tc_kernel<false, STRIDED, false>;
+        int which = 0;
+        if (a.split > 0) { kernel = hmar_bwd_tc_kernel<true, STRIDED, false>; which = 1; }
+        else if (args.plain_permille < kOneMaskBelowPermille) { kernel = hmar_bwd_tc_kernel<false, STRIDED, true>; which = 2; }
+        const cudaError_t e = opt_in[which]((const void*)kernel, smem);
+        if (e != cudaSuccess) return e;
+        kernel<<<grid, NUM_THREADS, smem, stream>>>(q, k, v, dout_map, dq_acc_map, a);
     }
     const size_t n8 = n_rows * D / 8;
     {

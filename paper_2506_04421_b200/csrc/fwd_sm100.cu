@@ -485,7 +485,8 @@ size_t fwd_tc_smem_bytes() { return sizeof(SharedStorage) + 1024; }
 cudaError_t launch_fwd_tc(const CUtensorMap& q, const CUtensorMap& k0, const CUtensorMap& v0, const CUtensorMap& k1,
                           const CUtensorMap& v1, const FwdArgs& args, int BH, cudaStream_t stream) {
     const size_t smem = fwd_tc_smem_bytes();
-    cudaError_t e = cudaFuncSetAttribute(hmar_fwd_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SmemOptIn opt_in;
+    const cudaError_t e = opt_in((const void*)hmar_fwd_tc_kernel, smem);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)BH * (unsigned)args.n_work;
     {

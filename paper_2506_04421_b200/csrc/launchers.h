@@ -1,6 +1,7 @@
 // Internal launcher prototypes shared between the C-ABI layer and the kernel files.
 #pragma once
 #include <cuda_runtime.h>
+#include <atomic>
 #include "hmar_common.h"
 
 namespace hmar {
@@ -17,6 +18,22 @@ struct KernelTimer {
     cudaStream_t stream_;
     cudaEvent_t begin_;
     bool on_;
+};
+
+// Opts a kernel in to `bytes` of dynamic shared memory on the current device: once per kernel and device, not on every
+// call (0.4 us of host time each, three of them in a backward call).
+struct SmemOptIn {
+    std::atomic<unsigned long long> done{0};                // a bit per device
+    cudaError_t operator()(const void* kernel, size_t bytes) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        const unsigned long long bit = dev < 64 ? 1ull << dev : 0;
+        if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+        return e;
+    }
 };
 
 template <typename T>

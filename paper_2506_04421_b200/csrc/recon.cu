@@ -367,14 +367,15 @@ cudaError_t launch_recon_downsample(const float* xhat, float* out, int B, int C,
         const unsigned grid = (unsigned)((n_planes + warps - 1) / warps);
         cudaError_t e = cudaSuccess;
         KernelTimer timer("hmar_recon_downsample_kernel", stream);
-        auto go = [&](auto kernel) {
-            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDownStageSmem);
+        static SmemOptIn opt_in[4];
+        auto go = [&](auto kernel, int which) {
+            e = opt_in[which]((const void*)kernel, kDownStageSmem);
             if (e == cudaSuccess) kernel<<<grid, warps * 32, smem, stream>>>(xhat, out, n_planes, in_side, out_side, warps);
         };
-        if (in_side == 16) go(hmar_recon_downsample_staged_kernel<16>);
-        else if (in_side == 32) go(hmar_recon_downsample_staged_kernel<32>);
-        else if (in_side == 64) go(hmar_recon_downsample_staged_kernel<64>);
-        else go(hmar_recon_downsample_staged_kernel<0>);
+        if (in_side == 16) go(hmar_recon_downsample_staged_kernel<16>, 0);
+        else if (in_side == 32) go(hmar_recon_downsample_staged_kernel<32>, 1);
+        else if (in_side == 64) go(hmar_recon_downsample_staged_kernel<64>, 2);
+        else go(hmar_recon_downsample_staged_kernel<0>, 3);
         if (e != cudaSuccess) return e;
         count_launch(1);
         return cudaGetLastError();

@@ -354,7 +354,8 @@ static int count_tiles(const ScaleTable& st) {
 template <typename T, int D>
 static cudaError_t simt_fwd_any(const T* q, const T* k0, const T* v0, const T* k1, const T* v1, T* out, float* lse, int BH,
                                 const ScaleTable& st, int n_q, int n0, int n1, int dense, float scale, cudaStream_t stream) {
-    const cudaError_t e = cudaFuncSetAttribute(simt_fwd_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FwdSmem<D>));
+    static SmemOptIn opt_in;
+    const cudaError_t e = opt_in((const void*)simt_fwd_kernel<T, D>, sizeof(FwdSmem<D>));
     if (e != cudaSuccess) return e;
     simt_fwd_kernel<T, D><<<dim3(count_tiles(st), BH), THREADS, sizeof(FwdSmem<D>), stream>>>(q, k0, v0, k1, v1, out, lse, st, n_q, n0, n1,
                                                                                              dense, scale);
@@ -387,7 +388,8 @@ static cudaError_t simt_bwd_d(const T* q, const T* k, const T* v, const T* out, 
                               cudaStream_t stream) {
     const int L = st.start[st.n_scales];
     const size_t n_rows = (size_t)BH * L;
-    const cudaError_t e = cudaFuncSetAttribute(simt_bwd_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BwdSmem<D>));
+    static SmemOptIn opt_in;
+    const cudaError_t e = opt_in((const void*)simt_bwd_kernel<T, D>, sizeof(BwdSmem<D>));
     if (e != cudaSuccess) return e;
     simt_delta_kernel<T, D><<<(unsigned)((n_rows + THREADS / 2 - 1) / (THREADS / 2)), THREADS, 0, stream>>>(out, dout, delta, n_rows);
     const int n_tiles = count_tiles(st);

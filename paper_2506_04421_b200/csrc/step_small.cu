@@ -254,10 +254,9 @@ int step_small(const __nv_bfloat16* q, const __nv_bfloat16* k_prev, const __nv_b
     const int warps = (n_cur + 31) / 32;
     const int keys_pad = (n_prev + n_cur + 15) & ~15;
     const size_t smem = (size_t)2 * keys_pad * ROW_BYTES;
-    // the largest window needs more than the default 48 KB of dynamic shared memory (per function and device; cheap to repeat)
-    if (cudaFuncSetAttribute(hmar_step_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             2 * kSmallMaxKeys * ROW_BYTES) != cudaSuccess)
-        return HMAR_ERR_CUDA;
+    // the largest window needs more than the default 48 KB of dynamic shared memory
+    static SmemOptIn opt_in;
+    if (opt_in((const void*)hmar_step_small_kernel, 2 * kSmallMaxKeys * ROW_BYTES) != cudaSuccess) return HMAR_ERR_CUDA;
     {
         KernelTimer timer("hmar_step_small_kernel", stream);
         hmar_step_small_kernel<<<BH, warps * 32, smem, stream>>>(a);
