@@ -57,15 +57,31 @@ constexpr int D = kHeadDim;
 constexpr int NSTAGE = 3;
 constexpr int AUX_STAGES = 8;        // ring of lse / delta rows, loaded this many steps ahead
 constexpr int TILE_BYTES = 128 * D * 2;          // 16 KB
-constexpr int WORK_CACHE = 64;       // work tiles of a head kept in shared memory
-constexpr int MAX_CHUNKS = 64;       // runs of consecutive items a block can be given
+constexpr int ITEM_STAGES = 8;       // ring of items handed out by the scheduler warp
+constexpr int ITEM_READERS = 15;     // warps that read every item: all but the scheduler
 constexpr int NUM_COMPUTE_THREADS = 256;
-constexpr int DRAIN_WARP0 = 8, PRODUCER_WARP = 12, MMA_WARP = 13, AUX_WARP = 14;
+constexpr int DRAIN_WARP0 = 8, PRODUCER_WARP = 12, MMA_WARP = 13, AUX_WARP = 14, SCHED_WARP = 15;
 constexpr int NUM_THREADS = 512;
 constexpr int REGS_COMPUTE = 160, REGS_DRAIN = 88, REGS_MISC = 104;
 static_assert(2 * REGS_COMPUTE + REGS_DRAIN + REGS_MISC == 4 * 128, "register budget of the block");
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t COL_ST = 0, COL_DPT = 128, COL_DK = 256, COL_DV = 320, COL_DQ = 384, COL_K = 448, COL_V = 480;
+
+// A work item as the roles see it: key rows [row_begin, row_begin + row_count) of head bh (head `head` of batch `batch`)
+// and `steps` steps over the query rows [q_begin, q_end).  steps == 0: there are no more items.
+struct Item {
+    int bh, head, batch;
+    int row_begin, row_count;
+    int q_begin, q_end;
+    int steps_uniform;                      // steps * 2 + uniform
+    __device__ __forceinline__ int steps() const { return steps_uniform >> 1; }
+    __device__ __forceinline__ bool uniform() const { return steps_uniform & 1; }
+    // number of query columns of half h of step i handed to the tensor core (a multiple of 16)
+    __device__ __forceinline__ int half_cols(int i, int h) const {
+        const int n_eff = (min(BQ, q_end - (q_begin + i * BQ)) + 15) & ~15;
+        return h == 0 ? min(n_eff, HQ) : max(n_eff - HQ, 0);
+    }
+};
 
 struct __align__(1024) SharedStorage {
     uint8_t k[2][TILE_BYTES];               // K of the current item and of the next one (B operand of dQ)
@@ -80,13 +96,10 @@ struct __align__(1024) SharedStorage {
     uint64_t qdo_full[NSTAGE], q_empty[NSTAGE], aux_full[AUX_STAGES], aux_empty[AUX_STAGES];
     uint64_t s_full[2], p_full[2];            // [half of the step]
     uint64_t dq_full, dq_empty, acc_full, acc_empty;
-    BwdWork work[WORK_CACHE];               // the head's work list (its first WORK_CACHE tiles)
+    Item item[ITEM_STAGES];
+    uint64_t item_full[ITEM_STAGES], item_empty[ITEM_STAGES];
     uint32_t tmem_base;
     uint32_t gave_up;                       // offset of the barrier whose wait ran out (0: none did)
-    // The block's items: n_chunks runs of consecutive items; run c starts at item chunk_item[c] and holds the
-    // block's items number chunk_first[c] .. chunk_first[c + 1] - 1.
-    int chunk_item[MAX_CHUNKS], chunk_first[MAX_CHUNKS + 1];
-    int n_chunks;
 };
 #define AT(field) (base + (uint32_t)offsetof(SharedStorage, field))     // shared-memory address
 
@@ -200,22 +213,6 @@ __device__ __forceinline__ void softmax_grad_half(uint32_t lane_base, int cbase,
     }
 }
 
-// Work items of one block.  Item g is tile g % n_work of head g / n_work; items are ordered head by
-// head (a head's Q and dO tiles stay in L2 while its key tiles are processed) and every block takes a
-// contiguous run of items of about the same total cost (steps plus a constant per item).
-__device__ __forceinline__ int first_item_at_cost(const BwdArgs& args, long long cost) {
-    const long long head = cost / args.head_cost;
-    const int rem = (int)(cost - head * args.head_cost);
-    int lo = 0, hi = args.n_work;                       // first tile whose starting cost is >= rem
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (__ldg(&args.work[mid].cost_begin) >= rem) hi = mid; else lo = mid + 1;
-    }
-    return (int)head * args.n_work + lo;
-}
-
-// CHUNKED: the block's items are several runs (long sequences, see the launcher); otherwise one contiguous run,
-// and the item loops compile to plain counting.
 // STRIDED: the bf16 tensors have the strides given in the arguments (packed projection layouts); otherwise they are
 // dense [BH, L, 64] and every address is formed with compile-time strides (the dense instantiation is the one the
 // benchmarks run: the extra address arithmetic and code of the strided one cost it a tenth of its speed).
@@ -224,7 +221,7 @@ __device__ __forceinline__ int first_item_at_cost(const BwdArgs& args, long long
 // partial or packed (L = 680: 11 % faster, a third of the instruction-cache requests of the three-variant code
 // miss there); where most steps belong to full tiles the plain variant's shorter arithmetic wins (L = 2240: the
 // one-variant code is 4 % slower).
-template <bool CHUNKED, bool STRIDED, bool ONE_MASK>
+template <bool STRIDED, bool ONE_MASK>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                    const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do,
@@ -244,7 +241,6 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     }
 
     const int L = args.L;
-    const int n_work = args.n_work;
 
     if (threadIdx.x == 0) {
         sm.gave_up = 0;
@@ -270,33 +266,12 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         mbar_init(&sm.dq_empty, 128);
         mbar_init(&sm.acc_full, 1);
         mbar_init(&sm.acc_empty, 128);
-        fence_mbar_init();
-        int nch = 0, cnt = 0;
-        if (!CHUNKED) {
-            // one run: a contiguous stretch of the item list of about 1 / gridDim.x of the total cost
-            const long long total = (long long)args.n_heads * args.head_cost;
-            const int ib = first_item_at_cost(args, total * blockIdx.x / gridDim.x);
-            const int ie = blockIdx.x + 1 == gridDim.x ? args.n_heads * n_work
-                                                       : first_item_at_cost(args, total * (blockIdx.x + 1) / gridDim.x);
-            if (ie > ib) { sm.chunk_item[0] = ib; sm.chunk_first[0] = 0; cnt = ie - ib; nch = 1; }
-        } else {
-            // Long sequences: every head is cut into `split` runs of equal cost, and the runs are dealt to the blocks
-            // in turn.  The blocks then work on gridDim.x / split heads at a time instead of one head each, so that
-            // the fp32 dQ accumulator lines of the heads in flight (and their Q, dO tiles) stay in L2.
-            const int n_runs = args.n_heads * args.split;
-            for (int k = blockIdx.x; k < n_runs && nch < MAX_CHUNKS; k += gridDim.x) {
-                const int head = k / args.split, c = k - head * args.split;
-                const int lo_cost = (int)((long long)args.head_cost * c / args.split);
-                const int hi_cost = (int)((long long)args.head_cost * (c + 1) / args.split);
-                const int tb = first_item_at_cost(args, lo_cost);                       // tile index: the head is 0 here
-                const int te = c + 1 == args.split ? n_work : first_item_at_cost(args, hi_cost);
-                if (te > tb) { sm.chunk_item[nch] = head * n_work + tb; sm.chunk_first[nch] = cnt; cnt += te - tb; ++nch; }
-            }
+        for (int s = 0; s < ITEM_STAGES; ++s) {
+            mbar_init(&sm.item_full[s], 1);
+            mbar_init(&sm.item_empty[s], ITEM_READERS);
         }
-        sm.chunk_first[nch] = cnt;
-        sm.n_chunks = nch;
+        fence_mbar_init();
     }
-    for (int t = threadIdx.x; t < min(n_work, WORK_CACHE); t += NUM_THREADS) sm.work[t] = args.work[t];
     if (warp == MMA_WARP) {
         tmem_alloc(&sm.tmem_base, TMEM_COLS);
         tmem_relinquish();
@@ -305,36 +280,64 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sm.tmem_base;
-    const int n_chunks = sm.n_chunks, n_items = sm.chunk_first[n_chunks];
-    // item number n of this block (n rises, or steps back by one or two, from call to call: `run` follows it)
-    const int first_item = sm.chunk_item[0];
-    auto item_at = [&](int n, int& run) -> int {
-        if (!CHUNKED) return first_item + n;
-        while (n >= sm.chunk_first[run + 1] && run + 1 < n_chunks) ++run;
-        while (n < sm.chunk_first[run] && run > 0) --run;
-        return sm.chunk_item[run] + (n - sm.chunk_first[run]);
-    };
     auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
         if (warp_wait(bar, parity)) return true;
         if (lane == 0) sm.gave_up = bar - base;
         return false;
     };
 
-    auto get_work = [&](int g) -> BwdWork {
-        const int t = g % n_work;
-        return t < WORK_CACHE ? sm.work[t] : args.work[t];
+    // The block's items go through a ring.  `look(n)` waits until item n is there; its fields are then read in place, and
+    // `done(n)` gives the slot back (once per warp; items are looked at and done in order).
+    auto look = [&](int n) -> bool { return wait(AT(item_full) + (n % ITEM_STAGES) * 8, (n / ITEM_STAGES) & 1); };
+    auto done = [&](int n) {
+        __syncwarp();
+        if (lane == 0) bar_arrive(AT(item_empty) + (n % ITEM_STAGES) * 8);
     };
-    auto steps_of = [](const BwdWork& w) { return (w.q_end - w.q_begin + BQ - 1) / BQ; };
-    // number of query columns of half h of step i handed to the tensor core (a multiple of 16)
-    auto half_cols = [](const BwdWork& w, int i, int h) {
-        const int n_valid = min(BQ, w.q_end - (w.q_begin + i * BQ));
-        const int n_eff = (n_valid + 15) & ~15;
-        return h == 0 ? min(n_eff, HQ) : max(n_eff - HQ, 0);
-    };
+    auto item_at = [&](int n) -> const Item& { return sm.item[n % ITEM_STAGES]; };
 
     if (warp >= PRODUCER_WARP) {
         reg_dec<REGS_MISC>();
-        if (warp == PRODUCER_WARP) {
+        if (warp == SCHED_WARP) {
+            // ================================================================== item scheduler
+            // A head's tiles are ordered by cost; tiles of equal cost are one class.  The launch works class by class,
+            // head by head inside a class, and the items are dealt to the blocks round by round, back and forth.  The
+            // blocks' sums then differ by 0.6 % (L = 9451, 192 heads) where a stretch or several runs of heads per block
+            // differed by 12 %, and the blocks work on few heads at a time: at L = 2240 18, whose dQ accumulators stay
+            // in L2.  The last records say that there are no more (the readers look up to two items ahead).
+            const int total = args.n_heads * args.n_work;
+            int extra = 0;
+            for (int n = 0; extra < 3; ++n) {
+                const int slot = n % ITEM_STAGES;
+                if (n >= ITEM_STAGES && !wait(AT(item_empty) + slot * 8, ((n / ITEM_STAGES) & 1) ^ 1)) break;
+                int pos = n * (int)gridDim.x + ((n & 1) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x);
+                Item it;
+                it.steps_uniform = 0;
+                if (pos < total) {
+                    int t = 0, count = __ldg(&args.work[0].class_count);
+                    while (pos >= args.n_heads * count) {
+                        pos -= args.n_heads * count;
+                        t += count;
+                        count = __ldg(&args.work[t].class_count);
+                    }
+                    it.bh = pos / count;
+                    const BwdWork w = args.work[t + pos - it.bh * count];
+                    it.batch = STRIDED ? it.bh / args.heads_per_batch : 0;
+                    it.head = it.bh - it.batch * args.heads_per_batch * (STRIDED ? 1 : 0);
+                    it.row_begin = w.row_begin;
+                    it.row_count = w.row_count;
+                    it.q_begin = w.q_begin;
+                    it.q_end = w.q_end;
+                    it.steps_uniform = ((w.q_end - w.q_begin + BQ - 1) / BQ) * 2 + (w.uniform != 0);
+                } else {
+                    ++extra;
+                }
+                if (lane == 0) {
+                    sm.item[slot] = it;
+                    bar_arrive(AT(item_full) + slot * 8);
+                }
+                __syncwarp();
+            }
+        } else if (warp == PRODUCER_WARP) {
             // ================================================================== producer
             // The whole warp runs the control flow; one elected lane issues the copies.
             const bool leader = elect_one();
@@ -346,13 +349,13 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             }
             bool ok = true;
             int gs = 0;                                     // steps issued so far, over all items
-            int run = 0;
-            for (int item = 0; item < n_items && ok; ++item) {
-                const int g = item_at(item, run);
-                const int bh = g / n_work;
-                const int batch = STRIDED ? bh / args.heads_per_batch : 0, head = STRIDED ? bh - batch * args.heads_per_batch : bh;
-                const BwdWork w = get_work(g);
-                const int n_steps = steps_of(w);
+            for (int item = 0; ok; ++item) {
+                ok = look(item);
+                if (!ok) break;
+                const Item w = item_at(item);
+                done(item);
+                const int n_steps = w.steps(), head = w.head, batch = w.batch;
+                if (n_steps == 0) break;
                 if (item >= 2) {
                     // the buffer held K of the item before the previous one, read by its dQ products
                     ok = wait(AT(k_free) + (item & 1) * 8, ((item >> 1) & 1) ^ 1);
@@ -391,12 +394,13 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             // their use (plain loads: their row offsets are not 16-byte aligned, so TMA cannot fetch them).
             bool ok = true;
             int gs = 0;
-            int run = 0;
-            for (int item = 0; item < n_items && ok; ++item) {
-                const int g = item_at(item, run);
-                const int bh = g / n_work;
-                const BwdWork w = get_work(g);
-                const int n_steps = steps_of(w);
+            for (int item = 0; ok; ++item) {
+                ok = look(item);
+                if (!ok) break;
+                const Item w = item_at(item);
+                done(item);
+                const int n_steps = w.steps(), bh = w.bh;
+                if (n_steps == 0) break;
                 for (int i = 0; i < n_steps; ++i, ++gs) {
                     const int aslot = gs % AUX_STAGES;
                     if (gs >= AUX_STAGES) {
@@ -480,38 +484,40 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             // The steps of all items form one sequence: while the compute warpgroups work on a step, the
             // tensor core gets the next step's S^T, dP^T even when that step belongs to the next item (whose
             // K, V rows the drain warps have put into TMEM by then).
-            int run = 0;
-            if (n_items > 0) {
-                const BwdWork w0 = get_work(item_at(0, run));
-                ok = wait2(AT(kv_tmem), 0, AT(qdo_full) + (0) * 8, 0, true);
+            ok = look(0) && look(1);
+            bool live = ok && item_at(0).steps() > 0;
+            if (live) {
+                const Item& w0 = item_at(0);
+                ok = wait2(AT(kv_tmem), 0, AT(qdo_full), 0, true);
                 if (ok) {
                     tc_fence_after();
                     if (leader) {
-                        scores(0, half_cols(w0, 0, 0), 0);
-                        const int n1 = half_cols(w0, 0, 1);
+                        scores(0, w0.half_cols(0, 0), 0);
+                        const int n1 = w0.half_cols(0, 1);
                         if (n1 > 0) scores(1, n1, 0);
-                        if (steps_of(w0) == 1 && 1 < n_items) commit_at(AT(kv_free));
+                        if (w0.steps() == 1 && item_at(1).steps() > 0) commit_at(AT(kv_free));
                     }
                     __syncwarp();
                 }
             }
-            for (int item = 0; item < n_items && ok; ++item) {
-                const BwdWork w = get_work(item_at(item, run));
-                const int n_steps = steps_of(w);
-                const bool next_item = item + 1 < n_items;
-                const BwdWork wn = next_item ? get_work(item_at(item + 1, run)) : w;
-                const int n_steps_next = steps_of(wn);
+            for (int item = 0; live && ok; ++item) {
+                ok = look(item + 2);
+                if (!ok) break;
+                const Item w = item_at(item);
+                const Item wn = item_at(item + 1);
+                const int n_steps = w.steps(), n_steps_next = wn.steps();
+                const bool next_item = n_steps_next > 0, item_after = item_at(item + 2).steps() > 0;
                 const uint64_t k_mn = k_mn0 + (item & 1) * 1024;
                 for (int i = 0; i < n_steps && ok; ++i, ++gs) {
                     const int slot = gs % NSTAGE, slot_next = (gs + 1) % NSTAGE;
                     const bool more = i + 1 < n_steps;          // the item has another step
                     const bool cross = !more && next_item;      // the next step is the next item's first
                     const bool any_next = more || cross;
-                    const int n0 = half_cols(w, i, 0), n1 = half_cols(w, i, 1);
-                    const int m0 = more ? half_cols(w, i + 1, 0) : cross ? half_cols(wn, 0, 0) : 0;
-                    const int m1 = more ? half_cols(w, i + 1, 1) : cross ? half_cols(wn, 0, 1) : 0;
+                    const int n0 = w.half_cols(i, 0), n1 = w.half_cols(i, 1);
+                    const int m0 = more ? w.half_cols(i + 1, 0) : cross ? wn.half_cols(0, 0) : 0;
+                    const int m1 = more ? w.half_cols(i + 1, 1) : cross ? wn.half_cols(0, 1) : 0;
                     // the next step is the last one that reads its item's K, V rows in TMEM, and another item follows
-                    const bool frees_kv = more ? (i + 2 == n_steps && next_item) : (cross && n_steps_next == 1 && item + 2 < n_items);
+                    const bool frees_kv = more ? (i + 2 == n_steps && next_item) : (cross && n_steps_next == 1 && item_after);
                     // ---- burst X: needs P^T, dS^T of half 0 and the next step's Q / dO tile
                     ok = wait2(AT(p_full) + (0) * 8, ng[0] & 1, AT(qdo_full) + (slot_next) * 8, ((gs + 1) / NSTAGE) & 1, any_next);
                     if (!ok) break;
@@ -563,6 +569,8 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     }
                     __syncwarp();
                 }
+                done(item);
+                live = next_item;
             }
         }
     } else if (warp >= DRAIN_WARP0) {
@@ -587,15 +595,14 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         // in registers until the previous item's last scores have been computed; the K row is read from the
         // tile that the copy engine has put into shared memory for the dQ products.  Rows past the end of
         // the sequence are zeros.
-        auto copy_kv = [&](int gc, int item, bool wait_free) -> bool {
-            const BwdWork wc = get_work(gc);
+        auto copy_kv = [&](int item, bool wait_free) -> bool {
+            const Item& wc = item_at(item);
             const int row = wc.row_begin + r;
             const uint4* vsrc;
             if (STRIDED) {
-                const int cbh = gc / n_work, cb = cbh / args.heads_per_batch, ch = cbh - cb * args.heads_per_batch;
-                vsrc = reinterpret_cast<const uint4*>(args.v + cb * args.in_batch + ch * args.in_head + (long long)row * args.in_row);
+                vsrc = reinterpret_cast<const uint4*>(args.v + wc.batch * args.in_batch + wc.head * args.in_head + (long long)row * args.in_row);
             } else {
-                vsrc = reinterpret_cast<const uint4*>(args.v + ((size_t)(gc / n_work) * L + row) * D);
+                vsrc = reinterpret_cast<const uint4*>(args.v + ((size_t)wc.bh * L + row) * D);
             }
             const long long v_off = reinterpret_cast<const __nv_bfloat16*>(vsrc) - args.v;
             const bool v_in = row < L && HMAR_IN_BOUNDS(v_off >= 0 && v_off + D <= args.in_extent, args.status, 0xB202);
@@ -617,25 +624,27 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             bar_arrive(AT(kv_tmem));
             return true;
         };
-        int run = 0;
-        if (n_items > 0) {
-            ok = copy_kv(item_at(0, run), 0, false);
-            if (ok && steps_of(get_work(item_at(0, run))) == 1 && 1 < n_items) ok = copy_kv(item_at(1, run), 1, true);
+        ok = look(0) && look(1);
+        if (ok && item_at(0).steps() > 0) {
+            ok = copy_kv(0, false);
+            if (ok && item_at(0).steps() == 1 && item_at(1).steps() > 0) ok = copy_kv(1, true);
         }
-        for (int item = 0; item < n_items && ok; ++item) {
-            const int g = item_at(item, run);
-            const int bh = g / n_work;
-            const BwdWork w = get_work(g);
-            const int n_steps = steps_of(w);
-            const bool next_item = item + 1 < n_items;
-            const int n_steps_next = next_item ? steps_of(get_work(item_at(item + 1, run))) : 0;
+        for (int item = 0; ok; ++item) {
+            const Item w = item_at(item);
+            const int n_steps = w.steps();
+            if (n_steps == 0) break;
+            ok = look(item + 2);
+            if (!ok) break;
+            const int bh = w.bh;
+            const int n_steps_next = item_at(item + 1).steps();
+            const bool next_item = n_steps_next > 0, item_after = item_at(item + 2).steps() > 0;
             for (int i = 0; i < n_steps; ++i, ++gs) {
                 const bool more = i + 1 < n_steps;
                 // the next step is the last one of its item and another item follows: that item's K, V rows
                 // go to TMEM as soon as the next step's scores are complete
-                if (more ? (i + 2 == n_steps && next_item) : (next_item && n_steps_next == 1 && item + 2 < n_items)) {
+                if (more ? (i + 2 == n_steps && next_item) : (next_item && n_steps_next == 1 && item_after)) {
                     const int nc = more ? item + 1 : item + 2;
-                    ok = copy_kv(item_at(nc, run), nc, true);
+                    ok = copy_kv(nc, true);
                     if (!ok) break;
                 }
                 if (!more) {
@@ -656,8 +665,7 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                             __nv_bfloat16* base = part < 2 ? args.dk : args.dv;
                             uint4* dst;
                             if (STRIDED) {
-                                const int ob = bh / args.heads_per_batch, oh = bh - ob * args.heads_per_batch;
-                                dst = reinterpret_cast<uint4*>(base + ob * args.g_batch + oh * args.g_head +
+                                dst = reinterpret_cast<uint4*>(base + w.batch * args.g_batch + w.head * args.g_head +
                                                                (long long)(w.row_begin + r) * args.g_row + (part & 1) * 32);
                             } else {
                                 dst = reinterpret_cast<uint4*>(base + ((size_t)bh * L + w.row_begin + r) * D + (part & 1) * 32);
@@ -706,6 +714,7 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     }
                 }
             }
+            if (ok) done(item);
         }
         if (lane == 0) bulk_wait_all();         // the staging buffer must outlive the last reduction's read
     } else {
@@ -719,13 +728,16 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         int gs = 0;                                         // steps seen so far (aux ring, dS buffer parity)
         int nsh = 0;                                        // non-empty halves of this warpgroup seen so far
 
-        int run = 0;
-        for (int item = 0; item < n_items && ok; ++item) {
-            const BwdWork w = get_work(item_at(item, run));
-            const int n_steps = steps_of(w);
+        for (int item = 0; ok; ++item) {
+            ok = look(item);
+            if (!ok) break;
+            const Item w = item_at(item);
+            done(item);
+            const int n_steps = w.steps();
+            if (n_steps == 0) break;
             // the four key rows this thread works on in the softmax-gradient layout, and the queries that may see them
-            const bool tile_masked = ONE_MASK || (!w.uniform) || (w.row_count < BKV);
-            const bool rows_only = !ONE_MASK && w.uniform != 0;   // only rows past the end of the tile are hidden
+            const bool tile_masked = ONE_MASK || (!w.uniform()) || (w.row_count < BKV);
+            const bool rows_only = !ONE_MASK && w.uniform();        // only rows past the end of the tile are hidden
             int qlo[4], qhi[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -733,7 +745,7 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 qlo[i] = w.q_begin; qhi[i] = w.q_end;
                 if (tile_masked) {
                     if (rr >= w.row_count) { qlo[i] = 0; qhi[i] = 0; }
-                    else if (!w.uniform) {
+                    else if (!w.uniform()) {
                         const int sc = scale_of_row(args.st, w.row_begin + rr);
                         qlo[i] = args.st.start[first_query_scale(args.st.window, sc)];
                         qhi[i] = args.st.start[last_query_scale(args.st.window, sc, args.st.n_scales) + 1];
@@ -744,7 +756,7 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             for (int i = 0; i < n_steps && ok; ++i, ++gs) {
                 const int q0 = w.q_begin + i * BQ;
                 const int n_valid = min(BQ, w.q_end - q0);
-                const int n_cols = half_cols(w, i, h);
+                const int n_cols = w.half_cols(i, h);
                 const int cbase = h * HQ;                   // first query column of this half inside the step
 
                 const int aslot = gs % AUX_STAGES;
@@ -890,23 +902,12 @@ static cudaError_t launch_bwd_tc_layout(const CUtensorMap& q, const CUtensorMap&
         KernelTimer timer("hmar_bwd_tc_kernel", stream);
         const long long items = (long long)BH * args.n_work;
         const unsigned grid = (unsigned)(items < sm_count() ? items : sm_count());
-        BwdArgs a = args;
-        // Long sequences only (measured: at L = 2240 the kernel does not care how many heads are in flight, at
-        // L = 9451 it is a fifth slower with one head per block): 8 runs per head, fewer if a block would get
-        // more runs than its table holds.
-        a.split = 0;
-        if (args.L >= 4096 && (unsigned)BH >= grid) {       // (with fewer heads than blocks the runs would not balance)
-            a.split = 8;
-            while (a.split > 0 && ((long long)BH * a.split + grid - 1) / grid > MAX_CHUNKS) a.split >>= 1;
-        }
-        static SmemOptIn opt_in[3];
-        auto kernel = hmar_bwd_tc_kernel<false, STRIDED, false>;
-        int which = 0;
-        if (a.split > 0) { kernel = hmar_bwd_tc_kernel<true, STRIDED, false>; which = 1; }
-        else if (args.plain_permille < kOneMaskBelowPermille) { kernel = hmar_bwd_tc_kernel<false, STRIDED, true>; which = 2; }
-        const cudaError_t e = opt_in[which]((const void*)kernel, smem);
+        static SmemOptIn opt_in[2];
+        const bool one_mask = args.plain_permille < kOneMaskBelowPermille;
+        auto kernel = one_mask ? hmar_bwd_tc_kernel<STRIDED, true> : hmar_bwd_tc_kernel<STRIDED, false>;
+        const cudaError_t e = opt_in[one_mask]((const void*)kernel, smem);
         if (e != cudaSuccess) return e;
-        kernel<<<grid, NUM_THREADS, smem, stream>>>(q, k, v, dout_map, dq_acc_map, a);
+        kernel<<<grid, NUM_THREADS, smem, stream>>>(q, k, v, dout_map, dq_acc_map, args);
     }
     const size_t n8 = n_rows * D / 8;
     {

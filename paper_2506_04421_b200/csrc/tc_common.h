@@ -3,6 +3,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <algorithm>
 #include "hmar_common.h"
 
 namespace hmar {
@@ -37,19 +38,19 @@ struct BwdWork {
     int32_t row_begin, row_count;
     int32_t q_begin, q_end;
     int32_t uniform;
-    int32_t cost_begin;      // cost of the head's tiles before this one (see bwd_fill_costs)
+    int32_t class_count;     // tiles of the head that cost as much as this one; they follow one another (see bwd_fill_classes)
     int32_t pad[2];
 };
 
-// Cost model of the backward's persistent blocks: a tile costs its number of 128-query steps plus a
-// constant for the work at its start and end.  Fills cost_begin and returns the cost of a whole head.
-inline int bwd_fill_costs(BwdWork* work, int n) {
-    int acc = 0;
-    for (int i = 0; i < n; ++i) {
-        work[i].cost_begin = acc;
-        acc += (work[i].q_end - work[i].q_begin + 127) / 128 + 2;
+// A head's tiles in classes of equal cost (equal numbers of 128-query steps), the costliest first.
+inline void bwd_fill_classes(BwdWork* work, int n) {
+    auto steps = [](const BwdWork& w) { return (w.q_end - w.q_begin + 127) / 128; };
+    std::stable_sort(work, work + n, [&](const BwdWork& a, const BwdWork& b) { return steps(a) > steps(b); });
+    for (int i = 0, first = 0; i <= n; ++i) {
+        if (i < n && steps(work[i]) == steps(work[first])) continue;
+        for (int k = first; k < i; ++k) work[k].class_count = i - first;
+        first = i;
     }
-    return acc;
 }
 
 // Share, in thousandths, of a head's steps that belong to full tiles (128 key rows that all see the whole query
@@ -68,9 +69,7 @@ struct BwdArgs {
     const BwdWork* work;
     int n_work;
     int n_heads;             // B * H
-    int head_cost;           // from bwd_fill_costs
     int plain_permille;      // from bwd_plain_permille: picks the instantiation of the main kernel
-    int split;               // set by the launcher: runs per head dealt to the blocks in turn (0: one contiguous run per block)
     int L;
     float scale_log2;        // softmax_scale * log2(e)
     float softmax_scale;
