@@ -31,6 +31,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <cstddef>
+
 #include "hmar_common.h"
 #include "launchers.h"
 #include "ptx_sm100.cuh"
@@ -64,8 +66,9 @@ struct __align__(1024) SharedStorage {
     uint64_t k_full[NSTAGE], k_empty[NSTAGE], v_full[NSTAGE], v_empty[NSTAGE];
     uint64_t s_full, p_full, o_done;
     uint32_t tmem_base;
-    int abort_flag;
+    uint32_t gave_up;                       // offset of the barrier whose wait ran out (0: none did)
 };
+#define AT(field) (base + (uint32_t)offsetof(SharedStorage, field))     // shared-memory address
 
 struct KvTile {
     int seg;        // 0 or 1
@@ -108,14 +111,19 @@ __global__ void __launch_bounds__(NUM_THREADS, 4)
 hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k0,
                    const __grid_constant__ CUtensorMap map_v0, const __grid_constant__ CUtensorMap map_k1,
                    const __grid_constant__ CUtensorMap map_v1, const FwdArgs args) {
-    extern __shared__ uint8_t smem_raw[];
-    SharedStorage& sm = *reinterpret_cast<SharedStorage*>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    // aligned by its declaration, so that every shared-memory address is a constant of the code; checked below
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    SharedStorage& sm = *reinterpret_cast<SharedStorage*>(smem_raw);
+    const uint32_t base = smem_u32(&sm);
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
 
     // A block of this launch (or an earlier one) already gave up on a wait: do no further work.
     if (args.status != nullptr && *reinterpret_cast<volatile int*>(args.status) != 0) return;
+    if ((base & 1023u) != 0) {
+        if (threadIdx.x == 0) report_timeout(args.status, 0x3FF);
+        return;
+    }
 
     // ---- which tile of which head
     const int bh = blockIdx.x / args.n_work;
@@ -137,7 +145,7 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 
     // ---- set-up
     if (threadIdx.x == 0) {
-        sm.abort_flag = 0;
+        sm.gave_up = 0;
         mbar_init(&sm.q_full, 1);
         for (int s = 0; s < NSTAGE; ++s) {
             mbar_init(&sm.k_full[s], 1);
@@ -167,7 +175,11 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sm.tmem_base;
-    volatile int* abort_flag = &sm.abort_flag;
+    auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
+        if (warp_wait(bar, parity)) return true;
+        if (lane == 0) sm.gave_up = bar - base;
+        return false;
+    };
 
     if (warp >= PRODUCER_WARP) {
         reg_dec<REGS_MISC>();
@@ -187,18 +199,18 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 const int slot = j % NSTAGE;
                 const uint32_t par = ((j / NSTAGE) & 1) ^ 1;     // parity of the previous use of the slot
                 const KvTile t = kv_tile(w, tiles0, j);
-                if (j >= NSTAGE) ok = __all_sync(0xffffffffu, mbar_wait(&sm.k_empty[slot], par, abort_flag));
-                if (!ok) { if (lane == 0) report_timeout(args.status, 0x100 + j); break; }
+                if (j >= NSTAGE) ok = wait(AT(k_empty) + (slot) * 8, par);
+            if (!ok) break;
                 if (leader) {
-                    mbar_arrive_expect_tx(&sm.k_full[slot], TILE_BYTES);
-                    tma_load_4d(sm.k[slot], t.seg ? &map_k1 : &map_k0, &sm.k_full[slot], 0, t.coord, head, batch);
+                    bar_expect_tx(AT(k_full) + (slot) * 8, TILE_BYTES);
+                    tma_load_4d_at(AT(k) + slot * TILE_BYTES, t.seg ? &map_k1 : &map_k0, AT(k_full) + (slot) * 8, 0, t.coord, head, batch);
                 }
                 __syncwarp();
-                if (j >= NSTAGE) ok = __all_sync(0xffffffffu, mbar_wait(&sm.v_empty[slot], par, abort_flag));
-                if (!ok) { if (lane == 0) report_timeout(args.status, 0x200 + j); break; }
+                if (j >= NSTAGE) ok = wait(AT(v_empty) + (slot) * 8, par);
+            if (!ok) break;
                 if (leader) {
-                    mbar_arrive_expect_tx(&sm.v_full[slot], TILE_BYTES);
-                    tma_load_4d(sm.v[slot], t.seg ? &map_v1 : &map_v0, &sm.v_full[slot], 0, t.coord, head, batch);
+                    bar_expect_tx(AT(v_full) + (slot) * 8, TILE_BYTES);
+                    tma_load_4d_at(AT(v) + slot * TILE_BYTES, t.seg ? &map_v1 : &map_v0, AT(v_full) + (slot) * 8, 0, t.coord, head, batch);
                 }
                 __syncwarp();
             }
@@ -212,16 +224,11 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             // The whole warp runs the control flow; one elected lane issues.  Descriptors are built once and
             // advanced by adding (byte offset >> 4), so issuing an MMA costs a few instructions.
             const bool leader = elect_one();
-            const uint64_t q_kd = smem_desc_sw128(smem_u32(sm.q), 16);
-            const uint64_t k_kd0 = smem_desc_sw128(smem_u32(sm.k[0]), 16);      // ring slots are 8 KB apart
-            const uint64_t v_mn0 = smem_desc_sw128(smem_u32(sm.v[0]), 1024);
+            const uint64_t q_kd = smem_desc_sw128(AT(q), 16);
+            const uint64_t k_kd0 = smem_desc_sw128(AT(k), 16);      // ring slots are 8 KB apart
+            const uint64_t v_mn0 = smem_desc_sw128(AT(v), 1024);
             constexpr uint32_t idesc_pv = idesc_bf16_f32(BM, D, false, true);
             constexpr uint32_t SLOT_UNITS = TILE_BYTES >> 4;
-            auto wait = [&](uint64_t* bar, uint32_t parity, int code) -> bool {
-                if (__all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag))) return true;
-                if (lane == 0) report_timeout(args.status, code);
-                return false;
-            };
             // S = Q K^T for n keys of the tile in ring slot `slot`
             auto issue_s = [&](int n, int slot) {
                 const uint32_t idesc = idesc_bf16_f32(BM, n, false, false);
@@ -229,7 +236,7 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 #pragma unroll
                 for (int ks = 0; ks < D / 16; ++ks)
                     mma_ss(tmem + COL_S, q_kd + ks * 2, kd + ks * 2, idesc, ks > 0);
-                tc_commit(&sm.s_full);
+                commit_at(AT(s_full));
             };
             // O += P V for n keys
             auto issue_pv = [&](int n, int slot, bool first) {
@@ -243,15 +250,15 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 
             bool ok = true;
             {
-                const bool rq = mbar_try_wait(&sm.q_full, 0), rk = mbar_try_wait(&sm.k_full[0], 0);
-                if (!__all_sync(0xffffffffu, rq && rk))
-                    ok = (rq || wait(&sm.q_full, 0, 0x300)) && (rk || wait(&sm.k_full[0], 0, 0x400));
+                bool rq, rk;
+                warp_try_wait2(AT(q_full), 0, AT(k_full), 0, rq, rk);
+                ok = (rq || wait(AT(q_full), 0)) && (rk || wait(AT(k_full), 0));
             }
             if (ok) {
                 tc_fence_after();
                 if (leader) {
                     issue_s(tile_cols(kv_tile(w, tiles0, 0).n_valid), 0);
-                    if (NSTAGE < n_tiles) tc_commit(&sm.k_empty[0]);
+                    if (NSTAGE < n_tiles) commit_at(AT(k_empty) + (0) * 8);
                 }
                 __syncwarp();
             }
@@ -265,11 +272,11 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 // at a barrier is a shared-memory round trip, and after the softmax warps' arrival every such trip
                 // delays the products they are waiting for.
                 {
-                    const bool rv = mbar_try_wait(&sm.v_full[slot], (j / NSTAGE) & 1);
-                    const bool rk = !more || mbar_try_wait(&sm.k_full[slot_next], ((j + 1) / NSTAGE) & 1);
-                    if (!__all_sync(0xffffffffu, rv && rk))
-                        ok = (rv || wait(&sm.v_full[slot], (j / NSTAGE) & 1, 0x500 + j)) &&
-                             (rk || wait(&sm.k_full[slot_next], ((j + 1) / NSTAGE) & 1, 0x400 + j));
+                    const uint32_t v_bar = AT(v_full) + slot * 8, v_par = (j / NSTAGE) & 1;
+                    const uint32_t k_bar = more ? AT(k_full) + slot_next * 8 : v_bar, k_par = more ? ((j + 1) / NSTAGE) & 1 : v_par;
+                    bool rv, rk;
+                    warp_try_wait2(v_bar, v_par, k_bar, k_par, rv, rk);
+                    ok = (rv || wait(v_bar, v_par)) && (rk || wait(k_bar, k_par));
                 }
                 // The last tile of a key segment may be ragged: the rows between its last key and the next multiple of
                 // 16 (the granularity of the product over keys) belong to another scale, or to nobody.  Their P is
@@ -285,7 +292,7 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         __syncwarp();
                     }
                 }
-                if (ok) ok = wait(&sm.p_full, j & 1, 0x600 + j);
+                if (ok) ok = wait(AT(p_full), j & 1);
                 if (!ok) break;
                 tc_fence_after();
                 if (leader) {
@@ -295,9 +302,9 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     // free only if a later tile will use it (the block may exit as soon as the softmax warps have
                     // seen o_done: an arrival that lands after that would hit the barriers of the next block on
                     // this SM)
-                    if (j + NSTAGE < n_tiles) tc_commit(&sm.v_empty[slot]);
-                    if (j + 1 + NSTAGE < n_tiles) tc_commit(&sm.k_empty[slot_next]);
-                    if (!more) tc_commit(&sm.o_done);
+                    if (j + NSTAGE < n_tiles) commit_at(AT(v_empty) + (slot) * 8);
+                    if (j + 1 + NSTAGE < n_tiles) commit_at(AT(k_empty) + (slot_next) * 8);
+                    if (!more) commit_at(AT(o_done));
                 }
                 __syncwarp();
             }
@@ -331,8 +338,8 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             const bool two = n > 32;                           // second 32-column chunk present
             const bool need_mask = (!w.uniform) || (t.n_valid < (two ? 64 : 32));
 
-            ok = __all_sync(0xffffffffu, mbar_wait(&sm.s_full, j & 1, abort_flag));
-            if (!ok) { if (lane == 0) report_timeout(args.status, 0x800 + j); break; }
+            ok = wait(AT(s_full), j & 1);
+            if (!ok) break;
             tc_fence_after();
 
             tmem_ld32(s_addr, b0);
@@ -404,14 +411,11 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             l += l_add;
             tmem_st_wait();
             tc_fence_before();
-            mbar_arrive(&sm.p_full);
+            bar_arrive(AT(p_full));
         }
 
         // ---- epilogue: out = O / l, lse = ln(l) + m (natural log of the scaled logits' sum)
-        if (ok) {
-            ok = __all_sync(0xffffffffu, mbar_wait(&sm.o_done, 0, abort_flag));
-            if (!ok && lane == 0) report_timeout(args.status, 0xA00);
-        }
+        if (ok) ok = wait(AT(o_done), 0);
         if (ok) {
             tc_fence_after();
             const float inv = 1.f / l;
@@ -454,6 +458,7 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         tc_fence_after();
         tmem_dealloc(tmem, TMEM_COLS);
     }
+    if (threadIdx.x == 0 && sm.gave_up != 0) report_timeout(args.status, (int)sm.gave_up);
 }
 
 // Self-test of the bounded waits: one block waits on a barrier that nothing ever arrives on, with a limit of
@@ -480,7 +485,7 @@ cudaError_t launch_selftest_wait(int* status, cudaStream_t stream) {
     return cudaGetLastError();
 }
 
-size_t fwd_tc_smem_bytes() { return sizeof(SharedStorage) + 1024; }
+size_t fwd_tc_smem_bytes() { return sizeof(SharedStorage); }
 
 cudaError_t launch_fwd_tc(const CUtensorMap& q, const CUtensorMap& k0, const CUtensorMap& v0, const CUtensorMap& k1,
                           const CUtensorMap& v1, const FwdArgs& args, int BH, cudaStream_t stream) {
