@@ -309,6 +309,16 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 __syncwarp();
             }
         }
+    } else if (warp * 32 >= w.row_count) {
+        // ================================================================== softmax warp past the tile's last row
+        // It only answers: its rows of P hold whatever S left there and reach its rows of O alone.  A scale of 324 tokens
+        // has one such warp in twelve, one of 169 two in eight.
+        reg_inc<REGS_SOFTMAX>();
+#pragma unroll 1
+        for (int j = 0; j < n_tiles; ++j) {
+            if (!wait(AT(s_full), j & 1)) break;
+            bar_arrive(AT(p_full));
+        }
     } else {
         // ================================================================== softmax warps + epilogue
         reg_inc<REGS_SOFTMAX>();
