@@ -66,6 +66,7 @@ struct __align__(1024) SharedStorage {
     uint64_t k_full[NSTAGE], k_empty[NSTAGE], v_full[NSTAGE], v_empty[NSTAGE];
     uint64_t s_full, p_full, o_done;
     uint32_t tmem_base;
+    int skip;
     uint32_t gave_up;                       // offset of the barrier whose wait ran out (0: none did)
 };
 #define AT(field) (base + (uint32_t)offsetof(SharedStorage, field))     // shared-memory address
@@ -118,12 +119,12 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
 
-    // A block of this launch (or an earlier one) already gave up on a wait: do no further work.
-    if (args.status != nullptr && *reinterpret_cast<volatile int*>(args.status) != 0) return;
     if ((base & 1023u) != 0) {
         if (threadIdx.x == 0) report_timeout(args.status, 0x3FF);
         return;
     }
+    // whether a block of this launch (or an earlier one) already gave up on a wait: asked for now, looked at after the set-up
+    const int given_up = threadIdx.x == 0 && args.status != nullptr ? *reinterpret_cast<volatile int*>(args.status) : 0;
 
     // ---- which tile of which head
     const int bh = blockIdx.x / args.n_work;
@@ -171,6 +172,7 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         tmem_alloc(&sm.tmem_base, TMEM_COLS);
         tmem_relinquish();
     }
+    if (threadIdx.x == 0) sm.skip = given_up;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -181,7 +183,10 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         return false;
     };
 
-    if (warp >= PRODUCER_WARP) {
+    if (sm.skip != 0) {
+        // do no further work; the first copies have to land before the block's shared memory is given back
+        if (warp == 0) wait(AT(q_full), 0) && wait(AT(k_full), 0) && wait(AT(v_full), 0);
+    } else if (warp >= PRODUCER_WARP) {
         reg_dec<REGS_MISC>();
         if (warp == PRODUCER_WARP) {
             // ================================================================== TMA producer
@@ -432,31 +437,33 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             tmem_ld32(o_addr, b0);
             tmem_ld32(o_addr + 32, b1);
             tmem_ld_wait();
-            const long long out_off = batch * args.out_batch_stride + head * args.out_head_stride + row * args.out_row_stride;
             const long long lse_off = (long long)bh * args.n_q_rows + row;
-            if (row_ok && HMAR_IN_BOUNDS(out_off >= 0 && out_off + D <= args.out_extent, args.status, 0xB101) &&
-                HMAR_IN_BOUNDS(args.lse == nullptr || (lse_off >= 0 && lse_off < args.lse_extent), args.status, 0xB102)) {
-                uint4* dst = reinterpret_cast<uint4*>(args.out + out_off);
+            if (row_ok && args.lse != nullptr && HMAR_IN_BOUNDS(lse_off >= 0 && lse_off < args.lse_extent, args.status, 0xB102))
+                args.lse[lse_off] = (m_used + log2f(l)) * 0.6931471805599453f;
+            // The warp's 32 rows go through the shared memory of its own query rows (read for the last time by the products
+            // that o_done covers), 16-byte pieces swizzled by the row, so that a store instruction covers four whole rows and
+            // not a piece of each of 32 (L1 takes a line at a time: 256 lines a warp, now 32).
+            uint8_t* stage = sm.q + warp * 4096;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    uint4 v4;
-                    v4.x = pack_bf16(__uint_as_float(b0[8 * i + 0]) * inv, __uint_as_float(b0[8 * i + 1]) * inv);
-                    v4.y = pack_bf16(__uint_as_float(b0[8 * i + 2]) * inv, __uint_as_float(b0[8 * i + 3]) * inv);
-                    v4.z = pack_bf16(__uint_as_float(b0[8 * i + 4]) * inv, __uint_as_float(b0[8 * i + 5]) * inv);
-                    v4.w = pack_bf16(__uint_as_float(b0[8 * i + 6]) * inv, __uint_as_float(b0[8 * i + 7]) * inv);
-                    dst[i] = v4;
-                }
+            for (int i = 0; i < 8; ++i) {
+                const uint32_t* src = i < 4 ? b0 + 8 * i : b1 + 8 * (i - 4);
+                uint4 v4;
+                v4.x = pack_bf16(__uint_as_float(src[0]) * inv, __uint_as_float(src[1]) * inv);
+                v4.y = pack_bf16(__uint_as_float(src[2]) * inv, __uint_as_float(src[3]) * inv);
+                v4.z = pack_bf16(__uint_as_float(src[4]) * inv, __uint_as_float(src[5]) * inv);
+                v4.w = pack_bf16(__uint_as_float(src[6]) * inv, __uint_as_float(src[7]) * inv);
+                *reinterpret_cast<uint4*>(stage + lane * 128 + ((i ^ (lane & 7)) << 4)) = v4;
+            }
+            __syncwarp();
+            const int first = w.row_begin + warp * 32, piece = lane & 7;
+            const long long out_off = batch * args.out_batch_stride + head * args.out_head_stride + piece * 8;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    uint4 v4;
-                    v4.x = pack_bf16(__uint_as_float(b1[8 * i + 0]) * inv, __uint_as_float(b1[8 * i + 1]) * inv);
-                    v4.y = pack_bf16(__uint_as_float(b1[8 * i + 2]) * inv, __uint_as_float(b1[8 * i + 3]) * inv);
-                    v4.z = pack_bf16(__uint_as_float(b1[8 * i + 4]) * inv, __uint_as_float(b1[8 * i + 5]) * inv);
-                    v4.w = pack_bf16(__uint_as_float(b1[8 * i + 6]) * inv, __uint_as_float(b1[8 * i + 7]) * inv);
-                    dst[4 + i] = v4;
-                }
-                if (args.lse != nullptr)
-                    args.lse[lse_off] = (m_used + log2f(l)) * 0.6931471805599453f;
+            for (int i = 0; i < 8; ++i) {
+                const int rr = i * 4 + (lane >> 3);
+                const uint4 v4 = *reinterpret_cast<const uint4*>(stage + rr * 128 + ((piece ^ (rr & 7)) << 4));
+                const long long off = out_off + (first + rr) * args.out_row_stride;
+                if (warp * 32 + rr < w.row_count && HMAR_IN_BOUNDS(off >= 0 && off + 8 <= args.out_extent, args.status, 0xB101))
+                    *reinterpret_cast<uint4*>(args.out + off) = v4;
             }
         }
     }
