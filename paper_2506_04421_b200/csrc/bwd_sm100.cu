@@ -62,7 +62,7 @@ constexpr int ITEM_READERS = 15;     // warps that read every item: all but the 
 constexpr int NUM_COMPUTE_THREADS = 256;
 constexpr int DRAIN_WARP0 = 8, PRODUCER_WARP = 12, MMA_WARP = 13, AUX_WARP = 14, SCHED_WARP = 15;
 constexpr int NUM_THREADS = 512;
-constexpr int REGS_COMPUTE = 160, REGS_DRAIN = 88, REGS_MISC = 104;
+constexpr int REGS_COMPUTE = 152, REGS_DRAIN = 104, REGS_MISC = 104;
 static_assert(2 * REGS_COMPUTE + REGS_DRAIN + REGS_MISC == 4 * 128, "register budget of the block");
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t COL_ST = 0, COL_DPT = 128, COL_DK = 256, COL_DV = 320, COL_DQ = 384, COL_K = 448, COL_V = 480;
@@ -578,6 +578,7 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         const int quarter = warp & 3;
         const int r = quarter * 32 + lane;
         const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
+        const int sub_row = lane >> 3, piece = lane & 7;      // whole rows: lane's row among four and its 16-byte piece
         uint8_t* stage = sm.dq_stage + quarter * 4096;
         uint8_t* stage_row = stage + (lane >> 3) * 1024 + (lane & 7) * 128;
         if (lane == 0) prefetch_tensormap(&map_dq);
@@ -585,26 +586,31 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         bool ok = true;
         int gs = 0;
         // K and V rows of item gc (the block's item number `item`) to TMEM, one key row per thread: the A
-        // operands of S^T = K Q^T and dP^T = V dO^T.  The V row comes straight from global memory and waits
-        // in registers until the previous item's last scores have been computed; the K row is read from the
-        // tile that the copy engine has put into shared memory for the dQ products.  Rows past the end of
-        // the sequence are zeros.
+        // operands of S^T = K Q^T and dP^T = V dO^T.  The V rows come straight from global memory, four whole rows per
+        // load instruction and through the staging buffer into the thread that owns the row, and wait in registers until
+        // the previous item's last scores have been computed; the K row is read from the tile that the copy engine has put
+        // into shared memory for the dQ products.  Rows past the end of the sequence are zeros.
         auto copy_kv = [&](int item, bool wait_free) -> bool {
             const Item& wc = item_at(item);
-            const int row = wc.row_begin + r;
-            const uint4* vsrc;
-            if (STRIDED) {
-                vsrc = reinterpret_cast<const uint4*>(args.v + wc.batch * args.in_batch + wc.head * args.in_head + (long long)row * args.in_row);
-            } else {
-                vsrc = reinterpret_cast<const uint4*>(args.v + ((size_t)wc.bh * L + row) * D);
-            }
-            const long long v_off = reinterpret_cast<const __nv_bfloat16*>(vsrc) - args.v;
-            const bool v_in = row < L && HMAR_IN_BOUNDS(v_off >= 0 && v_off + D <= args.in_extent, args.status, 0xB202);
+            const int row0 = wc.row_begin + quarter * 32 + sub_row;
+            const __nv_bfloat16* vsrc = STRIDED ? args.v + wc.batch * args.in_batch + wc.head * args.in_head + row0 * args.in_row
+                                                : args.v + ((size_t)wc.bh * L + row0) * D;
+            const long long step = STRIDED ? 4 * args.in_row : 4 * D;
+            uint4 rows[8];
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
-                const uint4 val = v_in ? __ldg(vsrc + c) : make_uint4(0u, 0u, 0u, 0u);
-                buf[4 * c] = val.x; buf[4 * c + 1] = val.y; buf[4 * c + 2] = val.z; buf[4 * c + 3] = val.w;
+                const __nv_bfloat16* src = vsrc + c * step + piece * 8;
+                const bool v_in = row0 + 4 * c < L && HMAR_IN_BOUNDS(src >= args.v && src - args.v + 8 <= args.in_extent, args.status, 0xB202);
+                rows[c] = v_in ? __ldg(reinterpret_cast<const uint4*>(src)) : make_uint4(0u, 0u, 0u, 0u);
             }
+            if (lane == 0) bulk_wait_read_all();                // the last piece of dQ has been read out of the staging buffer
+            __syncwarp();
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                *reinterpret_cast<uint4*>(stage + (4 * c + sub_row) * 128 + ((piece ^ ((4 * c + sub_row) & 7)) << 4)) = rows[c];
+            __syncwarp();
+            load_swizzled_row(stage, lane, buf);
+            __syncwarp();
             if (wait_free) {
                 if (!wait(AT(kv_free), (item - 1) & 1)) return false;
                 tc_fence_after();
@@ -654,27 +660,37 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                             tc_fence_before();
                             bar_arrive(AT(acc_empty));         // the next item's products may overwrite dK / dV
                         }
-                        if (r < w.row_count) {
-                            const float mul = part < 2 ? args.softmax_scale : 1.f;
-                            __nv_bfloat16* base = part < 2 ? args.dk : args.dv;
-                            uint4* dst;
-                            if (STRIDED) {
-                                dst = reinterpret_cast<uint4*>(base + w.batch * args.g_batch + w.head * args.g_head +
-                                                               (long long)(w.row_begin + r) * args.g_row + (part & 1) * 32);
-                            } else {
-                                dst = reinterpret_cast<uint4*>(base + ((size_t)bh * L + w.row_begin + r) * D + (part & 1) * 32);
-                            }
-                            const long long g_off = reinterpret_cast<__nv_bfloat16*>(dst) - base;
-                            const bool g_in = HMAR_IN_BOUNDS(g_off >= 0 && g_off + 32 <= args.g_extent, args.status, 0xB203);
+                        // rows go through the staging buffer, so that a store instruction covers four whole rows (a thread
+                        // storing its own row touches 32 lines per instruction, which L1 takes one by one)
+                        const float mul = part < 2 ? args.softmax_scale : 1.f;
+                        if ((part & 1) == 0) {
+                            if (lane == 0) bulk_wait_read_all();
+                            __syncwarp();
+                        }
 #pragma unroll
-                            for (int t = 0; t < 4 && g_in; ++t) {
-                                uint4 o;
-                                o.x = pack_bf16(__uint_as_float(buf[8 * t + 0]) * mul, __uint_as_float(buf[8 * t + 1]) * mul);
-                                o.y = pack_bf16(__uint_as_float(buf[8 * t + 2]) * mul, __uint_as_float(buf[8 * t + 3]) * mul);
-                                o.z = pack_bf16(__uint_as_float(buf[8 * t + 4]) * mul, __uint_as_float(buf[8 * t + 5]) * mul);
-                                o.w = pack_bf16(__uint_as_float(buf[8 * t + 6]) * mul, __uint_as_float(buf[8 * t + 7]) * mul);
-                                dst[t] = o;
+                        for (int t = 0; t < 4; ++t) {
+                            uint4 o;
+                            o.x = pack_bf16(__uint_as_float(buf[8 * t + 0]) * mul, __uint_as_float(buf[8 * t + 1]) * mul);
+                            o.y = pack_bf16(__uint_as_float(buf[8 * t + 2]) * mul, __uint_as_float(buf[8 * t + 3]) * mul);
+                            o.z = pack_bf16(__uint_as_float(buf[8 * t + 4]) * mul, __uint_as_float(buf[8 * t + 5]) * mul);
+                            o.w = pack_bf16(__uint_as_float(buf[8 * t + 6]) * mul, __uint_as_float(buf[8 * t + 7]) * mul);
+                            *reinterpret_cast<uint4*>(stage_row + ((((part & 1) * 4 + t) ^ (lane & 7)) << 4)) = o;
+                        }
+                        if ((part & 1) == 1) {
+                            __syncwarp();
+                            __nv_bfloat16* base = part < 2 ? args.dk : args.dv;
+                            const int row0 = quarter * 32 + sub_row;
+                            __nv_bfloat16* dst = base + piece * 8 + (STRIDED ? w.batch * args.g_batch + w.head * args.g_head + (w.row_begin + row0) * args.g_row
+                                                                            : (long long)((size_t)bh * L + w.row_begin + row0) * D);
+                            const long long step = STRIDED ? 4 * args.g_row : 4 * D;
+#pragma unroll
+                            for (int c = 0; c < 8; ++c) {
+                                const uint4 o = *reinterpret_cast<const uint4*>(stage + (4 * c + sub_row) * 128 + ((piece ^ ((4 * c + sub_row) & 7)) << 4));
+                                __nv_bfloat16* at = dst + c * step;
+                                if (row0 + 4 * c < w.row_count && HMAR_IN_BOUNDS(at >= base && at - base + 8 <= args.g_extent, args.status, 0xB203))
+                                    *reinterpret_cast<uint4*>(at) = o;
                             }
+                            __syncwarp();
                         }
                     }
                 }
