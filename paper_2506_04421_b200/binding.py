@@ -152,7 +152,7 @@ def hmar_attn_fwd(q, k, v, side_lens, softmax_scale, out=None, lse=None, stream=
     if out is None:
         out = torch.empty_like(q)
     if lse is None:
-        lse = torch.empty((B, H, L), dtype=torch.float32, device=q.device)
+        lse = q.new_empty((B, H, L), dtype=torch.float32)
     sides, n = _sides(side_lens)
     if window != HMAR_WINDOW_MARKOV:
         fn = lib().hmar_attn_fwd_window_f32 if _is_f32(q) else lib().hmar_attn_fwd_window
@@ -173,9 +173,9 @@ def hmar_attn_fwd_packed(qkv, side_lens, softmax_scale, out=None, lse=None, stre
     if three != 3:
         raise ValueError("qkv must be [B, L, 3, H, D]")
     if out is None:
-        out = torch.empty((B, L, H, D), dtype=qkv.dtype, device=qkv.device)
+        out = qkv.new_empty((B, L, H, D))
     if lse is None:
-        lse = torch.empty((B, H, L), dtype=torch.float32, device=qkv.device)
+        lse = qkv.new_empty((B, H, L), dtype=torch.float32)
     sides, n = _sides(side_lens)
     _check(lib().hmar_attn_fwd_packed(_ptr(qkv), _ptr(out), _ptr(lse), B, H, D, n, sides, float(softmax_scale),
                                       _stream(stream)), "hmar_attn_fwd_packed")
@@ -191,7 +191,7 @@ def hmar_attn_bwd_packed(qkv, out, lse, dout, side_lens, softmax_scale, dqkv=Non
         raise ValueError("qkv must be bfloat16 [B, L, 3, H, D]")
     dqkv = torch.empty_like(qkv) if dqkv is None else dqkv
     if workspace is None:
-        workspace = torch.empty(hmar_attn_bwd_workspace_bytes(B, H, D, side_lens), dtype=torch.uint8, device=qkv.device)
+        workspace = qkv.new_empty(hmar_attn_bwd_workspace_bytes(B, H, D, side_lens), dtype=torch.uint8)
     sides, n = _sides(side_lens)
     _check(lib().hmar_attn_bwd_packed(_ptr(qkv), _ptr(out), _ptr(lse), _ptr(dout), _ptr(dqkv), _ptr(workspace),
                                       workspace.numel(), B, H, D, n, sides, float(softmax_scale), _stream(stream)),
@@ -214,8 +214,7 @@ def hmar_attn_bwd(q, k, v, out, lse, dout, side_lens, softmax_scale, dq=None, dk
     dk = torch.empty_like(q) if dk is None else dk
     dv = torch.empty_like(q) if dv is None else dv
     if workspace is None:
-        workspace = torch.empty(hmar_attn_bwd_workspace_bytes(B, H, D, side_lens), dtype=torch.uint8,
-                                device=q.device)
+        workspace = q.new_empty(hmar_attn_bwd_workspace_bytes(B, H, D, side_lens), dtype=torch.uint8)
     sides, n = _sides(side_lens)
     if window != HMAR_WINDOW_MARKOV:
         fn = lib().hmar_attn_bwd_window_f32 if _is_f32(q) else lib().hmar_attn_bwd_window
@@ -258,7 +257,7 @@ def hmar_attn_scale_step(q, k_prev, v_prev, k_cur, v_cur, side_prev, side_cur, s
     if out is None:
         out = torch.empty_like(q)
     if lse is None and want_lse:
-        lse = torch.empty((B, H, n_cur), dtype=torch.float32, device=q.device)
+        lse = q.new_empty((B, H, n_cur), dtype=torch.float32)
     fn = lib().hmar_attn_scale_step_f32 if _is_f32(q) else lib().hmar_attn_scale_step
     _check(fn(_ptr(q), _ptr(k_prev), _ptr(v_prev), _ptr(k_cur), _ptr(v_cur), _ptr(out), _ptr(lse),
               B, H, D, int(side_prev), int(side_cur), float(softmax_scale), _stream(stream)),
@@ -276,16 +275,17 @@ def hmar_attn_scale_step_strided(q, k_prev, v_prev, k_cur, v_cur, side_prev, sid
     def head_stride(t):
         if t is None:
             return 0
-        if not t.is_cuda or t.stride(3) != 1 or t.stride(2) != D or (t.shape[1] > 1 and t.shape[0] > 1 and t.stride(0) != H * t.stride(1)):
+        (b, h, rows, _), (sb, sh, sr, sd) = t.shape, t.stride()
+        if not t.is_cuda or sd != 1 or sr != D or (h > 1 and b > 1 and sb != H * sh):
             raise ValueError("views must have contiguous rows and evenly spaced heads")
-        return t.stride(1) if t.shape[1] > 1 else (t.stride(0) if t.shape[0] > 1 else t.shape[2] * D)
+        return sh if h > 1 else (sb if b > 1 else rows * D)
 
     if _is_f32(q):
         raise TypeError("hmar_attn_scale_step_strided takes bfloat16 tensors")
     if out is None:
-        out = torch.empty((B, H, n_cur, D), dtype=q.dtype, device=q.device)
+        out = q.new_empty((B, H, n_cur, D))
     if lse is None and want_lse:
-        lse = torch.empty((B, H, n_cur), dtype=torch.float32, device=q.device)
+        lse = q.new_empty((B, H, n_cur), dtype=torch.float32)
     _check(lib().hmar_attn_scale_step_strided(
         _ptr(q), _ptr(k_prev), _ptr(v_prev), _ptr(k_cur), _ptr(v_cur), _ptr(out), _ptr(lse), B, H, D, int(side_prev),
         int(side_cur), head_stride(q), head_stride(k_prev), head_stride(k_cur), head_stride(out), float(softmax_scale),
@@ -316,7 +316,7 @@ def hmar_recon_downsample(xhat, out_side, out=None, stream=None):
         raise TypeError("xhat must be float32")
     B, C, S, _ = xhat.shape
     if out is None:
-        out = torch.empty((B, C, out_side, out_side), dtype=torch.float32, device=xhat.device)
+        out = xhat.new_empty((B, C, out_side, out_side))
     elif out.dtype != torch.float32 or tuple(out.shape) != (B, C, out_side, out_side):
         raise ValueError("out must be float32 [B, C, out_side, out_side]")
     _check(lib().hmar_recon_downsample(_ptr(xhat), _ptr(out), B, C, S, int(out_side), _stream(stream)), "hmar_recon_downsample")
