@@ -8,10 +8,10 @@
 // (a = -0.75, half-pixel sample positions, border indices clamped) and add the result to the running
 // reconstruction in place.  The reconstruction is read and written exactly once (the algorithmic HBM bytes
 // of the step); the codebook (V x C fp32, 512 KB for V = 4096, C = 32) and the token maps stay in L2 / L1.
-// Two kernels: for token maps of at most 32 x 32 (every scale of the paper's schedules) a block takes one image
-// and stages the looked-up coarse map in shared memory; larger maps go through the plain kernel, in which a
-// thread owns one output pixel and walks the channels.  In both a warp's accesses to the [B, C, H, W] tensor
-// are 128-byte rows.
+// Three kernels: for reconstructions of at most 64 x 64 a block stages the looked-up coarse map of an image, or of a strip
+// of it, in shared memory; equal sizes are added without interpolation; larger reconstructions go through the plain
+// kernel, in which a thread owns one output pixel and walks the channels.  In all a warp's accesses to the
+// [B, C, H, W] tensor are rows of 128 bytes or more.
 #include <cuda_runtime.h>
 
 #include "hmar_common.h"
@@ -74,29 +74,60 @@ hmar_recon_accumulate_kernel(float* __restrict__ xhat, const float* __restrict__
     }
 }
 
-// Staged variant for token maps of at most 32 x 32 and reconstructions of at most 64 x 64: one block per image
-// and group of 8 channels.  The selected tokens' code values are gathered once into shared memory as a
-// channel-major coarse map (channel rows padded to 4 words past a multiple of 32, so the transposing stores spread
-// over the banks), then every warp takes a channel and walks down the output rows, interpolating separably from
-// shared memory and adding one 128-byte row segment into the reconstruction at a time.  Each code vector is
-// fetched once per image instead of once per output pixel and tap, and a launch at the sampler's batch still has
-// a few hundred blocks.
-constexpr int kStageMaxSide = 32;
+// Staged variant for reconstructions of at most 64 x 64: one block per image, group of 8 channels and strip of output
+// rows.  The selected tokens' code values that the strip needs are gathered once into shared memory as a channel-major
+// coarse map (channel rows padded to 4 words past a multiple of 32, so the transposing stores spread over the banks),
+// then every warp takes a channel and walks down the output rows, interpolating separably from shared memory and adding
+// one 128- or 256-byte row segment into the reconstruction at a time.  Each code vector is fetched once per strip instead of
+// once per output pixel and tap, and a launch at the sampler's batch still has a few hundred blocks.  Token maps of at
+// most 32 x 32 are one strip; larger ones are cut so that a strip's tokens fit (36 x 36 -> 64 x 64, 256 images: 1 095 us in
+// the plain kernel, 58 us in strips).
+constexpr int kStageTokens = 1024;                          // tokens a block stages
 constexpr int kStageChannels = 8;
 constexpr int kStageMaxOut = 64;
 
+// Adds W consecutive values to memory (8-byte aligned for W = 2) without waiting for them.
+template <int W>
+__device__ __forceinline__ void red_add(float* p, const float (&v)[W]) {
+    if (W == 2) asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(v[0]), "f"(v[W - 1]) : "memory");
+    else atomicAdd(p, v[0]);
+}
+
+__device__ __forceinline__ int selected_token(const int* tokens_old, const int* tokens_new, const unsigned char* mask, long long at) {
+    return (mask == nullptr || mask[at] != 0) ? tokens_new[at] : tokens_old[at];
+}
+
+// The output rows [y0, y1) of a strip and the source rows [r0, r1) that they read, with a row to spare on either side (in
+// whole numbers, so that the launcher and the kernel agree; the kernel's sample positions are floats).
+struct Strip { int y0, y1, r0, r1; };
+__host__ __device__ __forceinline__ Strip strip_rows(int strip, int n_strips, int side, int out_side) {
+    Strip s;
+    s.y0 = strip * out_side / n_strips;
+    s.y1 = (strip + 1) * out_side / n_strips;
+    const int lo = (2 * s.y0 + 1) * side / (2 * out_side) - 3, hi = (2 * s.y1 - 1) * side / (2 * out_side) + 3;
+    s.r0 = lo < 0 ? 0 : lo;
+    s.r1 = hi >= side ? side : hi + 1;
+    return s;
+}
+
+// W: output columns per lane.  Rows of more than 32 pixels go two at a time (8-byte reductions: 5.9 TB/s against 5.4 for
+// 64-pixel rows); for shorter ones half of the lanes would be idle.
+// STRIPS: false for maps that fit whole (16 x 16 images: 41 us for 2 048, 50 with the strip arithmetic).
+template <int W, bool STRIPS>
 __global__ void __launch_bounds__(256)
 hmar_recon_accumulate_staged_kernel(float* __restrict__ xhat, const float* __restrict__ codebook,
                                     const int* __restrict__ tokens_old, const int* __restrict__ tokens_new,
                                     const unsigned char* __restrict__ mask, int* __restrict__ tokens_out,
-                                    int C, int V, int side, int out_side, int n_groups) {
-    __shared__ float coarse[kStageChannels * (kStageMaxSide * kStageMaxSide + 4)];
-    __shared__ int ids[kStageMaxSide * kStageMaxSide];
+                                    int C, int V, int side, int out_side, int n_groups, int n_strips) {
+    __shared__ float coarse[kStageChannels * (kStageTokens + 4)];
+    __shared__ int ids[kStageTokens];
     __shared__ float4 row_w[kStageMaxOut];                  // per output row: the four vertical weights ...
     __shared__ int row_src[kStageMaxOut];                   // ... and the source row of the second one
-    const int b = blockIdx.x / n_groups, grp = blockIdx.x - b * n_groups;
+    const int unit = STRIPS ? blockIdx.x / n_strips : blockIdx.x, strip = STRIPS ? blockIdx.x - unit * n_strips : 0;
+    const int b = unit / n_groups, grp = unit - b * n_groups;
     const int c0 = grp * kStageChannels, nc = min(kStageChannels, C - c0);
-    const int n_tok = side * side;
+    const Strip rows = STRIPS ? strip_rows(strip, n_strips, side, out_side) : Strip{0, out_side, 0, side};
+    const int n_map = side * side, first = rows.r0 * side, n_tok = (rows.r1 - rows.r0) * side;
     const int stride = n_tok + ((4 - n_tok) & 31);          // = 4 mod 32: the gather's transposing stores miss each other's banks
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
     const float ratio = (float)side / (float)out_side;
@@ -108,12 +139,19 @@ hmar_recon_accumulate_staged_kernel(float* __restrict__ xhat, const float* __res
         row_w[threadIdx.x] = make_float4(wy[0], wy[1], wy[2], wy[3]);
         row_src[threadIdx.x] = iy;
     }
-    // ---- token selection (written out by the image's first channel group)
+    // ---- token selection (the map is written out by the image's first channel group, a share by each strip)
     for (int pos = threadIdx.x; pos < n_tok; pos += blockDim.x) {
-        const long long gp = (long long)b * n_tok + pos;
-        const int t = (mask == nullptr || mask[gp] != 0) ? tokens_new[gp] : tokens_old[gp];
-        if (tokens_out != nullptr && grp == 0) tokens_out[gp] = t;
+        const long long gp = (long long)b * n_map + first + pos;
+        const int t = selected_token(tokens_old, tokens_new, mask, gp);
+        if (!STRIPS && tokens_out != nullptr && grp == 0) tokens_out[gp] = t;
         ids[pos] = min(max(t, 0), V - 1);
+    }
+    if (STRIPS && tokens_out != nullptr && grp == 0) {
+        const int end = (strip + 1) * n_map / n_strips;
+        for (int pos = strip * n_map / n_strips + threadIdx.x; pos < end; pos += blockDim.x) {
+            const long long gp = (long long)b * n_map + pos;
+            tokens_out[gp] = selected_token(tokens_old, tokens_new, mask, gp);
+        }
     }
     __syncthreads();
     // ---- gather: a pair of lanes per token reads the group's 8 channels (32 bytes, one sector) as two 16-byte
@@ -134,7 +172,7 @@ hmar_recon_accumulate_staged_kernel(float* __restrict__ xhat, const float* __res
         }
     }
     __syncthreads();
-    // ---- interpolate and accumulate: lane per output column, warp per channel, walking down the output rows.
+    // ---- interpolate and accumulate: lane per W output columns, warp per channel, walking down the output rows.
     // The interpolation is separable: a source row's four horizontal taps are combined once (h) and reused by
     // every output row whose vertical window holds that source row; going down, the window of four h values
     // moves by at most one source row per output row (the step only ever enlarges a map), so an output value costs
@@ -142,39 +180,81 @@ hmar_recon_accumulate_staged_kernel(float* __restrict__ xhat, const float* __res
     // addition, issued as a reduction to memory: nothing waits for the old value, and with a single addend per
     // element the result does not depend on the order in which the reductions land.
     const long long plane = (long long)out_side * out_side;
-    for (int ox = lane; ox < out_side; ox += 32) {
-        const float sx = (ox + 0.5f) * ratio - 0.5f;
-        const int ix = (int)floorf(sx);
-        float wx[4];
-        cubic_weights(sx - (float)ix, wx);
-        int xx[4];
+    for (int ox = lane * W; ox < out_side; ox += 32 * W) {
+        float wx[W][4];
+        int xx[W][4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) xx[c] = min(max(ix - 1 + c, 0), side - 1);
+        for (int e = 0; e < W; ++e) {
+            const float sx = (ox + e + 0.5f) * ratio - 0.5f;
+            const int ix = (int)floorf(sx);
+            cubic_weights(sx - (float)ix, wx[e]);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) xx[e][c] = min(max(ix - 1 + c, 0), side - 1);
+        }
         for (int ch = warp; ch < nc; ch += n_warps) {
             const float* src = coarse + ch * stride;
-            auto hrow = [&](int r) -> float {
-                const float* row = src + min(max(r, 0), side - 1) * side;
-                float h = 0.f;
+            auto hrow = [&](int r, float (&h)[W]) {
+                const float* row = src + (min(max(r, 0), side - 1) - rows.r0) * side;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) h = fmaf(wx[c], row[xx[c]], h);
-                return h;
+                for (int e = 0; e < W; ++e) {
+                    h[e] = 0.f;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) h[e] = fmaf(wx[e][c], row[xx[e][c]], h[e]);
+                }
             };
-            float* dst = xhat + ((long long)b * C + c0 + ch) * plane + ox;
+            float* dst = xhat + ((long long)b * C + c0 + ch) * plane + (long long)rows.y0 * out_side + ox;
             int cur = -1000000;                             // source row of the window's second entry
-            float h0 = 0.f, h1 = 0.f, h2 = 0.f, h3 = 0.f;
+            float h0[W] = {}, h1[W] = {}, h2[W] = {}, h3[W] = {};
 #pragma unroll 4
-            for (int oy = 0; oy < out_side; ++oy, dst += out_side) {
+            for (int oy = rows.y0; oy < rows.y1; ++oy, dst += out_side) {
                 const int iy = row_src[oy];
                 const float4 wy = row_w[oy];
                 if (iy == cur + 1) {
-                    h0 = h1; h1 = h2; h2 = h3; h3 = hrow(iy + 2);
+#pragma unroll
+                    for (int e = 0; e < W; ++e) { h0[e] = h1[e]; h1[e] = h2[e]; h2[e] = h3[e]; }
+                    hrow(iy + 2, h3);
                 } else if (iy != cur) {
-                    h0 = hrow(iy - 1); h1 = hrow(iy); h2 = hrow(iy + 1); h3 = hrow(iy + 2);
+                    hrow(iy - 1, h0);
+                    hrow(iy, h1);
+                    hrow(iy + 1, h2);
+                    hrow(iy + 2, h3);
                 }
                 cur = iy;
-                atomicAdd(dst, fmaf(wy.w, h3, fmaf(wy.z, h2, fmaf(wy.y, h1, wy.x * h0))));
+                float o[W];
+#pragma unroll
+                for (int e = 0; e < W; ++e) o[e] = fmaf(wy.w, h3[e], fmaf(wy.z, h2[e], fmaf(wy.y, h1[e], wy.x * h0[e])));
+                red_add<W>(dst, o);
             }
         }
+    }
+}
+
+// Equal sizes (the last scale): every sample position is a pixel (weights 0, 1, 0, 0), so a code is added as it is.  A lane
+// takes a pixel and eight channels at a time: two 16-byte loads (one sector) of its code, eight reductions that are
+// coalesced over the lanes.  Nothing is staged.
+__global__ void __launch_bounds__(256)
+hmar_recon_accumulate_same_kernel(float* __restrict__ xhat, const float* __restrict__ codebook,
+                                  const int* __restrict__ tokens_old, const int* __restrict__ tokens_new,
+                                  const unsigned char* __restrict__ mask, int* __restrict__ tokens_out, int C, int V, int plane,
+                                  long long n_pix) {
+    const long long at = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (at >= n_pix) return;
+    const int t = selected_token(tokens_old, tokens_new, mask, at);
+    if (tokens_out != nullptr) tokens_out[at] = t;
+    const long long b = at / plane;
+    const float4* code = reinterpret_cast<const float4*>(codebook + (long long)min(max(t, 0), V - 1) * C);
+    float* dst = xhat + b * C * plane + (at - b * plane);
+#pragma unroll 4
+    for (int c = 0; c < C; c += 8, dst += 8ll * plane) {
+        const float4 u = __ldg(code + c / 4), v = __ldg(code + c / 4 + 1);
+        atomicAdd(dst, u.x);
+        atomicAdd(dst + plane, u.y);
+        atomicAdd(dst + 2 * plane, u.z);
+        atomicAdd(dst + 3 * plane, u.w);
+        atomicAdd(dst + 4 * plane, v.x);
+        atomicAdd(dst + 5 * plane, v.y);
+        atomicAdd(dst + 6 * plane, v.z);
+        atomicAdd(dst + 7 * plane, v.w);
     }
 }
 
@@ -331,12 +411,35 @@ hmar_recon_downsample_kernel(const float* __restrict__ xhat, float* __restrict__
 cudaError_t launch_recon_accumulate(float* xhat, const float* codebook, const int* tokens_old, const int* tokens_new,
                                     const unsigned char* mask, int* tokens_out, int B, int C, int V, int side, int out_side,
                                     cudaStream_t stream) {
-    if (side <= kStageMaxSide && out_side <= kStageMaxOut) {
-        const int n_groups = (C + kStageChannels - 1) / kStageChannels;
+    const bool rows16 = (C & 3) == 0 && (reinterpret_cast<uintptr_t>(codebook) & 15u) == 0;       // codes start on 16 bytes
+    if (side == out_side && (C & 7) == 0 && rows16) {
+        const long long n = (long long)B * side * side;
         {
             KernelTimer timer("hmar_recon_accumulate_kernel", stream);
-            hmar_recon_accumulate_staged_kernel<<<(unsigned)B * n_groups, 256, 0, stream>>>(xhat, codebook, tokens_old, tokens_new, mask,
-                                                                                            tokens_out, C, V, side, out_side, n_groups);
+            hmar_recon_accumulate_same_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(xhat, codebook, tokens_old, tokens_new, mask,
+                                                                                               tokens_out, C, V, side * side, n);
+        }
+        count_launch(1);
+        return cudaGetLastError();
+    }
+    if (out_side <= kStageMaxOut) {
+        const int n_groups = (C + kStageChannels - 1) / kStageChannels;
+        auto fits = [&](int n) {
+            for (int k = 0; k < n; ++k) {
+                const Strip r = strip_rows(k, n, side, out_side);
+                if ((r.r1 - r.r0) * side > kStageTokens) return false;
+            }
+            return true;
+        };
+        int n_strips = 1;                                   // 1 for side <= 32, at most 8
+        while (!fits(n_strips)) ++n_strips;
+        const bool pairs = out_side > 32 && (out_side & 1) == 0 && (reinterpret_cast<uintptr_t>(xhat) & 7u) == 0;
+        {
+            KernelTimer timer("hmar_recon_accumulate_kernel", stream);
+            auto kernel = n_strips > 1 ? (pairs ? hmar_recon_accumulate_staged_kernel<2, true> : hmar_recon_accumulate_staged_kernel<1, true>)
+                                       : (pairs ? hmar_recon_accumulate_staged_kernel<2, false> : hmar_recon_accumulate_staged_kernel<1, false>);
+            kernel<<<(unsigned)B * n_groups * n_strips, 256, 0, stream>>>(xhat, codebook, tokens_old, tokens_new, mask, tokens_out, C, V, side,
+                                                                           out_side, n_groups, n_strips);
         }
         count_launch(1);
         return cudaGetLastError();

@@ -646,6 +646,31 @@ def test_recon_downsample_matches_oracle(S, s, B, C):
     assert all(intact() for intact in guards)
 
 
+@pytest.mark.parametrize("side,out_side,C", [(33, 34, 8), (33, 64, 24), (41, 63, 8), (63, 64, 8), (47, 48, 12), (64, 64, 16), (1, 1, 8), (33, 33, 16),
+                                             (70, 70, 8), (31, 31, 12)])
+def test_recon_accumulate_strips_and_equal_sizes(side, out_side, C):
+    """Token maps of more than 32 x 32, which the staged kernel takes in strips of output rows (rows shared by two
+    strips, odd output sides, a channel group cut short), and equal sizes, which are added without interpolation
+    (C a multiple of 8) or go through the other kernels.  Weights and sums as in the test above: 1e-5 relative."""
+    rng = np.random.default_rng(100 * side + out_side)
+    B, V = 2, 70
+    codebook = rng.standard_normal((V, C)).astype(np.float32)
+    old, new = (rng.integers(0, V, (B, side, side)).astype(np.int32) for _ in range(2))
+    mask = rng.integers(0, 2, (B, side, side)).astype(np.uint8)
+    x0 = rng.standard_normal((B, C, out_side, out_side)).astype(np.float32)
+    guards = []
+    xhat = _guarded(x0.shape, torch.float32, guards)
+    xhat.copy_(torch.from_numpy(x0))
+    t_out = torch.full((B, side, side), -1, dtype=torch.int32, device="cuda")
+    hmar.hmar_recon_accumulate(xhat, *(torch.from_numpy(a).cuda() for a in (codebook, new, old, mask)), t_out)
+    sel = orc.select_tokens(old, new, mask)
+    ref = orc.recon_accumulate(x0, codebook, sel, out_side)
+    assert torch.equal(t_out.cpu(), torch.from_numpy(sel.astype(np.int32)))
+    err = np.abs(xhat.double().cpu().numpy() - ref)
+    assert err.max() <= 1e-5 * max(1.0, np.abs(ref).max()), f"max abs err {err.max():.3e}"
+    assert all(intact() for intact in guards)
+
+
 def test_recon_accumulate_codebook_off_16_byte_alignment():
     """A codebook whose base address is not a multiple of 16 bytes takes the staged kernel's one-value-at-a-time
     gather; same result as the oracle."""
