@@ -114,7 +114,7 @@ extern "C" int hmar_attn_bwd_noalloc(const void* q, const void* k, const void* v
         host_work[i].q_end = tiles[i].partner_end;
         host_work[i].uniform = tiles[i].uniform;
     }
-    bwd_fill_classes(host_work, (int)tiles.size());
+    const int head_steps = bwd_fill_classes(host_work, (int)tiles.size());
     const int plain_permille = bwd_plain_permille(host_work, (int)tiles.size());
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     for (size_t first = 0; first < tiles.size(); first += kFillChunk) {
@@ -137,6 +137,7 @@ extern "C" int hmar_attn_bwd_noalloc(const void* q, const void* k, const void* v
     a.work = reinterpret_cast<const BwdWork*>(scratch);
     a.n_work = (int)tiles.size();
     a.n_heads = BH;
+    a.head_steps = head_steps;
     a.plain_permille = plain_permille;
     a.L = (int)L;
     a.scale_log2 = softmax_scale * 1.4426950408889634f;

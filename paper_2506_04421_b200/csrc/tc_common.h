@@ -42,8 +42,9 @@ struct BwdWork {
     int32_t pad[2];
 };
 
-// A head's tiles in classes of equal cost (equal numbers of 128-query steps), the costliest first.
-inline void bwd_fill_classes(BwdWork* work, int n) {
+// A head's tiles in classes of equal cost (equal numbers of 128-query steps), the costliest first; returns the sum of
+// the steps.
+inline int bwd_fill_classes(BwdWork* work, int n) {
     auto steps = [](const BwdWork& w) { return (w.q_end - w.q_begin + 127) / 128; };
     std::stable_sort(work, work + n, [&](const BwdWork& a, const BwdWork& b) { return steps(a) > steps(b); });
     for (int i = 0, first = 0; i <= n; ++i) {
@@ -51,6 +52,9 @@ inline void bwd_fill_classes(BwdWork* work, int n) {
         for (int k = first; k < i; ++k) work[k].class_count = i - first;
         first = i;
     }
+    int total = 0;
+    for (int i = 0; i < n; ++i) total += steps(work[i]);
+    return total;
 }
 
 // Share, in thousandths, of a head's steps that belong to full tiles (128 key rows that all see the whole query
@@ -70,6 +74,8 @@ struct BwdArgs {
     int n_work;
     int n_heads;             // B * H
     int plain_permille;      // from bwd_plain_permille: picks the instantiation of the main kernel
+    int head_steps;          // steps of all tiles of a head (from bwd_fill_classes)
+    int by_head;             // set by the launcher: items in head order instead of class by class
     int L;
     float scale_log2;        // softmax_scale * log2(e)
     float softmax_scale;

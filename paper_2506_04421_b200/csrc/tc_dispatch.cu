@@ -75,6 +75,7 @@ struct Plan {
     BwdWork* bwd_work = nullptr;
     int n_fwd = 0;
     int n_bwd = 0;
+    int bwd_head_steps = 0;
     int bwd_plain_permille = 1000;
     int zero_begin = 0, zero_end = 0;   // key rows of a head that no query sees: their dK, dV are zeros
 };
@@ -145,7 +146,7 @@ static const Plan* get_plan(const ScaleTable& st) {
     Plan plan;
     std::vector<BwdWork> bwork = make_bwd_work(st, plan.zero_begin, plan.zero_end);
     static_assert(sizeof(FwdWork) == sizeof(BwdWork), "work tiles share one allocation");
-    bwd_fill_classes(bwork.data(), (int)bwork.size());
+    plan.bwd_head_steps = bwd_fill_classes(bwork.data(), (int)bwork.size());
     plan.bwd_plain_permille = bwd_plain_permille(bwork.data(), (int)bwork.size());
     plan.n_fwd = (int)work.size();
     plan.n_bwd = (int)bwork.size();
@@ -290,6 +291,7 @@ static int tc_bwd_strided(const bf16* q, const bf16* k, const bf16* v, const bf1
     a.work = plan->bwd_work;
     a.n_work = plan->n_bwd;
     a.n_heads = BH;
+    a.head_steps = plan->bwd_head_steps;
     a.plain_permille = plan->bwd_plain_permille;
     a.L = L;
     a.scale_log2 = scale * 1.4426950408889634f;
