@@ -8,7 +8,8 @@
 // 16-byte shared-memory loads feed 128 FMAs, which leaves the FMA pipe as the bound (a warp's loads take half of the
 // shared-memory cycles its FMAs last).  One row per thread pair, an operand of every FMA from shared memory, was bound
 // by those loads: B2 H16 L680 D64, forward + backward, 954 us, against 70 us of FMAs.
-// Tiles of the last (largest) scale come first in the grid.
+// Blocks are ordered tile by tile over all heads, the tiles of the last (largest) scale first, so that the costly blocks
+// start first and spread over the SMs (head by head, an SM could get three of them and another none).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include "hmar_common.h"
@@ -152,11 +153,11 @@ __global__ void __launch_bounds__(THREADS)
 simt_fwd_kernel(const T* __restrict__ q, const T* __restrict__ k0, const T* __restrict__ v0,
                 const T* __restrict__ k1, const T* __restrict__ v1,
                 T* __restrict__ out, float* __restrict__ lse,
-                const __grid_constant__ ScaleTable st, int n_q, int n0, int n1, int dense, float scale) {
+                const __grid_constant__ ScaleTable st, int n_heads, int n_q, int n0, int n1, int dense, float scale) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     FwdSmem<D>& sm = *reinterpret_cast<FwdSmem<D>*>(smem_raw);
-    const int bh = blockIdx.y;
-    const TileRows tile = tile_rows(st, blockIdx.x);
+    const int bh = blockIdx.x % n_heads;
+    const TileRows tile = tile_rows(st, blockIdx.x / n_heads);
     const int tx = threadIdx.x & 15, r0 = (threadIdx.x >> 4) * 8;
     const bool live = (threadIdx.x >> 5) * 16 < tile.n;     // the warp has rows of the tile
     const int lo = dense ? 0 : st.start[first_key_scale(st.window, tile.s)];
@@ -249,8 +250,8 @@ simt_delta_kernel(const T* __restrict__ out, const T* __restrict__ dout, float* 
 }
 
 // ---------------------------------------------------------------------------------------------
-// Backward: the first half of the grid owns key tiles (dK, dV over the queries that see them), the second half query
-// tiles (dQ over their keys); one launch, so that both halves fill the chip together.  Each result has one owner that
+// Backward: a tile's first block owns it as a key tile (dK, dV over the queries that see it), its second as a query tile
+// (dQ over its keys); one launch, so that both kinds fill the chip together.  Each result has one owner that
 // adds in a fixed order: the gradients are bit-reproducible.
 template <int D> struct BwdSmem { RowTile<D> a, b, x, y; SquareTile p; float lse[TR], delta[TR]; };
 
@@ -259,12 +260,13 @@ __global__ void __launch_bounds__(THREADS)
 simt_bwd_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
                 const T* __restrict__ dout, const float* __restrict__ lse, const float* __restrict__ delta,
                 T* __restrict__ dq, T* __restrict__ dk, T* __restrict__ dv,
-                const __grid_constant__ ScaleTable st, int L, int n_tiles, float scale) {
+                const __grid_constant__ ScaleTable st, int n_heads, int L, float scale) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     BwdSmem<D>& sm = *reinterpret_cast<BwdSmem<D>*>(smem_raw);
-    const size_t head = (size_t)blockIdx.y * L;
-    const bool keys = (int)blockIdx.x < n_tiles;            // the block owns a key tile
-    const TileRows tile = tile_rows(st, keys ? blockIdx.x : blockIdx.x - n_tiles);
+    const int unit = blockIdx.x / n_heads;
+    const size_t head = (size_t)(blockIdx.x - unit * n_heads) * L;
+    const bool keys = (unit & 1) == 0;                      // the block owns a key tile
+    const TileRows tile = tile_rows(st, unit >> 1);
     const int tx = threadIdx.x & 15, r0 = (threadIdx.x >> 4) * 8;
     const bool live = (threadIdx.x >> 5) * 16 < tile.n;     // the warp has rows of the tile
     // Own rows a, b against partner rows x, y: keys own K, V and walk Q, dO; queries own Q, dO and walk K, V.
@@ -357,8 +359,8 @@ static cudaError_t simt_fwd_any(const T* q, const T* k0, const T* v0, const T* k
     static SmemOptIn opt_in;
     const cudaError_t e = opt_in((const void*)simt_fwd_kernel<T, D>, sizeof(FwdSmem<D>));
     if (e != cudaSuccess) return e;
-    simt_fwd_kernel<T, D><<<dim3(count_tiles(st), BH), THREADS, sizeof(FwdSmem<D>), stream>>>(q, k0, v0, k1, v1, out, lse, st, n_q, n0, n1,
-                                                                                             dense, scale);
+    simt_fwd_kernel<T, D><<<(unsigned)count_tiles(st) * BH, THREADS, sizeof(FwdSmem<D>), stream>>>(q, k0, v0, k1, v1, out, lse, st, BH, n_q,
+                                                                                                 n0, n1, dense, scale);
     count_launch(1);
     return cudaGetLastError();
 }
@@ -392,9 +394,8 @@ static cudaError_t simt_bwd_d(const T* q, const T* k, const T* v, const T* out, 
     const cudaError_t e = opt_in((const void*)simt_bwd_kernel<T, D>, sizeof(BwdSmem<D>));
     if (e != cudaSuccess) return e;
     simt_delta_kernel<T, D><<<(unsigned)((n_rows + THREADS / 2 - 1) / (THREADS / 2)), THREADS, 0, stream>>>(out, dout, delta, n_rows);
-    const int n_tiles = count_tiles(st);
-    simt_bwd_kernel<T, D><<<dim3(2 * n_tiles, BH), THREADS, sizeof(BwdSmem<D>), stream>>>(q, k, v, dout, lse, delta, dq, dk, dv, st, L,
-                                                                                         n_tiles, scale);
+    simt_bwd_kernel<T, D><<<2u * count_tiles(st) * BH, THREADS, sizeof(BwdSmem<D>), stream>>>(q, k, v, dout, lse, delta, dq, dk, dv, st, BH, L,
+                                                                                            scale);
     count_launch(2);
     return cudaGetLastError();
 }
