@@ -31,6 +31,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstddef>
 
 #include "hmar_common.h"
@@ -127,8 +128,17 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     const int given_up = threadIdx.x == 0 && args.status != nullptr ? *reinterpret_cast<volatile int*>(args.status) : 0;
 
     // ---- which tile of which head
-    const int bh = blockIdx.x / args.n_work;
-    const int wi = blockIdx.x % args.n_work;
+    int bh, wi;
+    if (args.work != nullptr) {
+        const int group = blockIdx.x / (args.group_heads * args.n_work);
+        const int first_head = group * args.group_heads, in_group = blockIdx.x - first_head * args.n_work;
+        const int heads = min(args.group_heads, args.n_heads - first_head);
+        wi = in_group / heads;
+        bh = first_head + in_group - wi * heads;
+    } else {
+        bh = blockIdx.x / args.n_work;
+        wi = blockIdx.x - bh * args.n_work;
+    }
     const int batch = bh / args.heads_per_batch, head = bh - batch * args.heads_per_batch;
     FwdWork w;
     if (args.work != nullptr) {
@@ -205,14 +215,14 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 const uint32_t par = ((j / NSTAGE) & 1) ^ 1;     // parity of the previous use of the slot
                 const KvTile t = kv_tile(w, tiles0, j);
                 if (j >= NSTAGE) ok = wait(AT(k_empty) + (slot) * 8, par);
-            if (!ok) break;
+                if (!ok) break;
                 if (leader) {
                     bar_expect_tx(AT(k_full) + (slot) * 8, TILE_BYTES);
                     tma_load_4d_at(AT(k) + slot * TILE_BYTES, t.seg ? &map_k1 : &map_k0, AT(k_full) + (slot) * 8, 0, t.coord, head, batch);
                 }
                 __syncwarp();
                 if (j >= NSTAGE) ok = wait(AT(v_empty) + (slot) * 8, par);
-            if (!ok) break;
+                if (!ok) break;
                 if (leader) {
                     bar_expect_tx(AT(v_full) + (slot) * 8, TILE_BYTES);
                     tma_load_4d_at(AT(v) + slot * TILE_BYTES, t.seg ? &map_v1 : &map_v0, AT(v_full) + (slot) * 8, 0, t.coord, head, batch);
@@ -502,6 +512,8 @@ cudaError_t launch_selftest_wait(int* status, cudaStream_t stream) {
     return cudaGetLastError();
 }
 
+constexpr size_t kGroupBytes = 128000000;      // L2 holds 126 MiB
+
 size_t fwd_tc_smem_bytes() { return sizeof(SharedStorage); }
 
 cudaError_t launch_fwd_tc(const CUtensorMap& q, const CUtensorMap& k0, const CUtensorMap& v0, const CUtensorMap& k1,
@@ -511,9 +523,21 @@ cudaError_t launch_fwd_tc(const CUtensorMap& q, const CUtensorMap& k0, const CUt
     const cudaError_t e = opt_in((const void*)hmar_fwd_tc_kernel, smem);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)BH * (unsigned)args.n_work;
+    // The blocks of a training pass go group by group of heads and, inside a group, costliest tiles first over its heads:
+    // with all tiles of a head in turn, the last blocks to start hold costly tiles and the launch ends in a thin wave.
+    // A group's Q, K and V are what L2 holds, since a head's rows are read once per tile of the head: one group of all
+    // heads is slower where they exceed it (L = 2240, 384 heads: 425 us, head by head 412).  Head by head -> groups, us:
+    // L = 2240 96 heads 115 -> 100, 192 heads 200 -> 186, 384 heads 365 -> 352; L = 9451 48 heads 675 -> 610, 192 heads
+    // 2355 -> 2295; L = 680 128 heads 30 -> 26; L = 1000 192 heads 55 -> 49; L = 1300 39 heads 43 -> 34; L = 680 960
+    // heads and L = 395 768 heads equal.  Groups of 48 MB are 1 to 4 % slower than these, of 96 or 160 MB equal.
+    // The tiles of an inference step all cost the same, and stay head by head (groups: 0 to 15 % slower).
+    FwdArgs a = args;
+    const size_t groups = (BH * args.head_bytes + kGroupBytes - 1) / kGroupBytes;
+    a.n_heads = BH;
+    a.group_heads = (int)((BH + groups - 1) / groups);
     {
         KernelTimer timer(args.work != nullptr ? "hmar_fwd_tc_kernel" : "hmar_fwd_tc_kernel/scale_step", stream);
-        hmar_fwd_tc_kernel<<<grid, NUM_THREADS, smem, stream>>>(q, k0, v0, k1, v1, args);
+        hmar_fwd_tc_kernel<<<grid, NUM_THREADS, smem, stream>>>(q, k0, v0, k1, v1, a);
     }
     count_launch(1);
     return cudaGetLastError();

@@ -22,6 +22,9 @@ struct FwdArgs {
     const FwdWork* work;     // n_work tiles per head; nullptr = inference step (tiles derived in-kernel)
     int n_work;
     int n_q_rows;            // rows per head of q / out / lse
+    size_t head_bytes;       // Q, K and V of one head
+    int n_heads;             // set by the launcher, as group_heads: the blocks go group by group of this many heads, and
+    int group_heads;         // tile by tile over the heads of a group
     int heads_per_batch;     // H: head bh is head bh % H of batch bh / H (the tensor maps are 4-D: D, rows, H, B)
     long long out_row_stride, out_head_stride, out_batch_stride;   // of `out`, in elements (lse is always [B*H, rows])
     long long out_extent, lse_extent;   // elements reachable through out / lse (read by the checking build only)

@@ -198,6 +198,7 @@ static int tc_fwd_strided(const bf16* q, const bf16* k, const bf16* v, bf16* out
     a.work = plan->fwd_work;
     a.n_work = plan->n_fwd;
     a.n_q_rows = L;
+    a.head_bytes = (size_t)L * 3 * kHeadDim * sizeof(bf16);
     a.heads_per_batch = H;
     a.out_row_stride = out_row;
     a.out_head_stride = out_head;
@@ -254,6 +255,7 @@ int tc_scale_step(const bf16* q, const bf16* k_prev, const bf16* v_prev, const b
     a.work = nullptr;
     a.n_work = (n_cur + kTileRows - 1) / kTileRows;
     a.n_q_rows = n_cur;
+    a.head_bytes = (size_t)(3 * n_cur + 2 * n_prev) * kHeadDim * sizeof(bf16);
     a.heads_per_batch = BH;
     a.out_row_stride = kHeadDim;
     a.out_head_stride = st.out;
