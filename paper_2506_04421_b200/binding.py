@@ -1,4 +1,4 @@
-"""ctypes binding of libhmar.so: argument marshalling only.
+"""Binding of libhmar.so: argument marshalling only, for the hot calls in a compiled module, for the others by ctypes.
 
 Every function here has the name and argument order of the C entry point it wraps (see
 include/hmar.h). Tensors are torch CUDA tensors used purely as device buffers; all of the
@@ -7,6 +7,8 @@ is missing or fails to load, importing this module raises.
 """
 import ctypes
 import functools
+import importlib.machinery
+import importlib.util
 import os
 
 import torch
@@ -14,6 +16,7 @@ import torch
 from . import build as _build
 
 _LIB = None
+_HOST = None
 
 HMAR_OK = 0
 HMAR_ERR_BAD_ARG = -1
@@ -108,8 +111,6 @@ def _sides(side_lens):
     return _sides_array(tuple(map(int, side_lens)))
 
 
-# A call of a coarse scale is host time only (14 us, 3 of them a Stream object built to read one integer, 2 the wrapping of
-# every pointer in a ctypes object), so pointers and the stream go to the library as plain integers: 7 us.
 def _ptr(t):
     return None if t is None else t.data_ptr()
 
@@ -123,6 +124,33 @@ def _stream(stream):
     if _current_raw_stream is not None:
         return _current_raw_stream(torch.cuda.current_device())
     return torch.cuda.current_stream().cuda_stream
+
+
+def _host():
+    """The compiled module that checks the tensors, allocates the results and makes the call (csrc/host_binding.cpp)."""
+    return _HOST if _HOST is not None else _load_host()
+
+
+def _load_host():
+    global _HOST
+    library = lib()
+    loader = importlib.machinery.ExtensionFileLoader("_hmar_host", _build.build_host())
+    module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_hmar_host", loader))
+    loader.exec_module(module)
+    module.bind(library._handle)
+    _HOST = module
+    return module
+
+
+def _handle(stream):
+    return None if stream is None else stream.cuda_stream
+
+
+def _done(result, where):
+    """What a function of the compiled module returned: its results, or the library's status."""
+    if result.__class__ is int:
+        raise HmarError(result, where)
+    return result
 
 
 def _check(status, where):
@@ -147,56 +175,19 @@ def _need(*tensors):
 def hmar_attn_fwd(q, k, v, side_lens, softmax_scale, out=None, lse=None, stream=None, window=HMAR_WINDOW_MARKOV):
     """Training forward. q, k, v: [B,H,L,D]. Returns (out [B,H,L,D], lse [B,H,L] fp32).
     `window` other than HMAR_WINDOW_MARKOV goes through hmar_attn_fwd_window."""
-    _need(q, k, v, out, lse)
-    B, H, L, D = q.shape
-    if out is None:
-        out = torch.empty_like(q)
-    if lse is None:
-        lse = q.new_empty((B, H, L), dtype=torch.float32)
-    sides, n = _sides(side_lens)
-    if window != HMAR_WINDOW_MARKOV:
-        fn = lib().hmar_attn_fwd_window_f32 if _is_f32(q) else lib().hmar_attn_fwd_window
-        _check(fn(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), B, H, D, n, sides, int(window),
-                  float(softmax_scale), _stream(stream)), "hmar_attn_fwd_window")
-        return out, lse
-    fn = lib().hmar_attn_fwd_f32 if _is_f32(q) else lib().hmar_attn_fwd
-    _check(fn(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), B, H, D, n, sides,
-              float(softmax_scale), _stream(stream)), "hmar_attn_fwd")
-    return out, lse
+    return _done(_host().fwd(q, k, v, out, lse, side_lens, softmax_scale, _handle(stream), window), "hmar_attn_fwd")
 
 
 def hmar_attn_fwd_packed(qkv, side_lens, softmax_scale, out=None, lse=None, stream=None):
     """Training forward on the packed projection output. qkv: [B,L,3,H,D] bf16.
     Returns (out [B,L,H,D], lse [B,H,L] fp32)."""
-    _need(qkv, out, lse)
-    B, L, three, H, D = qkv.shape
-    if three != 3:
-        raise ValueError("qkv must be [B, L, 3, H, D]")
-    if out is None:
-        out = qkv.new_empty((B, L, H, D))
-    if lse is None:
-        lse = qkv.new_empty((B, H, L), dtype=torch.float32)
-    sides, n = _sides(side_lens)
-    _check(lib().hmar_attn_fwd_packed(_ptr(qkv), _ptr(out), _ptr(lse), B, H, D, n, sides, float(softmax_scale),
-                                      _stream(stream)), "hmar_attn_fwd_packed")
-    return out, lse
+    return _done(_host().fwd_packed(qkv, out, lse, side_lens, softmax_scale, _handle(stream)), "hmar_attn_fwd_packed")
 
 
 def hmar_attn_bwd_packed(qkv, out, lse, dout, side_lens, softmax_scale, dqkv=None, workspace=None, stream=None):
     """Training backward on the packed layouts. qkv [B,L,3,H,D], out and dout [B,L,H,D], lse [B,H,L].
     Returns dqkv [B,L,3,H,D]."""
-    _need(qkv, out, lse, dout, dqkv, workspace)
-    B, L, three, H, D = qkv.shape
-    if three != 3 or _is_f32(qkv):
-        raise ValueError("qkv must be bfloat16 [B, L, 3, H, D]")
-    dqkv = torch.empty_like(qkv) if dqkv is None else dqkv
-    if workspace is None:
-        workspace = qkv.new_empty(hmar_attn_bwd_workspace_bytes(B, H, D, side_lens), dtype=torch.uint8)
-    sides, n = _sides(side_lens)
-    _check(lib().hmar_attn_bwd_packed(_ptr(qkv), _ptr(out), _ptr(lse), _ptr(dout), _ptr(dqkv), _ptr(workspace),
-                                      workspace.numel(), B, H, D, n, sides, float(softmax_scale), _stream(stream)),
-           "hmar_attn_bwd_packed")
-    return dqkv
+    return _done(_host().bwd_packed(qkv, out, lse, dout, side_lens, softmax_scale, dqkv, workspace, _handle(stream)), "hmar_attn_bwd_packed")
 
 
 def hmar_attn_bwd_workspace_bytes(B, H, D, side_lens):
@@ -208,25 +199,7 @@ def hmar_attn_bwd(q, k, v, out, lse, dout, side_lens, softmax_scale, dq=None, dk
                   workspace=None, stream=None, window=HMAR_WINDOW_MARKOV):
     """Training backward. Returns (dq, dk, dv), each [B,H,L,D].
     `window` other than HMAR_WINDOW_MARKOV goes through hmar_attn_bwd_window."""
-    _need(q, k, v, out, lse, dout, dq, dk, dv, workspace)
-    B, H, L, D = q.shape
-    dq = torch.empty_like(q) if dq is None else dq
-    dk = torch.empty_like(q) if dk is None else dk
-    dv = torch.empty_like(q) if dv is None else dv
-    if workspace is None:
-        workspace = q.new_empty(hmar_attn_bwd_workspace_bytes(B, H, D, side_lens), dtype=torch.uint8)
-    sides, n = _sides(side_lens)
-    if window != HMAR_WINDOW_MARKOV:
-        fn = lib().hmar_attn_bwd_window_f32 if _is_f32(q) else lib().hmar_attn_bwd_window
-        _check(fn(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), _ptr(dout), _ptr(dq), _ptr(dk), _ptr(dv),
-                  _ptr(workspace), workspace.numel() * workspace.element_size(), B, H, D, n, sides, int(window),
-                  float(softmax_scale), _stream(stream)), "hmar_attn_bwd_window")
-        return dq, dk, dv
-    fn = lib().hmar_attn_bwd_f32 if _is_f32(q) else lib().hmar_attn_bwd
-    _check(fn(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), _ptr(dout), _ptr(dq), _ptr(dk), _ptr(dv),
-              _ptr(workspace), workspace.numel() * workspace.element_size(), B, H, D, n, sides,
-              float(softmax_scale), _stream(stream)), "hmar_attn_bwd")
-    return dq, dk, dv
+    return _done(_host().bwd(q, k, v, out, lse, dout, side_lens, softmax_scale, dq, dk, dv, workspace, _handle(stream), window), "hmar_attn_bwd")
 
 
 HMAR_NOALLOC_MAX_ROWS = 32768
@@ -252,17 +225,8 @@ def hmar_attn_scale_step(q, k_prev, v_prev, k_cur, v_cur, side_prev, side_cur, s
                          out=None, lse=None, want_lse=True, stream=None):
     """Inference step of one scale. q, k_cur, v_cur: [B,H,side_cur^2,D]; k_prev, v_prev:
     [B,H,side_prev^2,D] or None when side_prev == 0. Returns (out, lse or None)."""
-    _need(q, k_prev, v_prev, k_cur, v_cur, out, lse)
-    B, H, n_cur, D = q.shape
-    if out is None:
-        out = torch.empty_like(q)
-    if lse is None and want_lse:
-        lse = q.new_empty((B, H, n_cur), dtype=torch.float32)
-    fn = lib().hmar_attn_scale_step_f32 if _is_f32(q) else lib().hmar_attn_scale_step
-    _check(fn(_ptr(q), _ptr(k_prev), _ptr(v_prev), _ptr(k_cur), _ptr(v_cur), _ptr(out), _ptr(lse),
-              B, H, D, int(side_prev), int(side_cur), float(softmax_scale), _stream(stream)),
-           "hmar_attn_scale_step")
-    return out, lse
+    return _done(_host().scale_step(q, k_prev, v_prev, k_cur, v_cur, side_prev, side_cur, softmax_scale, out, lse, want_lse,
+                                    _handle(stream)), "hmar_attn_scale_step")
 
 
 def hmar_attn_scale_step_strided(q, k_prev, v_prev, k_cur, v_cur, side_prev, side_cur, softmax_scale,
@@ -270,57 +234,20 @@ def hmar_attn_scale_step_strided(q, k_prev, v_prev, k_cur, v_cur, side_prev, sid
     """Inference step on views whose heads are not packed back to back, e.g. slices of one K/V ring
     [B,H,ring_rows,D] (k_prev = ring[:, :, a:a+n_prev], k_cur = ring[:, :, a+n_prev:a+n_prev+n_cur]).
     Every tensor is a [B,H,rows,D] view with contiguous rows and heads a constant stride apart."""
-    B, H, n_cur, D = q.shape
-
-    def head_stride(t):
-        if t is None:
-            return 0
-        (b, h, rows, _), (sb, sh, sr, sd) = t.shape, t.stride()
-        if not t.is_cuda or sd != 1 or sr != D or (h > 1 and b > 1 and sb != H * sh):
-            raise ValueError("views must have contiguous rows and evenly spaced heads")
-        return sh if h > 1 else (sb if b > 1 else rows * D)
-
-    if _is_f32(q):
-        raise TypeError("hmar_attn_scale_step_strided takes bfloat16 tensors")
-    if out is None:
-        out = q.new_empty((B, H, n_cur, D))
-    if lse is None and want_lse:
-        lse = q.new_empty((B, H, n_cur), dtype=torch.float32)
-    _check(lib().hmar_attn_scale_step_strided(
-        _ptr(q), _ptr(k_prev), _ptr(v_prev), _ptr(k_cur), _ptr(v_cur), _ptr(out), _ptr(lse), B, H, D, int(side_prev),
-        int(side_cur), head_stride(q), head_stride(k_prev), head_stride(k_cur), head_stride(out), float(softmax_scale),
-        _stream(stream)), "hmar_attn_scale_step_strided")
-    return out, lse
+    return _done(_host().scale_step_strided(q, k_prev, v_prev, k_cur, v_cur, side_prev, side_cur, softmax_scale, out, lse, want_lse,
+                                            _handle(stream)), "hmar_attn_scale_step_strided")
 
 
 def hmar_recon_accumulate(xhat, codebook, tokens_new, tokens_old=None, mask=None, tokens_out=None, stream=None):
     """xhat [B,C,S,S] fp32 += bicubic(lookup(codebook [V,C], selected tokens [B,s,s])); returns xhat.
     `mask` (uint8 [B,s,s]) chooses tokens_new over tokens_old per position; `tokens_out` receives the selection."""
-    _need(xhat, codebook, tokens_new, tokens_old, mask, tokens_out)
-    if xhat.dtype != torch.float32 or codebook.dtype != torch.float32 or tokens_new.dtype != torch.int32:
-        raise TypeError("xhat and codebook must be float32, tokens int32")
-    if mask is not None and mask.dtype != torch.uint8:
-        raise TypeError("mask must be uint8")
-    B, C, S, _ = xhat.shape
-    V = codebook.shape[0]
-    side = tokens_new.shape[1]
-    _check(lib().hmar_recon_accumulate(_ptr(xhat), _ptr(codebook), _ptr(tokens_old), _ptr(tokens_new), _ptr(mask),
-                                       _ptr(tokens_out), B, C, V, side, S, _stream(stream)), "hmar_recon_accumulate")
-    return xhat
+    return _done(_host().recon_accumulate(xhat, codebook, tokens_new, tokens_old, mask, tokens_out, _handle(stream)),
+                 "hmar_recon_accumulate")
 
 
 def hmar_recon_downsample(xhat, out_side, out=None, stream=None):
     """Area interpolation of xhat [B,C,S,S] fp32 down to [B,C,out_side,out_side]; returns the result."""
-    _need(xhat, out)
-    if xhat.dtype != torch.float32:
-        raise TypeError("xhat must be float32")
-    B, C, S, _ = xhat.shape
-    if out is None:
-        out = xhat.new_empty((B, C, out_side, out_side))
-    elif out.dtype != torch.float32 or tuple(out.shape) != (B, C, out_side, out_side):
-        raise ValueError("out must be float32 [B, C, out_side, out_side]")
-    _check(lib().hmar_recon_downsample(_ptr(xhat), _ptr(out), B, C, S, int(out_side), _stream(stream)), "hmar_recon_downsample")
-    return out
+    return _done(_host().recon_downsample(xhat, out_side, out, _handle(stream)), "hmar_recon_downsample")
 
 
 def hmar_schedule_tiles(side_lens, direction, window=HMAR_WINDOW_MARKOV):

@@ -1,8 +1,9 @@
-"""In-tree build of libhmar.so (nvcc, sm_100a only)."""
+"""In-tree build of libhmar.so (nvcc, sm_100a only) and of the compiled half of the Python binding (g++, against torch)."""
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
@@ -47,6 +48,36 @@ def build(force=False, verbose=False, checked=False):
         raise RuntimeError("nvcc failed building libhmar.so")
     if verbose:
         sys.stderr.write(res.stdout + res.stderr)
+    if not checked:
+        build_host(force)
+    return target
+
+
+def host_path():
+    """The binding's compiled module; its name holds what it was compiled against."""
+    import torch
+    return os.path.join(PKG_DIR, "_hmar_host-%s-%s.so" % (sysconfig.get_config_var("SOABI"), torch.__version__))
+
+
+def build_host(force=False):
+    """Compile csrc/host_binding.cpp unless it is up to date; returns the module's path."""
+    target = host_path()
+    deps = [os.path.join(CSRC, "host_binding.cpp"), os.path.join(PKG_DIR, "..", "include", "hmar.h")]
+    if not force and os.path.exists(target) and all(os.path.getmtime(d) <= os.path.getmtime(target) for d in deps):
+        return target
+    import torch
+    root = os.path.dirname(os.path.abspath(torch.__file__))
+    cuda = os.path.dirname(os.path.dirname(_nvcc()))
+    partial = "%s.%d" % (target, os.getpid())              # another process may be loading or building the same file
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-Wall", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI]
+    cmd += ["-I" + d for d in (os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+                               sysconfig.get_paths()["include"], os.path.join(cuda, "include"))]
+    cmd += [deps[0], "-L" + os.path.join(root, "lib"), "-ltorch_python", "-lc10_cuda", "-ltorch", "-ltorch_cpu", "-lc10", "-o", partial]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        sys.stderr.write(res.stdout + res.stderr)
+        raise RuntimeError("g++ failed building the binding's compiled module")
+    os.replace(partial, target)
     return target
 
 

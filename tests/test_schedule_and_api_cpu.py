@@ -197,3 +197,17 @@ def test_backward_full_tile_share_picks_the_instantiation():
     assert hmar.hmar_schedule_bwd_full_tile_share((1, 2)) == 0
     with pytest.raises(hmar.HmarError):
         hmar.hmar_schedule_bwd_full_tile_share((1, 0))
+
+
+@pytest.mark.parametrize("call, error", [
+    (lambda t: hmar.hmar_attn_fwd(t, t, t, (2,), 0.125), ValueError),                         # a CPU tensor
+    (lambda t: hmar.hmar_attn_fwd("q", t, t, (2,), 0.125), TypeError),                        # not a tensor
+    (lambda t: hmar.hmar_attn_scale_step(t, None, None, t, t, 0, 2, 0.125), ValueError),
+    (lambda t: hmar.hmar_attn_scale_step_strided(t.float(), None, None, t, t, 0, 2, 0.125), TypeError),
+    (lambda t: hmar.hmar_attn_scale_step_strided(t.double(), None, None, t, t, 0, 2, 0.125), TypeError),
+    (lambda t: hmar.hmar_recon_downsample(t, 1), ValueError),
+])
+def test_binding_raises_python_errors(call, error):
+    import torch
+    with pytest.raises(error):
+        call(torch.zeros(1, 1, 4, 64, dtype=torch.bfloat16))
