@@ -228,7 +228,6 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
 
-    if (args.status != nullptr && *reinterpret_cast<volatile int*>(args.status) != 0) return;
     if ((base & 1023u) != 0) {
         if (threadIdx.x == 0) report_timeout(args.status, 0x3FF);
         return;
@@ -266,6 +265,8 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
         fence_mbar_init();
     }
+    grid_wait();
+    if (args.status != nullptr && *reinterpret_cast<volatile int*>(args.status) != 0) return;
     if (warp == MMA_WARP) {
         tmem_alloc(&sm.tmem_base, TMEM_COLS);
         tmem_relinquish();
@@ -842,11 +843,11 @@ struct RowLayout {
 // clears the fp32 dQ accumulator (32 bytes per lane), which saves a separate pass over it.
 template <bool STRIDED>
 __global__ void __launch_bounds__(256)
-hmar_bwd_delta_kernel(const __nv_bfloat16* __restrict__ out, const __nv_bfloat16* __restrict__ dout,
-                      float* __restrict__ delta, float* __restrict__ dq_acc, size_t n_rows, const RowLayout lay) {
+hmar_bwd_delta_kernel(const __nv_bfloat16* out, const __nv_bfloat16* dout, float* delta, float* dq_acc, size_t n_rows, const RowLayout lay) {
     const size_t row = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
     const int part = threadIdx.x & 7;
     float acc = 0.f;
+    grid_wait();
     if (row < n_rows) {
         float4* z = reinterpret_cast<float4*>(dq_acc + row * D + part * 8);
         z[0] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -872,10 +873,10 @@ hmar_bwd_delta_kernel(const __nv_bfloat16* __restrict__ out, const __nv_bfloat16
 // dq = bf16(scale * dq_acc)
 template <bool STRIDED>
 __global__ void __launch_bounds__(256)
-hmar_bwd_dq_convert_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq, float scale, size_t n8,
-                           const RowLayout lay) {
+hmar_bwd_dq_convert_kernel(const float* acc, __nv_bfloat16* dq, float scale, size_t n8, const RowLayout lay) {
     const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= n8) return;
+    grid_wait();
     const float4 a = reinterpret_cast<const float4*>(acc)[2 * idx];
     const float4 b = reinterpret_cast<const float4*>(acc)[2 * idx + 1];
     uint4 o;
@@ -916,7 +917,9 @@ static cudaError_t launch_bwd_tc_layout(const CUtensorMap& q, const CUtensorMap&
     {
         KernelTimer timer("hmar_bwd_delta_kernel", stream);
         const RowLayout lay{args.L, args.heads_per_batch, args.od_row, args.od_head, args.od_batch};
-        hmar_bwd_delta_kernel<STRIDED><<<(unsigned)((n_rows * 8 + 255) / 256), 256, 0, stream>>>(out, dout, args.delta_w, args.dq_acc, n_rows, lay);
+        const cudaError_t e = launch_overlapped(hmar_bwd_delta_kernel<STRIDED>, (unsigned)((n_rows * 8 + 255) / 256), 256, 0, stream, out, dout,
+                                                args.delta_w, args.dq_acc, n_rows, lay);
+        if (e != cudaSuccess) return e;
     }
     {
         KernelTimer timer("hmar_bwd_tc_kernel", stream);
@@ -932,15 +935,17 @@ static cudaError_t launch_bwd_tc_layout(const CUtensorMap& q, const CUtensorMap&
         static SmemOptIn opt_in[2];
         const bool one_mask = args.plain_permille < kOneMaskBelowPermille;
         auto kernel = one_mask ? hmar_bwd_tc_kernel<STRIDED, true> : hmar_bwd_tc_kernel<STRIDED, false>;
-        const cudaError_t e = opt_in[one_mask]((const void*)kernel, smem);
+        cudaError_t e = opt_in[one_mask]((const void*)kernel, smem);
+        if (e == cudaSuccess) e = launch_overlapped(kernel, grid, NUM_THREADS, smem, stream, q, k, v, dout_map, dq_acc_map, a);
         if (e != cudaSuccess) return e;
-        kernel<<<grid, NUM_THREADS, smem, stream>>>(q, k, v, dout_map, dq_acc_map, a);
     }
     const size_t n8 = n_rows * D / 8;
     {
         KernelTimer timer("hmar_bwd_dq_convert_kernel", stream);
         const RowLayout lay{args.L, args.heads_per_batch, args.g_row, args.g_head, args.g_batch};
-        hmar_bwd_dq_convert_kernel<STRIDED><<<(unsigned)((n8 + 255) / 256), 256, 0, stream>>>(args.dq_acc, dq, args.softmax_scale, n8, lay);
+        const cudaError_t e = launch_overlapped(hmar_bwd_dq_convert_kernel<STRIDED>, (unsigned)((n8 + 255) / 256), 256, 0, stream, args.dq_acc, dq,
+                                                args.softmax_scale, n8, lay);
+        if (e != cudaSuccess) return e;
     }
     count_launch(3);
     return cudaGetLastError();

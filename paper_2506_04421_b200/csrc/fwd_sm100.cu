@@ -124,9 +124,6 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         if (threadIdx.x == 0) report_timeout(args.status, 0x3FF);
         return;
     }
-    // whether a block of this launch (or an earlier one) already gave up on a wait: asked for now, looked at after the set-up
-    const int given_up = threadIdx.x == 0 && args.status != nullptr ? *reinterpret_cast<volatile int*>(args.status) : 0;
-
     // ---- which tile of which head
     int bh, wi;
     if (args.work != nullptr) {
@@ -155,6 +152,7 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     const int n_tiles = tiles0 + tiles1;
 
     // ---- set-up
+    int given_up = 0;
     if (threadIdx.x == 0) {
         sm.gave_up = 0;
         mbar_init(&sm.q_full, 1);
@@ -168,6 +166,9 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         mbar_init(&sm.p_full, NUM_SOFTMAX_THREADS);
         mbar_init(&sm.o_done, 1);
         fence_mbar_init();
+        grid_wait();
+        // whether a block of this launch (or an earlier one) already gave up on a wait: asked for now, looked at after the set-up
+        if (args.status != nullptr) given_up = *reinterpret_cast<volatile int*>(args.status);
         // The block's first copies (Q, first K and V tiles) start here, before the TMEM allocation and the
         // block-wide barrier, so that their latency overlaps the rest of the set-up.
         const KvTile t0 = kv_tile(w, tiles0, 0);
@@ -179,6 +180,7 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         tma_load_4d(sm.v[0], t0.seg ? &map_v1 : &map_v0, &sm.v_full[0], 0, t0.coord, head, batch);
     }
     if (warp == MMA_WARP) {
+        grid_wait();
         tmem_alloc(&sm.tmem_base, TMEM_COLS);
         tmem_relinquish();
     }
@@ -537,7 +539,8 @@ cudaError_t launch_fwd_tc(const CUtensorMap& q, const CUtensorMap& k0, const CUt
     a.group_heads = (int)((BH + groups - 1) / groups);
     {
         KernelTimer timer(args.work != nullptr ? "hmar_fwd_tc_kernel" : "hmar_fwd_tc_kernel/scale_step", stream);
-        hmar_fwd_tc_kernel<<<grid, NUM_THREADS, smem, stream>>>(q, k0, v0, k1, v1, a);
+        const cudaError_t launched = launch_overlapped(hmar_fwd_tc_kernel, grid, NUM_THREADS, smem, stream, q, k0, v0, k1, v1, a);
+        if (launched != cudaSuccess) return launched;
     }
     count_launch(1);
     return cudaGetLastError();

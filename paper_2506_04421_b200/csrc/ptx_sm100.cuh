@@ -327,6 +327,11 @@ __device__ __forceinline__ void tmem_st_wait() {
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
+// Returns when the previous kernel of the stream has ended and its stores can be seen (see launch_overlapped).  Pointers read
+// after it are not `const __restrict__`: a read through such a pointer counts as one of constant data, which a compiler may
+// move up across this.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ float ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
