@@ -19,13 +19,14 @@
 //   warps 8-11  per step: drain dQ_i from TMEM through a staging buffer into the fp32 accumulator with
 //               bulk tensor reductions (cp.reduce.async.bulk.tensor).  Per item: copy the next item's K
 //               and V rows into TMEM as soon as the current item's last scores are done, and write the
-//               finished dK, dV (scaled, bf16)
+//               finished dK, dV (scaled, bf16), V, dK and dV as whole rows per instruction
 //   warp 12     TMA producer: K per item (two buffers); Q_i, dO_i through a 3-stage ring
 //   warp 13     issues tcgen05.mma.  K and V in TMEM are the A operands of S^T = K Q_i^T and
 //               dP^T = V dO_i^T; dV += P^T dO_i and dK += dS^T Q_i read their A operand from TMEM too;
 //               dQ_i = dS K reads dS from shared memory as an MN-major operand
 //   warp 14     loads -lse_i * log2(e) and -delta_i with plain loads (their row offsets are not 16-byte
 //               aligned) into an 8-deep ring
+//   warp 15     works out the block's items and hands them to the other warps through an 8-slot ring
 // TMEM columns: S^T [0,128) (half h at h*64; P^T of half h over its first 32 columns), dP^T [128,256)
 // (dS^T likewise), dK [256,320), dV [320,384), dQ_i [384,448), K [448,480), V [480,512).
 // dK and dV stay in TMEM for a whole item and are written once at its end.
