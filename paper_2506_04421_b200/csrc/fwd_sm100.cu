@@ -326,156 +326,159 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 __syncwarp();
             }
         }
-    } else if (warp * 32 >= w.row_count) {
-        // ================================================================== softmax warp past the tile's last row
-        // It only answers: its rows of P hold whatever S left there and reach its rows of O alone.  A scale of 324 tokens
-        // has one such warp in twelve, one of 169 two in eight.
-        reg_inc<REGS_SOFTMAX>();
-#pragma unroll 1
-        for (int j = 0; j < n_tiles; ++j) {
-            if (!wait(AT(s_full), j & 1)) break;
-            bar_arrive(AT(p_full));
-        }
     } else {
-        // ================================================================== softmax warps + epilogue
+        // The registers move for a whole warpgroup: all of its threads execute this one instruction, and what tells its
+        // warps apart comes after it.
         reg_inc<REGS_SOFTMAX>();
-        const int r = warp * 32 + lane;                        // row inside the tile
-        const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
-        const int row = w.row_begin + r;
-        const bool row_ok = r < w.row_count;
-        int lo = w.s0_begin, hi = w.s0_end;                    // per-row key bounds (training, packed tiles)
-        if (!w.uniform && row_ok) {
-            const int s = scale_of_row(args.st, row);
-            lo = args.st.start[first_key_scale(args.st.window, s)];
-            hi = args.st.start[last_key_scale(args.st.window, s) + 1];
-        }
-        const float sl2 = args.scale_log2;
-        const uint32_t s_addr = lane_base + COL_S;
-        const uint32_t o_addr = lane_base + COL_O;
-        float m_used = -INFINITY, l = 0.f;
-        bool ok = true;
-        uint32_t b0[32], b1[32];
-
-        for (int j = 0; j < n_tiles && ok; ++j) {
-            const KvTile t = kv_tile(w, tiles0, j);
-            const int n = tile_cols(t.n_valid);
-            // key c of the tile is visible to this row iff c in [c_lo, c_hi)
-            const int c_lo = w.uniform ? 0 : max(lo - t.coord, 0);
-            const int c_hi = w.uniform ? t.n_valid : min(hi - t.coord, t.n_valid);
-            const bool two = n > 32;                           // second 32-column chunk present
-            const bool need_mask = (!w.uniform) || (t.n_valid < (two ? 64 : 32));
-
-            ok = wait(AT(s_full), j & 1);
-            if (!ok) break;
-            tc_fence_after();
-
-            tmem_ld32(s_addr, b0);
-            if (two) tmem_ld32(s_addr + 32, b1);
-            tmem_ld_wait();
-
-            // masked logits become -inf once, so the maximum and the exponentials treat them alike (columns the
-            // tensor core did not write hold stale values and lie outside [c_lo, c_hi) too)
-            if (need_mask) {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    if (!(i >= c_lo && i < c_hi)) b0[i] = 0xff800000u;
-                    if (!(32 + i >= c_lo && 32 + i < c_hi)) b1[i] = 0xff800000u;
-                }
-            }
-            float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};     // four chains of maxima, not one of 64
-#pragma unroll
-            for (int i = 0; i < 32; ++i) mx4[i & 3] = fmaxf(mx4[i & 3], __uint_as_float(b0[i]));
-            if (two) {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) mx4[i & 3] = fmaxf(mx4[i & 3], __uint_as_float(b1[i]));
-            }
-            const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * sl2;     // softmax_scale > 0
-
-            // Keep the running maximum unless this tile exceeds it by more than the threshold.  O is quiet
-            // here: the product that precedes S of this tile in the tensor core's queue is the last one that
-            // wrote it, and the next one waits for these warps.
-            const bool grow = mx > m_used + kRescaleThreshold;  // false for -inf > -inf
-            if (__any_sync(0xffffffffu, grow)) {
-                const float m_new = fmaxf(m_used, mx);
-                const float f = (m_used == -INFINITY) ? 0.f : ex2(m_used - m_new);
-                m_used = m_new;
-                l *= f;
-                if (j > 0) {
+        if (warp * 32 >= w.row_count) {
+            // ============================================================== softmax warp past the tile's last row
+            // It only answers: its rows of P hold whatever S left there and reach its rows of O alone.  A scale of 324
+            // tokens has one such warp in twelve, one of 169 two in eight.
 #pragma unroll 1
-                    for (int piece = 0; piece < 4; ++piece) {
-                        uint32_t o[16];
-                        tmem_ld16(o_addr + piece * 16, o);
-                        tmem_ld_wait();
+            for (int j = 0; j < n_tiles; ++j) {
+                if (!wait(AT(s_full), j & 1)) break;
+                bar_arrive(AT(p_full));
+            }
+        } else {
+            // ============================================================== softmax warps + epilogue
+            const int r = warp * 32 + lane;                        // row inside the tile
+            const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
+            const int row = w.row_begin + r;
+            const bool row_ok = r < w.row_count;
+            int lo = w.s0_begin, hi = w.s0_end;                    // per-row key bounds (training, packed tiles)
+            if (!w.uniform && row_ok) {
+                const int s = scale_of_row(args.st, row);
+                lo = args.st.start[first_key_scale(args.st.window, s)];
+                hi = args.st.start[last_key_scale(args.st.window, s) + 1];
+            }
+            const float sl2 = args.scale_log2;
+            const uint32_t s_addr = lane_base + COL_S;
+            const uint32_t o_addr = lane_base + COL_O;
+            float m_used = -INFINITY, l = 0.f;
+            bool ok = true;
+            uint32_t b0[32], b1[32];
+
+            for (int j = 0; j < n_tiles && ok; ++j) {
+                const KvTile t = kv_tile(w, tiles0, j);
+                const int n = tile_cols(t.n_valid);
+                // key c of the tile is visible to this row iff c in [c_lo, c_hi)
+                const int c_lo = w.uniform ? 0 : max(lo - t.coord, 0);
+                const int c_hi = w.uniform ? t.n_valid : min(hi - t.coord, t.n_valid);
+                const bool two = n > 32;                           // second 32-column chunk present
+                const bool need_mask = (!w.uniform) || (t.n_valid < (two ? 64 : 32));
+
+                ok = wait(AT(s_full), j & 1);
+                if (!ok) break;
+                tc_fence_after();
+
+                tmem_ld32(s_addr, b0);
+                if (two) tmem_ld32(s_addr + 32, b1);
+                tmem_ld_wait();
+
+                // masked logits become -inf once, so the maximum and the exponentials treat them alike (columns the
+                // tensor core did not write hold stale values and lie outside [c_lo, c_hi) too)
+                if (need_mask) {
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
-                        tmem_st16(o_addr + piece * 16, o);
+                    for (int i = 0; i < 32; ++i) {
+                        if (!(i >= c_lo && i < c_hi)) b0[i] = 0xff800000u;
+                        if (!(32 + i >= c_lo && 32 + i < c_hi)) b1[i] = 0xff800000u;
                     }
                 }
-            }
-            const float m_sub = (m_used == -INFINITY) ? 0.f : m_used;
-
-            // P = 2^(s * scale - m): fp32 row sum, bf16 P written over the S columns already read
-            uint32_t packed[16];
-            float l_add = 0.f;
+                float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};     // four chains of maxima, not one of 64
 #pragma unroll
-            for (int i = 0; i < 32; i += 2) {
-                const float p0 = ex2(fmaf(__uint_as_float(b0[i]), sl2, -m_sub));
-                const float p1 = ex2(fmaf(__uint_as_float(b0[i + 1]), sl2, -m_sub));
-                l_add += p0 + p1;
-                packed[i / 2] = pack_bf16(p0, p1);
-            }
-            tmem_st16(s_addr, packed);
-            if (two) {
+                for (int i = 0; i < 32; ++i) mx4[i & 3] = fmaxf(mx4[i & 3], __uint_as_float(b0[i]));
+                if (two) {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) mx4[i & 3] = fmaxf(mx4[i & 3], __uint_as_float(b1[i]));
+                }
+                const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * sl2;     // softmax_scale > 0
+
+                // Keep the running maximum unless this tile exceeds it by more than the threshold.  O is quiet
+                // here: the product that precedes S of this tile in the tensor core's queue is the last one that
+                // wrote it, and the next one waits for these warps.
+                const bool grow = mx > m_used + kRescaleThreshold;  // false for -inf > -inf
+                if (__any_sync(0xffffffffu, grow)) {
+                    const float m_new = fmaxf(m_used, mx);
+                    const float f = (m_used == -INFINITY) ? 0.f : ex2(m_used - m_new);
+                    m_used = m_new;
+                    l *= f;
+                    if (j > 0) {
+#pragma unroll 1
+                        for (int piece = 0; piece < 4; ++piece) {
+                            uint32_t o[16];
+                            tmem_ld16(o_addr + piece * 16, o);
+                            tmem_ld_wait();
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
+                            tmem_st16(o_addr + piece * 16, o);
+                        }
+                    }
+                }
+                const float m_sub = (m_used == -INFINITY) ? 0.f : m_used;
+
+                // P = 2^(s * scale - m): fp32 row sum, bf16 P written over the S columns already read
+                uint32_t packed[16];
+                float l_add = 0.f;
 #pragma unroll
                 for (int i = 0; i < 32; i += 2) {
-                    const float p0 = ex2(fmaf(__uint_as_float(b1[i]), sl2, -m_sub));
-                    const float p1 = ex2(fmaf(__uint_as_float(b1[i + 1]), sl2, -m_sub));
+                    const float p0 = ex2(fmaf(__uint_as_float(b0[i]), sl2, -m_sub));
+                    const float p1 = ex2(fmaf(__uint_as_float(b0[i + 1]), sl2, -m_sub));
                     l_add += p0 + p1;
                     packed[i / 2] = pack_bf16(p0, p1);
                 }
-                tmem_st16(s_addr + 16, packed);
+                tmem_st16(s_addr, packed);
+                if (two) {
+#pragma unroll
+                    for (int i = 0; i < 32; i += 2) {
+                        const float p0 = ex2(fmaf(__uint_as_float(b1[i]), sl2, -m_sub));
+                        const float p1 = ex2(fmaf(__uint_as_float(b1[i + 1]), sl2, -m_sub));
+                        l_add += p0 + p1;
+                        packed[i / 2] = pack_bf16(p0, p1);
+                    }
+                    tmem_st16(s_addr + 16, packed);
+                }
+                l += l_add;
+                tmem_st_wait();
+                tc_fence_before();
+                bar_arrive(AT(p_full));
             }
-            l += l_add;
-            tmem_st_wait();
-            tc_fence_before();
-            bar_arrive(AT(p_full));
-        }
 
-        // ---- epilogue: out = O / l, lse = ln(l) + m (natural log of the scaled logits' sum)
-        if (ok) ok = wait(AT(o_done), 0);
-        if (ok) {
-            tc_fence_after();
-            const float inv = 1.f / l;
-            tmem_ld32(o_addr, b0);
-            tmem_ld32(o_addr + 32, b1);
-            tmem_ld_wait();
-            const long long lse_off = (long long)bh * args.n_q_rows + row;
-            if (row_ok && args.lse != nullptr && HMAR_IN_BOUNDS(lse_off >= 0 && lse_off < args.lse_extent, args.status, 0xB102))
-                args.lse[lse_off] = (m_used + log2f(l)) * 0.6931471805599453f;
-            // The warp's 32 rows go through the shared memory of its own query rows (read for the last time by the products
-            // that o_done covers), 16-byte pieces swizzled by the row, so that a store instruction covers four whole rows and
-            // not a piece of each of 32 (L1 takes a line at a time: 256 lines a warp, now 32).
-            uint8_t* stage = sm.q + warp * 4096;
+            // ---- epilogue: out = O / l, lse = ln(l) + m (natural log of the scaled logits' sum)
+            if (ok) ok = wait(AT(o_done), 0);
+            if (ok) {
+                tc_fence_after();
+                const float inv = 1.f / l;
+                tmem_ld32(o_addr, b0);
+                tmem_ld32(o_addr + 32, b1);
+                tmem_ld_wait();
+                const long long lse_off = (long long)bh * args.n_q_rows + row;
+                if (row_ok && args.lse != nullptr && HMAR_IN_BOUNDS(lse_off >= 0 && lse_off < args.lse_extent, args.status, 0xB102))
+                    args.lse[lse_off] = (m_used + log2f(l)) * 0.6931471805599453f;
+                // The warp's 32 rows go through the shared memory of its own query rows (read for the last time by the products
+                // that o_done covers), 16-byte pieces swizzled by the row, so that a store instruction covers four whole rows and
+                // not a piece of each of 32 (L1 takes a line at a time: 256 lines a warp, now 32).
+                uint8_t* stage = sm.q + warp * 4096;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const uint32_t* src = i < 4 ? b0 + 8 * i : b1 + 8 * (i - 4);
-                uint4 v4;
-                v4.x = pack_bf16(__uint_as_float(src[0]) * inv, __uint_as_float(src[1]) * inv);
-                v4.y = pack_bf16(__uint_as_float(src[2]) * inv, __uint_as_float(src[3]) * inv);
-                v4.z = pack_bf16(__uint_as_float(src[4]) * inv, __uint_as_float(src[5]) * inv);
-                v4.w = pack_bf16(__uint_as_float(src[6]) * inv, __uint_as_float(src[7]) * inv);
-                *reinterpret_cast<uint4*>(stage + lane * 128 + ((i ^ (lane & 7)) << 4)) = v4;
-            }
-            __syncwarp();
-            const int first = w.row_begin + warp * 32, piece = lane & 7;
-            const long long out_off = batch * args.out_batch_stride + head * args.out_head_stride + piece * 8;
+                for (int i = 0; i < 8; ++i) {
+                    const uint32_t* src = i < 4 ? b0 + 8 * i : b1 + 8 * (i - 4);
+                    uint4 v4;
+                    v4.x = pack_bf16(__uint_as_float(src[0]) * inv, __uint_as_float(src[1]) * inv);
+                    v4.y = pack_bf16(__uint_as_float(src[2]) * inv, __uint_as_float(src[3]) * inv);
+                    v4.z = pack_bf16(__uint_as_float(src[4]) * inv, __uint_as_float(src[5]) * inv);
+                    v4.w = pack_bf16(__uint_as_float(src[6]) * inv, __uint_as_float(src[7]) * inv);
+                    *reinterpret_cast<uint4*>(stage + lane * 128 + ((i ^ (lane & 7)) << 4)) = v4;
+                }
+                __syncwarp();
+                const int first = w.row_begin + warp * 32, piece = lane & 7;
+                const long long out_off = batch * args.out_batch_stride + head * args.out_head_stride + piece * 8;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int rr = i * 4 + (lane >> 3);
-                const uint4 v4 = *reinterpret_cast<const uint4*>(stage + rr * 128 + ((piece ^ (rr & 7)) << 4));
-                const long long off = out_off + (first + rr) * args.out_row_stride;
-                if (warp * 32 + rr < w.row_count && HMAR_IN_BOUNDS(off >= 0 && off + 8 <= args.out_extent, args.status, 0xB101))
-                    *reinterpret_cast<uint4*>(args.out + off) = v4;
+                for (int i = 0; i < 8; ++i) {
+                    const int rr = i * 4 + (lane >> 3);
+                    const uint4 v4 = *reinterpret_cast<const uint4*>(stage + rr * 128 + ((piece ^ (rr & 7)) << 4));
+                    const long long off = out_off + (first + rr) * args.out_row_stride;
+                    if (warp * 32 + rr < w.row_count && HMAR_IN_BOUNDS(off >= 0 && off + 8 <= args.out_extent, args.status, 0xB101))
+                        *reinterpret_cast<uint4*>(args.out + off) = v4;
+                }
             }
         }
     }

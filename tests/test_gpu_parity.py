@@ -690,6 +690,25 @@ def test_recon_accumulate_codebook_off_16_byte_alignment():
     assert err.max() <= 1e-5 * max(1.0, np.abs(ref).max()), f"max abs err {err.max():.3e}"
 
 
+@pytest.mark.parametrize("side", [12, 13, 14, 15, 16, 17])
+def test_last_query_tiles_with_one_to_four_softmax_warps(side):
+    """The last query tile of side^2 rows has 16, 41, 68, 97, 128 or 33 of them, so one to four of the block's softmax
+    warps have rows and the others only answer the barriers; the registers move for all four alike.  The inference
+    step (a window of more than 128 keys, which the tcgen05 kernel takes) and the training forward, parity as above."""
+    _run_training(_Wl((side,)), torch.bfloat16, backward=False)
+    wl = _Wl((11, side), B=3, H=5)
+    q, kp, vp, kc, vc = scale_step_inputs(wl, 1, 0, bf16=True)
+    guards = []
+    out = _guarded((wl.B, wl.H, side * side, wl.D), torch.bfloat16, guards)
+    dev = [to_device(x, wl.B, wl.H, torch.bfloat16) for x in (q, kp, vp, kc, vc)]
+    _, lse = hmar.hmar_attn_scale_step(*dev, 11, side, wl.softmax_scale, out=out)
+    ref_out, ref_lse = orc.scale_step(q, kp, vp, kc, vc, wl.softmax_scale)
+    _assert_close("out", out, ref_out, False)
+    _assert_lse(lse, ref_lse, False)
+    assert all(intact() for intact in guards)
+    _no_device_error()
+
+
 def test_edge_cases_through_the_checking_build():
     """The library compiled with -DHMAR_BOUNDS_CHECK compares every address its kernels form by their own
     arithmetic (plain loads and stores; TMA copies are clipped by the hardware) with the extent of its tensor and
