@@ -267,6 +267,9 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         fence_mbar_init();
     }
     grid_wait();
+    // From here on memory is read with plain loads: delta was written by the kernel before, lse, V and (where the call
+    // allocates nothing) the work list by earlier ones, so none of it is read-only for the lifetime of this launch, which
+    // a non-coherent load would ask for.
     if (args.status != nullptr && *reinterpret_cast<volatile int*>(args.status) != 0) return;
     if (warp == MMA_WARP) {
         tmem_alloc(&sm.tmem_base, TMEM_COLS);
@@ -309,11 +312,11 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 Item it;
                 it.steps_uniform = 0;
                 if (pos < total) {
-                    int t = 0, count = args.by_head ? args.n_work : __ldg(&args.work[0].class_count);
+                    int t = 0, count = args.by_head ? args.n_work : args.work[0].class_count;
                     while (pos >= args.n_heads * count) {
                         pos -= args.n_heads * count;
                         t += count;
-                        count = __ldg(&args.work[t].class_count);
+                        count = args.work[t].class_count;
                     }
                     it.bh = pos / count;
                     const BwdWork w = args.work[t + pos - it.bh * count];
@@ -411,8 +414,8 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         const int row = q0 + t * 32 + lane;
                         const bool in = row < w.q_end &&
                                         HMAR_IN_BOUNDS(row >= 0 && row < L && bh >= 0 && bh < args.n_heads, args.status, 0xB201);
-                        lv[t] = in ? __ldg(args.lse + (size_t)bh * L + row) : INFINITY;
-                        dv[t] = in ? __ldg(args.delta + (size_t)bh * L + row) : 0.f;
+                        lv[t] = in ? args.lse[(size_t)bh * L + row] : INFINITY;
+                        dv[t] = in ? args.delta[(size_t)bh * L + row] : 0.f;
                     }
 #pragma unroll
                     for (int t = 0; t < BQ / 32; ++t) {
@@ -603,7 +606,7 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             for (int c = 0; c < 8; ++c) {
                 const __nv_bfloat16* src = vsrc + c * step + piece * 8;
                 const bool v_in = row0 + 4 * c < L && HMAR_IN_BOUNDS(src >= args.v && src - args.v + 8 <= args.in_extent, args.status, 0xB202);
-                rows[c] = v_in ? __ldg(reinterpret_cast<const uint4*>(src)) : make_uint4(0u, 0u, 0u, 0u);
+                rows[c] = v_in ? *reinterpret_cast<const uint4*>(src) : make_uint4(0u, 0u, 0u, 0u);
             }
             if (lane == 0) bulk_wait_read_all();                // the last piece of dQ has been read out of the staging buffer
             __syncwarp();

@@ -709,6 +709,46 @@ def test_last_query_tiles_with_one_to_four_softmax_warps(side):
     _no_device_error()
 
 
+@pytest.mark.parametrize("noalloc", [False, True])
+def test_overlapped_launches_see_what_the_calls_before_wrote(noalloc):
+    """Calls in a row on the same buffers, none waited for: each launch starts while the one before it ends, and has to
+    read the inputs, lse, delta and (noalloc) the work list that were written since its buffers were last read.  Short
+    launches of two side lists with new inputs each time; the results are those of the same calls waited for one by
+    one: out, lse, dK, dV bit for bit, dQ (summed by reductions in any order) to the bf16 tolerance."""
+    lists, sets, B, H, D = [(1, 2, 3, 4, 6, 9), (3, 12, 5)], 3, 1, 3, 64
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    data = {s: [torch.randn((4, B, H, sum(x * x for x in s), D), generator=gen, device="cuda").to(torch.bfloat16) for _ in range(sets)] for s in lists}
+    buf = {s: {n: torch.empty_like(data[s][0][0]) for n in ("q", "k", "v", "do", "out", "dq", "dk", "dv")} for s in lists}
+    lse = {s: torch.empty(data[s][0].shape[1:4], dtype=torch.float32, device="cuda") for s in lists}
+    size = max(hmar.hmar_attn_bwd_workspace_bytes(B, H, D, s) for s in lists)
+    workspace = torch.empty(size, dtype=torch.uint8, device="cuda")
+
+    def call(s, i, wait):
+        b, done = buf[s], []
+        for n, t in zip(("q", "k", "v", "do"), data[s][i]):
+            b[n].copy_(t)
+        ready = torch.cuda.synchronize if wait else (lambda: None)
+        ready()
+        hmar.hmar_attn_fwd(b["q"], b["k"], b["v"], s, 0.125, out=b["out"], lse=lse[s])
+        ready()
+        if noalloc:
+            hmar.hmar_attn_bwd_noalloc(b["q"], b["k"], b["v"], b["out"], lse[s], b["do"], s, 0.125, b["dq"], b["dk"], b["dv"])
+        else:
+            hmar.hmar_attn_bwd(b["q"], b["k"], b["v"], b["out"], lse[s], b["do"], s, 0.125, b["dq"], b["dk"], b["dv"], workspace)
+        ready()
+        return [x.clone() for x in (b["out"], lse[s], b["dk"], b["dv"], b["dq"])]
+
+    order = [(s, i) for i in range(sets) for s in lists]
+    alone = {key: call(*key, True) for key in order}
+    together = [(key, call(*key, False)) for _ in range(20) for key in order]
+    torch.cuda.synchronize()
+    for key, got in together:
+        for g, r in zip(got[:4], alone[key][:4]):
+            assert torch.equal(g, r)
+        assert (got[4].float() - alone[key][4].float()).abs().max().item() <= BF16_MAX
+    _no_device_error()
+
+
 def test_edge_cases_through_the_checking_build():
     """The library compiled with -DHMAR_BOUNDS_CHECK compares every address its kernels form by their own
     arithmetic (plain loads and stores; TMA copies are clipped by the hardware) with the extent of its tensor and
