@@ -73,6 +73,12 @@ float real(PyObject* o) {
     return (float)v;
 }
 
+bool truth(PyObject* o) {
+    const int v = PyObject_IsTrue(o);
+    if (v < 0) throw py::error_already_set();
+    return v != 0;
+}
+
 using Sides = c10::SmallVector<int, HMAR_MAX_SCALES>;
 
 Sides sides_of(PyObject* o) {
@@ -241,7 +247,7 @@ PyObject* scale_step(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const int B = (int)q.size(0), H = (int)q.size(1), D = (int)q.size(3), prev = (int)integer(a[5]), cur = (int)integer(a[6]);
     const at::Tensor out = or_empty(tensor(a[8]), q, q.sizes(), q.scalar_type());
     at::Tensor lse = tensor(a[9]);
-    const bool new_lse = !lse.defined() && PyObject_IsTrue(a[10]) == 1;
+    const bool new_lse = !lse.defined() && truth(a[10]);
     if (new_lse) lse = at::empty(q.sizes().slice(0, 3), q.options().dtype(at::kFloat));
     const float scale = real(a[7]);
     void* stream = stream_of(a[11]);
@@ -272,7 +278,7 @@ PyObject* scale_step_strided(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const int B = (int)q.size(0), H = (int)q.size(1), D = (int)q.size(3), prev = (int)integer(a[5]), cur = (int)integer(a[6]);
     const at::Tensor out = or_empty(tensor(a[8]), q, q.sizes(), q.scalar_type());
     at::Tensor lse = tensor(a[9]);
-    const bool new_lse = !lse.defined() && PyObject_IsTrue(a[10]) == 1;
+    const bool new_lse = !lse.defined() && truth(a[10]);
     if (new_lse) lse = at::empty(q.sizes().slice(0, 3), q.options().dtype(at::kFloat));
     const int status = call(entry.hmar_attn_scale_step_strided, ptr(q), ptr(kp), ptr(vp), ptr(kc), ptr(vc), ptr(out), (float*)ptr(lse), B, H, D, prev, cur, head_stride(q, H), head_stride(kp, H), head_stride(kc, H), head_stride(out, H), real(a[7]), stream_of(a[11]));
     if (status != HMAR_OK) return PyLong_FromLong(status);

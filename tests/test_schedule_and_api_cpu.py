@@ -211,3 +211,15 @@ def test_binding_raises_python_errors(call, error):
     import torch
     with pytest.raises(error):
         call(torch.zeros(1, 1, 4, 64, dtype=torch.bfloat16))
+
+
+def test_binding_passes_on_an_error_of_the_truth_test():
+    """An object whose truth cannot be told (an array, say) in the place of want_lse: its error comes out, nothing is called."""
+    import torch
+
+    class Undecided:
+        def __bool__(self):
+            raise ZeroDivisionError
+    t = torch.zeros(1, 1, 4, 64, dtype=torch.bfloat16)
+    with pytest.raises(ZeroDivisionError):
+        hmar.hmar_attn_scale_step_strided(t, None, None, t, t, 0, 2, 0.125, want_lse=Undecided())
