@@ -122,7 +122,9 @@ PyObject* results(T... o) {
     return tuple;
 }
 
-// The entry points run without the interpreter's lock: a launch waits where the queue of launches is full.
+// The entry points run without the interpreter's lock: a launch waits where the queue of launches is full.  What is checked,
+// converted or asked for is so in statements before the call, in the order of the checks: the order in which a call's
+// arguments are evaluated is the compiler's.
 template <typename F, typename... A>
 int call(F f, A... a) {
     py::gil_scoped_release no_lock;
@@ -211,7 +213,9 @@ PyObject* fwd_packed(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const at::Tensor out = or_empty(tensor(a[1]), qkv, {B, L, H, D}, qkv.scalar_type());
     const at::Tensor lse = or_empty(tensor(a[2]), qkv, {B, H, L}, at::kFloat);
     const Sides sides = sides_of(a[3]);
-    const int status = call(entry.hmar_attn_fwd_packed, ptr(qkv), ptr(out), (float*)ptr(lse), (int)B, (int)H, (int)D, (int)sides.size(), sides.data(), real(a[4]), stream_of(a[5]));
+    const float scale = real(a[4]);
+    void* stream = stream_of(a[5]);
+    const int status = call(entry.hmar_attn_fwd_packed, ptr(qkv), ptr(out), (float*)ptr(lse), (int)B, (int)H, (int)D, (int)sides.size(), sides.data(), scale, stream);
     if (status != HMAR_OK) return PyLong_FromLong(status);
     return results(wrap(a[1], out), wrap(a[2], lse));
     END_HANDLE_TH_ERRORS
@@ -230,7 +234,9 @@ PyObject* bwd_packed(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const Sides sides = sides_of(a[4]);
     at::Tensor ws = tensor(a[7]);
     if (!ws.defined()) ws = at::empty({(int64_t)entry.hmar_attn_bwd_workspace_bytes(B, H, D, (int)sides.size(), sides.data())}, qkv.options().dtype(at::kByte));
-    const int status = call(entry.hmar_attn_bwd_packed, ptr(qkv), ptr(out), (const float*)ptr(lse), ptr(dout), ptr(dqkv), ptr(ws), ws.nbytes(), B, H, D, (int)sides.size(), sides.data(), real(a[5]), stream_of(a[8]));
+    const float scale = real(a[5]);
+    void* stream = stream_of(a[8]);
+    const int status = call(entry.hmar_attn_bwd_packed, ptr(qkv), ptr(out), (const float*)ptr(lse), ptr(dout), ptr(dqkv), ptr(ws), ws.nbytes(), B, H, D, (int)sides.size(), sides.data(), scale, stream);
     if (status != HMAR_OK) return PyLong_FromLong(status);
     return wrap(a[6], dqkv);
     END_HANDLE_TH_ERRORS
@@ -280,7 +286,10 @@ PyObject* scale_step_strided(PyObject*, PyObject* const* a, Py_ssize_t n) {
     at::Tensor lse = tensor(a[9]);
     const bool new_lse = !lse.defined() && truth(a[10]);
     if (new_lse) lse = at::empty(q.sizes().slice(0, 3), q.options().dtype(at::kFloat));
-    const int status = call(entry.hmar_attn_scale_step_strided, ptr(q), ptr(kp), ptr(vp), ptr(kc), ptr(vc), ptr(out), (float*)ptr(lse), B, H, D, prev, cur, head_stride(q, H), head_stride(kp, H), head_stride(kc, H), head_stride(out, H), real(a[7]), stream_of(a[11]));
+    const long long q_stride = head_stride(q, H), prev_stride = head_stride(kp, H), cur_stride = head_stride(kc, H), out_stride = head_stride(out, H);
+    const float scale = real(a[7]);
+    void* stream = stream_of(a[11]);
+    const int status = call(entry.hmar_attn_scale_step_strided, ptr(q), ptr(kp), ptr(vp), ptr(kc), ptr(vc), ptr(out), (float*)ptr(lse), B, H, D, prev, cur, q_stride, prev_stride, cur_stride, out_stride, scale, stream);
     if (status != HMAR_OK) return PyLong_FromLong(status);
     return results(wrap(a[8], out), new_lse ? THPVariable_Wrap(lse) : Py_NewRef(a[9]));
     END_HANDLE_TH_ERRORS

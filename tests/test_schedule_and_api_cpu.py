@@ -223,3 +223,11 @@ def test_binding_passes_on_an_error_of_the_truth_test():
     t = torch.zeros(1, 1, 4, 64, dtype=torch.bfloat16)
     with pytest.raises(ZeroDivisionError):
         hmar.hmar_attn_scale_step_strided(t, None, None, t, t, 0, 2, 0.125, want_lse=Undecided())
+
+
+def test_strided_step_checks_its_views_before_it_asks_for_a_stream():
+    """Views in host memory are a ValueError, also on a machine whose stream cannot be asked for."""
+    import torch
+    t = torch.zeros(1, 1, 4, 64, dtype=torch.bfloat16)
+    with pytest.raises(ValueError):
+        hmar.hmar_attn_scale_step_strided(t, None, None, t, t, 0, 2, 0.125)
