@@ -146,10 +146,10 @@ def _handle(stream):
     return None if stream is None else stream.cuda_stream
 
 
-def _done(result, where):
+def _done(result, where, window=HMAR_WINDOW_MARKOV):
     """What a function of the compiled module returned: its results, or the library's status."""
     if result.__class__ is int:
-        raise HmarError(result, where)
+        raise HmarError(result, where if window == HMAR_WINDOW_MARKOV else where + "_window")
     return result
 
 
@@ -175,7 +175,7 @@ def _need(*tensors):
 def hmar_attn_fwd(q, k, v, side_lens, softmax_scale, out=None, lse=None, stream=None, window=HMAR_WINDOW_MARKOV):
     """Training forward. q, k, v: [B,H,L,D]. Returns (out [B,H,L,D], lse [B,H,L] fp32).
     `window` other than HMAR_WINDOW_MARKOV goes through hmar_attn_fwd_window."""
-    return _done(_host().fwd(q, k, v, out, lse, side_lens, softmax_scale, _handle(stream), window), "hmar_attn_fwd")
+    return _done(_host().fwd(q, k, v, out, lse, side_lens, softmax_scale, _handle(stream), window), "hmar_attn_fwd", window)
 
 
 def hmar_attn_fwd_packed(qkv, side_lens, softmax_scale, out=None, lse=None, stream=None):
@@ -199,7 +199,7 @@ def hmar_attn_bwd(q, k, v, out, lse, dout, side_lens, softmax_scale, dq=None, dk
                   workspace=None, stream=None, window=HMAR_WINDOW_MARKOV):
     """Training backward. Returns (dq, dk, dv), each [B,H,L,D].
     `window` other than HMAR_WINDOW_MARKOV goes through hmar_attn_bwd_window."""
-    return _done(_host().bwd(q, k, v, out, lse, dout, side_lens, softmax_scale, dq, dk, dv, workspace, _handle(stream), window), "hmar_attn_bwd")
+    return _done(_host().bwd(q, k, v, out, lse, dout, side_lens, softmax_scale, dq, dk, dv, workspace, _handle(stream), window), "hmar_attn_bwd", window)
 
 
 HMAR_NOALLOC_MAX_ROWS = 32768

@@ -231,3 +231,15 @@ def test_strided_step_checks_its_views_before_it_asks_for_a_stream():
     t = torch.zeros(1, 1, 4, 64, dtype=torch.bfloat16)
     with pytest.raises(ValueError):
         hmar.hmar_attn_scale_step_strided(t, None, None, t, t, 0, 2, 0.125)
+
+
+@pytest.mark.parametrize("window, suffix", [(hmar.HMAR_WINDOW_MARKOV, ""), (hmar.HMAR_WINDOW_CAUSAL, "_window")])
+def test_errors_name_the_entry_point_that_was_called(window, suffix, monkeypatch):
+    import types
+    from paper_2506_04421_b200 import binding
+    refuses = types.SimpleNamespace(fwd=lambda *a: hmar.HMAR_ERR_BAD_ARG, bwd=lambda *a: hmar.HMAR_ERR_BAD_ARG)
+    monkeypatch.setattr(binding, "_HOST", refuses)
+    with pytest.raises(hmar.HmarError, match="^hmar_attn_fwd%s:" % suffix):
+        hmar.hmar_attn_fwd(None, None, None, (2,), 0.125, window=window)
+    with pytest.raises(hmar.HmarError, match="^hmar_attn_bwd%s:" % suffix):
+        hmar.hmar_attn_bwd(None, None, None, None, None, None, (2,), 0.125, window=window)
