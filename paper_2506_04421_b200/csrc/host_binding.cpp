@@ -209,7 +209,7 @@ PyObject* fwd_packed(PyObject*, PyObject* const* a, Py_ssize_t n) {
     need(qkv, tensor(a[1]), tensor(a[2]));
     need_dims(qkv, 5);
     const int64_t B = qkv.size(0), L = qkv.size(1), H = qkv.size(3), D = qkv.size(4);
-    if (qkv.size(2) != 3) TORCH_CHECK_VALUE(false, "qkv must be [B, L, 3, H, D]");
+    if (qkv.size(2) != 3 || is_f32(qkv)) TORCH_CHECK_VALUE(false, "qkv must be bfloat16 [B, L, 3, H, D]");
     const at::Tensor out = or_empty(tensor(a[1]), qkv, {B, L, H, D}, qkv.scalar_type());
     const at::Tensor lse = or_empty(tensor(a[2]), qkv, {B, H, L}, at::kFloat);
     const Sides sides = sides_of(a[3]);

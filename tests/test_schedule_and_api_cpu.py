@@ -243,3 +243,19 @@ def test_errors_name_the_entry_point_that_was_called(window, suffix, monkeypatch
         hmar.hmar_attn_fwd(None, None, None, (2,), 0.125, window=window)
     with pytest.raises(hmar.HmarError, match="^hmar_attn_bwd%s:" % suffix):
         hmar.hmar_attn_bwd(None, None, None, None, None, None, (2,), 0.125, window=window)
+
+
+def _cuda_tensor_without_memory(*shape, dtype):
+    """A tensor of a CUDA device that no machine needs to have: it passes the checks of kind, and has no address."""
+    import torch
+    from torch._subclasses.fake_tensor import FakeTensorMode
+    with FakeTensorMode(allow_non_fake_inputs=True):
+        return torch.empty(shape, dtype=dtype, device="cuda")
+
+
+@pytest.mark.parametrize("dtype, error", [("float32", ValueError), ("float16", TypeError), ("float64", TypeError)])
+def test_packed_forward_takes_bfloat16_only(dtype, error):
+    import torch
+    qkv = _cuda_tensor_without_memory(1, 4, 3, 1, 64, dtype=getattr(torch, dtype))
+    with pytest.raises(error, match="bfloat16"):
+        hmar.hmar_attn_fwd_packed(qkv, (2,), 0.125)
