@@ -67,6 +67,17 @@ long long integer(PyObject* o) {
     return v;
 }
 
+// An integer, or something equal to one (4.0); other numbers and text are refused.
+long long whole(PyObject* o) {
+    if (PyLong_Check(o)) return integer(o);
+    const py::object number = py::reinterpret_steal<py::object>(PyNumber_Long(o));
+    if (!number) throw py::error_already_set();
+    const int equal = PyObject_RichCompareBool(o, number.ptr(), Py_EQ);
+    if (equal < 0) throw py::error_already_set();
+    if (equal == 0) TORCH_CHECK_VALUE(false, "expected a whole number");
+    return integer(number.ptr());
+}
+
 float real(PyObject* o) {
     const double v = PyFloat_AsDouble(o);
     if (v == -1.0 && PyErr_Occurred()) throw py::error_already_set();
@@ -320,7 +331,7 @@ PyObject* recon_downsample(PyObject*, PyObject* const* a, Py_ssize_t n) {
     need(xhat, tensor(a[2]));
     need_dims(xhat, 4);
     if (xhat.scalar_type() != at::kFloat) TORCH_CHECK_TYPE(false, "xhat must be float32");
-    const int64_t B = xhat.size(0), C = xhat.size(1), side = integer(a[1]);
+    const int64_t B = xhat.size(0), C = xhat.size(1), side = whole(a[1]);
     const at::Tensor out = or_empty(tensor(a[2]), xhat, {B, C, side, side}, at::kFloat);
     if (out.scalar_type() != at::kFloat || out.sizes() != at::IntArrayRef({B, C, side, side})) TORCH_CHECK_VALUE(false, "out must be float32 [B, C, out_side, out_side]");
     const int status = call(entry.hmar_recon_downsample, (const float*)ptr(xhat), (float*)ptr(out), (int)B, (int)C, (int)xhat.size(2), (int)side, stream_of(a[3]));

@@ -259,3 +259,13 @@ def test_packed_forward_takes_bfloat16_only(dtype, error):
     qkv = _cuda_tensor_without_memory(1, 4, 3, 1, 64, dtype=getattr(torch, dtype))
     with pytest.raises(error, match="bfloat16"):
         hmar.hmar_attn_fwd_packed(qkv, (2,), 0.125)
+
+
+@pytest.mark.parametrize("given", [None, (1, 1, 4, 4)])
+@pytest.mark.parametrize("side", [4.5, "4", None])
+def test_downsample_refuses_sides_that_are_not_whole(given, side):
+    import torch
+    x = _cuda_tensor_without_memory(1, 1, 8, 8, dtype=torch.float32)
+    out = given and _cuda_tensor_without_memory(*given, dtype=torch.float32)
+    with pytest.raises((TypeError, ValueError)):
+        hmar.hmar_recon_downsample(x, side, out=out)
