@@ -93,6 +93,7 @@ bool truth(PyObject* o) {
 using Sides = c10::SmallVector<int, HMAR_MAX_SCALES>;
 
 Sides sides_of(PyObject* o) {
+    if (PyObject_Size(o) < 0) throw py::error_already_set();
     const py::object items = py::reinterpret_steal<py::object>(PySequence_Fast(o, "side_lens must be a sequence"));
     if (!items) throw py::error_already_set();
     Sides s;

@@ -269,3 +269,11 @@ def test_downsample_refuses_sides_that_are_not_whole(given, side):
     out = given and _cuda_tensor_without_memory(*given, dtype=torch.float32)
     with pytest.raises((TypeError, ValueError)):
         hmar.hmar_recon_downsample(x, side, out=out)
+
+
+def test_side_lists_have_a_length():
+    """A generator is refused (a call could use it up once); every sized collection of numbers is taken."""
+    import torch
+    q = _cuda_tensor_without_memory(1, 1, 4, 64, dtype=torch.bfloat16)
+    with pytest.raises(TypeError):
+        hmar.hmar_attn_fwd(q, q, q, (s for s in (2,)), 0.125, out=q, lse=q)
