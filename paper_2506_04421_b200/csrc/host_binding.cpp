@@ -79,9 +79,10 @@ long long whole(PyObject* o) {
 }
 
 float real(PyObject* o) {
-    const double v = PyFloat_AsDouble(o);
-    if (v == -1.0 && PyErr_Occurred()) throw py::error_already_set();
-    return (float)v;
+    if (PyFloat_Check(o)) return (float)PyFloat_AS_DOUBLE(o);
+    const py::object number = py::reinterpret_steal<py::object>(PyNumber_Float(o));
+    if (!number) throw py::error_already_set();
+    return (float)PyFloat_AS_DOUBLE(number.ptr());
 }
 
 bool truth(PyObject* o) {

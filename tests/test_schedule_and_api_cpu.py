@@ -277,3 +277,14 @@ def test_side_lists_have_a_length():
     q = _cuda_tensor_without_memory(1, 1, 4, 64, dtype=torch.bfloat16)
     with pytest.raises(TypeError):
         hmar.hmar_attn_fwd(q, q, q, (s for s in (2,)), 0.125, out=q, lse=q)
+
+
+def test_softmax_scale_is_whatever_float_takes():
+    """float("0.125") is a number: the call gets past its arguments, to the tensor that has no address."""
+    import torch
+    q = _cuda_tensor_without_memory(1, 1, 4, 64, dtype=torch.bfloat16)
+    with pytest.raises(Exception) as e:
+        hmar.hmar_attn_fwd(q, q, q, (2,), "0.125", out=q, lse=q)
+    assert not isinstance(e.value, TypeError)
+    with pytest.raises(ValueError):
+        hmar.hmar_attn_fwd(q, q, q, (2,), "an eighth", out=q, lse=q)
