@@ -67,6 +67,14 @@ long long integer(PyObject* o) {
     return v;
 }
 
+// An integer or an integer type (numpy's, a tensor of one); floats are refused.
+long long index(PyObject* o) {
+    if (PyLong_Check(o)) return integer(o);
+    const py::object number = py::reinterpret_steal<py::object>(PyNumber_Index(o));
+    if (!number) throw py::error_already_set();
+    return integer(number.ptr());
+}
+
 // An integer, or something equal to one (4.0); other numbers and text are refused.
 long long whole(PyObject* o) {
     if (PyLong_Check(o)) return integer(o);
@@ -333,7 +341,7 @@ PyObject* recon_downsample(PyObject*, PyObject* const* a, Py_ssize_t n) {
     need(xhat, tensor(a[2]));
     need_dims(xhat, 4);
     if (xhat.scalar_type() != at::kFloat) TORCH_CHECK_TYPE(false, "xhat must be float32");
-    const int64_t B = xhat.size(0), C = xhat.size(1), side = whole(a[1]);
+    const int64_t B = xhat.size(0), C = xhat.size(1), side = a[2] == Py_None ? index(a[1]) : whole(a[1]);
     const at::Tensor out = or_empty(tensor(a[2]), xhat, {B, C, side, side}, at::kFloat);
     if (out.scalar_type() != at::kFloat || out.sizes() != at::IntArrayRef({B, C, side, side})) TORCH_CHECK_VALUE(false, "out must be float32 [B, C, out_side, out_side]");
     const int status = call(entry.hmar_recon_downsample, (const float*)ptr(xhat), (float*)ptr(out), (int)B, (int)C, (int)xhat.size(2), (int)side, stream_of(a[3]));

@@ -271,6 +271,12 @@ def test_downsample_refuses_sides_that_are_not_whole(given, side):
         hmar.hmar_recon_downsample(x, side, out=out)
 
 
+def test_downsample_makes_no_output_from_a_float_side():
+    import torch
+    with pytest.raises(TypeError):
+        hmar.hmar_recon_downsample(_cuda_tensor_without_memory(1, 1, 8, 8, dtype=torch.float32), 4.0)
+
+
 def test_side_lists_have_a_length():
     """A generator is refused (a call could use it up once); every sized collection of numbers is taken."""
     import torch
