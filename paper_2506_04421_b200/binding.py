@@ -2,14 +2,17 @@
 
 Every function here has the name and argument order of the C entry point it wraps (see
 include/hmar.h). Tensors are torch CUDA tensors used purely as device buffers; all of the
-arithmetic runs inside the library's kernels. There is no CPU fallback: if the shared library
-is missing or fails to load, importing this module raises.
+arithmetic runs inside the library's kernels. There is no CPU fallback: the first call loads the
+library, and the first hot call the compiled module, each compiled first where its file is missing
+or older than its sources (nvcc, g++, and a package directory that can be written), and raises
+where that fails. build.build() compiles both ahead of time.
 """
 import ctypes
 import functools
 import importlib.machinery
 import importlib.util
 import os
+import threading
 
 import torch
 
@@ -17,6 +20,7 @@ from . import build as _build
 
 _LIB = None
 _HOST = None
+_LOADING = threading.Lock()
 
 HMAR_OK = 0
 HMAR_ERR_BAD_ARG = -1
@@ -132,6 +136,11 @@ def _host():
 
 
 def _load_host():
+    with _LOADING:                         # threads whose first calls meet compile and load the module once
+        return _HOST if _HOST is not None else _load_host_locked()
+
+
+def _load_host_locked():
     global _HOST
     library = lib()
     loader = importlib.machinery.ExtensionFileLoader("_hmar_host", _build.build_host())

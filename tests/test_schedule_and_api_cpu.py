@@ -294,3 +294,18 @@ def test_softmax_scale_is_whatever_float_takes():
     assert not isinstance(e.value, TypeError)
     with pytest.raises(ValueError):
         hmar.hmar_attn_fwd(q, q, q, (2,), "an eighth", out=q, lse=q)
+
+
+def test_first_calls_of_several_threads_load_the_module_once(monkeypatch):
+    import threading
+    import time
+    from paper_2506_04421_b200 import binding
+    path, built, got = binding._build.build_host(), [], []
+    monkeypatch.setattr(binding, "_HOST", None)
+    monkeypatch.setattr(binding._build, "build_host", lambda: (built.append(1), time.sleep(0.2), path)[2])
+    threads = [threading.Thread(target=lambda: got.append(binding._host())) for _ in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert len(built) == 1 and len(got) == 4 and all(m is got[0] for m in got)
