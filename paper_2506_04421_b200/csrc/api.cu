@@ -130,7 +130,7 @@ static int fwd_impl(const T* q, const T* k, const T* v, T* out, float* lse, int 
         if (tensor_core && !g_force_simt.load())
             return tc_fwd(q, k, v, out, lse, B * H, st, softmax_scale, device_status_ptr(), s);
     }
-    return simt_fwd<T>(q, k, v, out, lse, B * H, D, st, softmax_scale, s) == cudaSuccess ? HMAR_OK : HMAR_ERR_CUDA;
+    return launch_status(simt_fwd<T>(q, k, v, out, lse, B * H, D, st, softmax_scale, s));
 }
 
 template <typename T>
@@ -163,8 +163,7 @@ static int bwd_impl(const T* q, const T* k, const T* v, const T* out, const floa
                           device_status_ptr(), s);
     }
     (void)dq_acc;
-    return simt_bwd<T>(q, k, v, out, lse, dout, dq, dk, dv, delta, B * H, D, st, softmax_scale, s) == cudaSuccess
-               ? HMAR_OK : HMAR_ERR_CUDA;
+    return launch_status(simt_bwd<T>(q, k, v, out, lse, dout, dq, dk, dv, delta, B * H, D, st, softmax_scale, s));
 }
 
 // strides == nullptr: dense [B,H,n,D] tensors
@@ -205,8 +204,7 @@ static int step_impl(const T* q, const T* k_prev, const T* v_prev, const T* k_cu
                                  device_status_ptr(), s);
     }
     if (!dense) return HMAR_ERR_UNSUPPORTED;      // the plain kernels take dense tensors only
-    return simt_scale_step<T>(q, k_prev, v_prev, k_cur, v_cur, out, lse, B * H, D, n_prev, n_cur, softmax_scale, s)
-                   == cudaSuccess ? HMAR_OK : HMAR_ERR_CUDA;
+    return launch_status(simt_scale_step<T>(q, k_prev, v_prev, k_cur, v_cur, out, lse, B * H, D, n_prev, n_cur, softmax_scale, s));
 }
 
 }  // namespace hmar
@@ -428,8 +426,8 @@ int hmar_recon_accumulate(float* xhat, const float* codebook, const int* tokens_
     if (tokens_out != nullptr && (tokens_out == tokens_new || tokens_out == tokens_old)) return HMAR_ERR_BAD_ARG;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return HMAR_ERR_CUDA; }
-    return launch_recon_accumulate(xhat, codebook, tokens_old, tokens_new, mask, tokens_out, B, C, V, side, out_side,
-                                   static_cast<cudaStream_t>(stream)) == cudaSuccess ? HMAR_OK : HMAR_ERR_CUDA;
+    return launch_status(launch_recon_accumulate(xhat, codebook, tokens_old, tokens_new, mask, tokens_out, B, C, V, side, out_side,
+                                                 static_cast<cudaStream_t>(stream)));
 }
 
 int hmar_recon_downsample(const float* xhat, float* out, int B, int C, int in_side, int out_side, void* stream) {
@@ -438,8 +436,7 @@ int hmar_recon_downsample(const float* xhat, float* out, int B, int C, int in_si
     if (xhat == nullptr || out == nullptr || xhat == out) return HMAR_ERR_BAD_ARG;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return HMAR_ERR_CUDA; }
-    return launch_recon_downsample(xhat, out, B, C, in_side, out_side, static_cast<cudaStream_t>(stream)) == cudaSuccess
-               ? HMAR_OK : HMAR_ERR_CUDA;
+    return launch_status(launch_recon_downsample(xhat, out, B, C, in_side, out_side, static_cast<cudaStream_t>(stream)));
 }
 
 int hmar_selftest_bounded_wait(void* stream) {
@@ -447,7 +444,7 @@ int hmar_selftest_bounded_wait(void* stream) {
     if (rc != HMAR_OK) return rc;
     int* status = device_status_ptr();
     if (status == nullptr) return HMAR_ERR_CUDA;
-    return launch_selftest_wait(status, static_cast<cudaStream_t>(stream)) == cudaSuccess ? HMAR_OK : HMAR_ERR_CUDA;
+    return launch_status(launch_selftest_wait(status, static_cast<cudaStream_t>(stream)));
 }
 
 int hmar_debug_force_simt(int enable) { return g_force_simt.exchange(enable ? 1 : 0); }

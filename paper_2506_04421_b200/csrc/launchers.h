@@ -36,6 +36,14 @@ struct SmemOptIn {
     }
 };
 
+// What an entry point returns for the outcome of its launches.  A refused launch or copy leaves its error in the runtime,
+// where the check behind the next launch, which nothing refused, would find it: it is taken out here.
+inline int launch_status(cudaError_t e) {
+    if (e == cudaSuccess) return HMAR_OK;
+    cudaGetLastError();
+    return HMAR_ERR_CUDA;
+}
+
 // Launches a kernel whose blocks may start as soon as the last block of the previous kernel of its stream has ended: its
 // parameters and its own set-up no longer wait for that kernel's stores to be flushed.  It calls grid_wait() before it
 // touches anything that another kernel writes or reads, and before it takes tensor memory.  1.5 to 3 us per launch: forward

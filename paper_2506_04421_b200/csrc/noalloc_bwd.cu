@@ -156,7 +156,6 @@ extern "C" int hmar_attn_bwd_noalloc(const void* q, const void* k, const void* v
     a.dv = static_cast<__nv_bfloat16*>(dv);
     a.status = nullptr;
     a.st = st;
-    return launch_bwd_tc(mq, mk, mv, mdo, macc, a, static_cast<const __nv_bfloat16*>(out),
-                         static_cast<const __nv_bfloat16*>(dout), static_cast<__nv_bfloat16*>(dq), BH, s) == cudaSuccess
-               ? HMAR_OK : HMAR_ERR_CUDA;
+    return launch_status(launch_bwd_tc(mq, mk, mv, mdo, macc, a, static_cast<const __nv_bfloat16*>(out),
+                                       static_cast<const __nv_bfloat16*>(dout), static_cast<__nv_bfloat16*>(dq), BH, s));
 }

@@ -256,13 +256,14 @@ int step_small(const __nv_bfloat16* q, const __nv_bfloat16* k_prev, const __nv_b
     const size_t smem = (size_t)2 * keys_pad * ROW_BYTES;
     // the largest window needs more than the default 48 KB of dynamic shared memory
     static SmemOptIn opt_in;
-    if (opt_in((const void*)hmar_step_small_kernel, 2 * kSmallMaxKeys * ROW_BYTES) != cudaSuccess) return HMAR_ERR_CUDA;
+    const cudaError_t opted_in = opt_in((const void*)hmar_step_small_kernel, 2 * kSmallMaxKeys * ROW_BYTES);
+    if (opted_in != cudaSuccess) return launch_status(opted_in);
     {
         KernelTimer timer("hmar_step_small_kernel", stream);
         hmar_step_small_kernel<<<BH, warps * 32, smem, stream>>>(a);
     }
     count_launch(1);
-    return cudaGetLastError() == cudaSuccess ? HMAR_OK : HMAR_ERR_CUDA;
+    return launch_status(cudaGetLastError());
 }
 
 }  // namespace hmar

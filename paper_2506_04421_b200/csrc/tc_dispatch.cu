@@ -212,7 +212,7 @@ static int tc_fwd_strided(const bf16* q, const bf16* k, const bf16* v, bf16* out
     a.lse = lse;
     a.status = status;
     a.st = st;
-    return launch_fwd_tc(mq, mk, mv, mk, mv, a, B * H, stream) == cudaSuccess ? HMAR_OK : HMAR_ERR_CUDA;
+    return launch_status(launch_fwd_tc(mq, mk, mv, mk, mv, a, B * H, stream));
 }
 
 // Contiguous [B*H, L, 64] tensors: one "batch" of BH heads.
@@ -270,7 +270,7 @@ int tc_scale_step(const bf16* q, const bf16* k_prev, const bf16* v_prev, const b
     a.status = status;
     a.st.n_scales = 0;
     a.st.window = HMAR_WINDOW_MARKOV;
-    return launch_fwd_tc(mq, mk0, mv0, mk1, mv1, a, BH, stream) == cudaSuccess ? HMAR_OK : HMAR_ERR_CUDA;
+    return launch_status(launch_fwd_tc(mq, mk0, mv0, mk1, mv1, a, BH, stream));
 }
 
 // Backward on tensors whose layout is given by strides (elements): q, k, v share one layout, out and dout another,
@@ -319,20 +319,20 @@ static int tc_bwd_strided(const bf16* q, const bf16* k, const bf16* v, const bf1
         const size_t rows = (size_t)(plan->zero_end - plan->zero_begin);
         if (g.row == kHeadDim && g.head == (long long)L * kHeadDim && (B == 1 || g.batch == (long long)H * g.head)) {
             const size_t pitch = (size_t)L * kHeadDim * sizeof(bf16), width = rows * kHeadDim * sizeof(bf16);
-            if (cudaMemset2DAsync(dk + (size_t)plan->zero_begin * kHeadDim, pitch, 0, width, BH, stream) != cudaSuccess ||
-                cudaMemset2DAsync(dv + (size_t)plan->zero_begin * kHeadDim, pitch, 0, width, BH, stream) != cudaSuccess)
-                return HMAR_ERR_CUDA;
+            cudaError_t e = cudaMemset2DAsync(dk + (size_t)plan->zero_begin * kHeadDim, pitch, 0, width, BH, stream);
+            if (e == cudaSuccess) e = cudaMemset2DAsync(dv + (size_t)plan->zero_begin * kHeadDim, pitch, 0, width, BH, stream);
+            if (e != cudaSuccess) return launch_status(e);
         } else {
             for (int b = 0; b < B; ++b)
                 for (int h = 0; h < H; ++h) {
                     const long long off = b * g.batch + h * g.head + (long long)plan->zero_begin * g.row;
-                    if (cudaMemset2DAsync(dk + off, (size_t)g.row * sizeof(bf16), 0, kHeadDim * sizeof(bf16), rows, stream) != cudaSuccess ||
-                        cudaMemset2DAsync(dv + off, (size_t)g.row * sizeof(bf16), 0, kHeadDim * sizeof(bf16), rows, stream) != cudaSuccess)
-                        return HMAR_ERR_CUDA;
+                    cudaError_t e = cudaMemset2DAsync(dk + off, (size_t)g.row * sizeof(bf16), 0, kHeadDim * sizeof(bf16), rows, stream);
+                    if (e == cudaSuccess) e = cudaMemset2DAsync(dv + off, (size_t)g.row * sizeof(bf16), 0, kHeadDim * sizeof(bf16), rows, stream);
+                    if (e != cudaSuccess) return launch_status(e);
                 }
         }
     }
-    return launch_bwd_tc(mq, mk, mv, mdo, macc, a, out, dout, dq, BH, stream) == cudaSuccess ? HMAR_OK : HMAR_ERR_CUDA;
+    return launch_status(launch_bwd_tc(mq, mk, mv, mdo, macc, a, out, dout, dq, BH, stream));
 }
 
 // Contiguous [B*H, L, 64] tensors: one "batch" of BH heads.

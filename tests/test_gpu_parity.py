@@ -749,6 +749,65 @@ def test_overlapped_launches_see_what_the_calls_before_wrote(noalloc):
     _no_device_error()
 
 
+class _RefusedLaunches:
+    """While this is entered the runtime refuses, on the host, all work on the legacy default stream: a stream that
+    synchronises with it is being captured."""
+
+    def __enter__(self):
+        import ctypes
+        torch.cuda.synchronize()
+        self.cuda, self.stream = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p()
+        assert self.cuda.cuStreamCreate(ctypes.byref(self.stream), 0) == 0
+        assert self.cuda.cuStreamBeginCapture_v2(self.stream, 1) == 0
+
+    def __exit__(self, *exc):
+        import ctypes
+        graph = ctypes.c_void_p()
+        self.cuda.cuStreamEndCapture(self.stream, ctypes.byref(graph))      # the refused work has ended the capture
+        assert not graph.value and self.cuda.cuStreamDestroy_v2(self.stream) == 0
+
+
+@pytest.mark.parametrize("name", ["fwd", "bwd", "bwd_prev", "fwd_f32", "bwd_f32", "step", "step_small", "accumulate", "downsample", "copy"])
+def test_a_refused_launch_leaves_no_error_behind(name):
+    """A call whose launch the runtime refuses reports it, and the next call, which nothing refuses, succeeds: no error
+    stays in the runtime for it to find."""
+    dtype = torch.float32 if name.endswith("f32") else torch.bfloat16
+    sides, scale = (1, 3, 11), 0.125
+    L = sum(s * s for s in sides)
+    q, k, v, do = torch.randn((4, 1, 2, L, 64), device="cuda").to(dtype)
+    window = hmar.HMAR_WINDOW_PREV if name == "bwd_prev" else hmar.HMAR_WINDOW_MARKOV
+    out, lse = hmar.hmar_attn_fwd(q, k, v, sides, scale, window=window)
+    dq, dk, dv = (torch.empty_like(q) for _ in range(3))
+    ws = torch.empty(hmar.hmar_attn_bwd_workspace_bytes(1, 2, 64, sides), dtype=torch.uint8, device="cuda")
+    x, y, z = (torch.zeros((1, 8, s, s), device="cuda") for s in (16, 8, 16))
+    codebook, tokens = torch.ones((4, 8), device="cuda"), torch.zeros((1, 5, 5), dtype=torch.int32, device="cuda")
+    rows = lambda t, n: t.flatten()[:2 * n * 64].view(1, 2, n, 64)                              # noqa: E731
+    legacy = torch.cuda.default_stream()
+    assert legacy.cuda_stream == 0
+    backward = lambda: hmar.hmar_attn_bwd(q, k, v, out, lse, do, sides, scale, dq, dk, dv, ws, legacy, window)      # noqa: E731
+    call = {
+        "fwd": lambda: hmar.hmar_attn_fwd(q, k, v, sides, scale, out, lse, legacy),
+        "fwd_f32": lambda: hmar.hmar_attn_fwd(q, k, v, sides, scale, out, lse, legacy),
+        "bwd": backward, "bwd_prev": backward, "bwd_f32": backward,
+        "step": lambda: hmar.hmar_attn_scale_step(rows(q, 121), rows(k, 9), rows(v, 9), rows(k, 121), rows(v, 121), 3, 11, scale,
+                                                  rows(dq, 121), want_lse=False, stream=legacy),
+        "step_small": lambda: hmar.hmar_attn_scale_step(rows(q, 9), rows(k, 1), rows(v, 1), rows(k, 9), rows(v, 9), 1, 3, scale,
+                                                        rows(dq, 9), want_lse=False, stream=legacy),
+        "accumulate": lambda: hmar.hmar_recon_accumulate(x, codebook, tokens, stream=legacy),
+        "downsample": lambda: hmar.hmar_recon_downsample(x, 8, y, legacy),
+        "copy": lambda: hmar.hmar_recon_downsample(x, 16, z, legacy),
+    }[name]
+    call()                                      # what a first call looks up or allocates is there
+    with _RefusedLaunches():
+        with pytest.raises(hmar.HmarError) as e:
+            call()
+        assert e.value.status == hmar.HMAR_ERR_CUDA
+    hmar.hmar_attn_fwd(q, k, v, sides, scale, window=window)
+    call()
+    torch.cuda.synchronize()
+    _no_device_error()
+
+
 def test_edge_cases_through_the_checking_build():
     """The library compiled with -DHMAR_BOUNDS_CHECK compares every address its kernels form by their own
     arithmetic (plain loads and stores; TMA copies are clipped by the hardware) with the extent of its tensor and
