@@ -104,13 +104,6 @@ struct __align__(1024) SharedStorage {
 };
 #define AT(field) (base + (uint32_t)offsetof(SharedStorage, field))     // shared-memory address
 
-__device__ __forceinline__ void report_timeout(int* status, int where) {
-    if (status != nullptr) {
-        atomicCAS(status, 0, HMAR_ERR_DEVICE_TIMEOUT);
-        atomicCAS(status + 1, 0, where);
-    }
-}
-
 __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
@@ -230,7 +223,7 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     const int lane = threadIdx.x & 31;
 
     if ((base & 1023u) != 0) {
-        if (threadIdx.x == 0) report_timeout(args.status, 0x3FF);
+        if (threadIdx.x == 0) report_gave_up(args.status, 0x3FF);
         return;
     }
 
@@ -279,11 +272,7 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sm.tmem_base;
-    auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
-        if (warp_wait(bar, parity)) return true;
-        if (lane == 0) sm.gave_up = bar - base;
-        return false;
-    };
+    auto wait = [&](uint32_t bar, uint32_t parity) -> bool { return warp_wait_or_give_up(bar, parity, &sm.gave_up, bar - base); };
 
     // The block's items go through a ring.  `look(n)` waits until item n is there; its fields are then read in place, and
     // `done(n)` gives the slot back (once per warp; items are looked at and done in order).
@@ -826,7 +815,7 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         tc_fence_after();
         tmem_dealloc(tmem, TMEM_COLS);
     }
-    if (threadIdx.x == 0 && sm.gave_up != 0) report_timeout(args.status, (int)sm.gave_up);
+    if (threadIdx.x == 0) report_gave_up(args.status, sm.gave_up);
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -95,13 +95,6 @@ __device__ __forceinline__ KvTile kv_tile(const FwdWork& w, int tiles0, int j) {
 // columns issued for a tile with n_valid keys (a multiple of 16)
 __device__ __forceinline__ int tile_cols(int n_valid) { return (n_valid + 15) & ~15; }
 
-__device__ __forceinline__ void report_timeout(int* status, int where) {
-    if (status != nullptr) {
-        atomicCAS(status, 0, HMAR_ERR_DEVICE_TIMEOUT);
-        atomicCAS(status + 1, 0, where);
-    }
-}
-
 template <int N> __device__ __forceinline__ void reg_inc() {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
 }
@@ -121,7 +114,7 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     const int lane = threadIdx.x & 31;
 
     if ((base & 1023u) != 0) {
-        if (threadIdx.x == 0) report_timeout(args.status, 0x3FF);
+        if (threadIdx.x == 0) report_gave_up(args.status, 0x3FF);
         return;
     }
     // ---- which tile of which head
@@ -189,11 +182,7 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sm.tmem_base;
-    auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
-        if (warp_wait(bar, parity)) return true;
-        if (lane == 0) sm.gave_up = bar - base;
-        return false;
-    };
+    auto wait = [&](uint32_t bar, uint32_t parity) -> bool { return warp_wait_or_give_up(bar, parity, &sm.gave_up, bar - base); };
 
     if (sm.skip != 0) {
         // do no further work; the first copies have to land before the block's shared memory is given back
@@ -490,23 +479,24 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         tc_fence_after();
         tmem_dealloc(tmem, TMEM_COLS);
     }
-    if (threadIdx.x == 0 && sm.gave_up != 0) report_timeout(args.status, (int)sm.gave_up);
+    if (threadIdx.x == 0) report_gave_up(args.status, sm.gave_up);
 }
 
 // Self-test of the bounded waits: one block waits on a barrier that nothing ever arrives on, with a limit of
-// one millisecond, through the very wait and report functions the kernels use.  The wait gives up, the block
+// about a millisecond, through the very wait and report functions the kernels use.  The wait gives up, the block
 // records HMAR_ERR_DEVICE_TIMEOUT with location 0xD1A6 in the status word and returns; nothing traps.
 __global__ void hmar_selftest_wait_kernel(int* status) {
     __shared__ uint64_t never;
-    __shared__ int abort_flag;
+    __shared__ uint32_t gave_up;
     if (threadIdx.x == 0) {
-        abort_flag = 0;
+        gave_up = 0;
         mbar_init(&never, 1);
         fence_mbar_init();
     }
     __syncthreads();
-    const bool ok = __all_sync(0xffffffffu, mbar_wait(&never, 0, &abort_flag, 1000000ull));
-    if (!ok && threadIdx.x == 0) report_timeout(status, 0xD1A6);
+    warp_wait_or_give_up(smem_u32(&never), 0, &gave_up, 0xD1A6, 2000000u);
+    __syncthreads();
+    if (threadIdx.x == 0) report_gave_up(status, gave_up);
 }
 
 }  // namespace

@@ -1,11 +1,12 @@
 // Thin inline-PTX wrappers for sm_100a: mbarrier, TMA (cp.async.bulk.tensor), tcgen05 (MMA, TMEM
 // allocation, TMEM loads/stores, commit, fences).  Every wait is bounded: it gives up after about a
-// second of wall time, and the caller turns that into an error status instead of a hang.
+// second of the SM's clocks, and the caller turns that into an error status instead of a hang.
 #pragma once
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <cstdint>
+#include "../../include/hmar.h"
 
 namespace hmar {
 namespace ptx {
@@ -42,41 +43,7 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t by
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
                  : "memory");
 }
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-constexpr uint64_t kWaitLimitNs = 1000000000ull;   // one second
-
-// Waits for the phase with the given parity to complete.  Returns false if `*abort_flag` is (or
-// becomes) set, or if the wait has lasted longer than `limit_ns`; in the latter case it sets the
-// flag so that every other wait of the block gives up too.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                          uint64_t limit_ns = kWaitLimitNs) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = globaltimer_ns();
-    uint32_t spins = 0;
-    while (true) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if ((++spins & 63u) == 0) {
-            if (*abort_flag) return false;
-            if (globaltimer_ns() - t0 > limit_ns) {
-                *abort_flag = 1;
-                return false;
-            }
-        }
-    }
-}
-
-// The same operations on shared-memory addresses, and waits by a whole converged warp.  A kernel whose roles share one
+// The operations on shared-memory addresses, and waits by a whole converged warp.  A kernel whose roles share one
 // instruction cache is slowed down by every instruction it contains: this wait is a dozen instructions (no flag that
 // other waits look at: a role that gives up returns, and the roles that wait for it give up in turn).
 __device__ __forceinline__ void bar_arrive(uint32_t bar) {
@@ -115,12 +82,26 @@ __device__ __forceinline__ void warp_try_wait2(uint32_t bar_a, uint32_t parity_a
     done_b = b != 0;
 }
 constexpr uint32_t kWaitLimitClocks = 2000000000u;   // about a second
-__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity) {
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, uint32_t limit = kWaitLimitClocks) {
     const uint32_t t0 = clock();
 #pragma unroll 1
     while (!warp_try_wait(bar, parity))
-        if (__any_sync(0xffffffffu, (uint32_t)clock() - t0 > kWaitLimitClocks)) return false;
+        if (__any_sync(0xffffffffu, (uint32_t)clock() - t0 > limit)) return false;
     return true;
+}
+// The wait of the kernels' roles: one that runs out leaves `where` (nonzero) in the block's word `gave_up`, which
+// report_gave_up hands to the status word once, at the end of the block.
+__device__ __forceinline__ bool warp_wait_or_give_up(uint32_t bar, uint32_t parity, uint32_t* gave_up, uint32_t where,
+                                                     uint32_t limit = kWaitLimitClocks) {
+    if (warp_wait(bar, parity, limit)) return true;
+    if ((threadIdx.x & 31) == 0) *gave_up = where;
+    return false;
+}
+__device__ __forceinline__ void report_gave_up(int* status, uint32_t gave_up) {
+    if (status != nullptr && gave_up != 0) {
+        atomicCAS(status, 0, HMAR_ERR_DEVICE_TIMEOUT);
+        atomicCAS(status + 1, 0, (int)gave_up);
+    }
 }
 
 // ---------------------------------------------------------------------------------- TMA
