@@ -248,7 +248,7 @@ int hmar_schedule_bwd_full_tile_share(int n_scales, const int* side_lens, int wi
 
 /* Blocks until the work queued on the current device has finished, then returns the code recorded
  * by the kernels since the last call (HMAR_OK, or HMAR_ERR_DEVICE_TIMEOUT with *detail, if not NULL,
- * telling which wait gave up) and clears it.
+ * telling which wait gave up first) and clears it.
  * Every wait inside the tensor-core kernels is bounded (2e9 clocks of the SM: about one second at full clock,
  * longer below it; on a GPU shared by time slicing the time the context is switched out counts too).  When one
  * runs out, its role of the block gives up, the roles that wait for it follow, each when its own wait runs out,
@@ -258,10 +258,11 @@ int hmar_schedule_bwd_full_tile_share(int n_scales, const int* side_lens, int wi
  * about: HMAR_OK means every kernel since the previous call ran to completion. */
 int hmar_device_status(int* detail);
 
-/* Self-test of that mechanism (no counterpart in the paper): launches one block that waits, through the
+/* Self-test of that mechanism (no counterpart in the paper): launches one block in which a warp waits, through the
  * kernels' own wait and report routines with a limit of 2e6 clocks (about a millisecond), on a barrier nothing ever
- * arrives on.  The wait gives up and the block returns; the next hmar_device_status() reports
- * HMAR_ERR_DEVICE_TIMEOUT with detail 0xD1A6 and clears it.  Nothing traps or faults; the context stays usable. */
+ * arrives on, and a second warp, with a limit of 6e6, for the first.  Both give up and the block returns; the next
+ * hmar_device_status() reports HMAR_ERR_DEVICE_TIMEOUT with detail 0xD1A6, the first one's location (0xD1A7 is the
+ * second's), and clears it.  Nothing traps or faults; the context stays usable. */
 int hmar_selftest_bounded_wait(void* stream);
 
 /* Per-kernel timing for benchmarks.  Between hmar_profile_begin() and hmar_profile_end() every kernel

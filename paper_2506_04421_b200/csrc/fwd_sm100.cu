@@ -482,19 +482,25 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     if (threadIdx.x == 0) report_gave_up(args.status, sm.gave_up);
 }
 
-// Self-test of the bounded waits: one block waits on a barrier that nothing ever arrives on, with a limit of
-// about a millisecond, through the very wait and report functions the kernels use.  The wait gives up, the block
-// records HMAR_ERR_DEVICE_TIMEOUT with location 0xD1A6 in the status word and returns; nothing traps.
+// Self-test of the bounded waits: a warp waits on a barrier that nothing ever arrives on, with a limit of about a
+// millisecond, through the very wait and report functions the kernels use, and a second warp waits, three times as long,
+// for the first.  Both give up; the block records HMAR_ERR_DEVICE_TIMEOUT with the first one's location, 0xD1A6, in the
+// status word and returns; nothing traps.
 __global__ void hmar_selftest_wait_kernel(int* status) {
-    __shared__ uint64_t never;
+    __shared__ uint64_t never, after;
     __shared__ uint32_t gave_up;
     if (threadIdx.x == 0) {
         gave_up = 0;
         mbar_init(&never, 1);
+        mbar_init(&after, 1);
         fence_mbar_init();
     }
     __syncthreads();
-    warp_wait_or_give_up(smem_u32(&never), 0, &gave_up, 0xD1A6, 2000000u);
+    if (threadIdx.x < 32) {
+        if (warp_wait_or_give_up(smem_u32(&never), 0, &gave_up, 0xD1A6, 2000000u) && threadIdx.x == 0) bar_arrive(smem_u32(&after));
+    } else {
+        warp_wait_or_give_up(smem_u32(&after), 0, &gave_up, 0xD1A7, 6000000u);
+    }
     __syncthreads();
     if (threadIdx.x == 0) report_gave_up(status, gave_up);
 }
@@ -502,7 +508,7 @@ __global__ void hmar_selftest_wait_kernel(int* status) {
 }  // namespace
 
 cudaError_t launch_selftest_wait(int* status, cudaStream_t stream) {
-    hmar_selftest_wait_kernel<<<1, 32, 0, stream>>>(status);
+    hmar_selftest_wait_kernel<<<1, 64, 0, stream>>>(status);
     count_launch(1);
     return cudaGetLastError();
 }

@@ -89,12 +89,13 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, uint32_
         if (__any_sync(0xffffffffu, (uint32_t)clock() - t0 > limit)) return false;
     return true;
 }
-// The wait of the kernels' roles: one that runs out leaves `where` (nonzero) in the block's word `gave_up`, which
-// report_gave_up hands to the status word once, at the end of the block.
+// The wait of the kernels' roles: the first of a block that runs out leaves `where` (nonzero) in the block's word `gave_up`,
+// which report_gave_up hands to the status word once, at the end of the block.  (The roles that wait for the one that gave
+// up run out in turn, a second later each: the last would name a victim, not the cause.)
 __device__ __forceinline__ bool warp_wait_or_give_up(uint32_t bar, uint32_t parity, uint32_t* gave_up, uint32_t where,
                                                      uint32_t limit = kWaitLimitClocks) {
     if (warp_wait(bar, parity, limit)) return true;
-    if ((threadIdx.x & 31) == 0) *gave_up = where;
+    if ((threadIdx.x & 31) == 0) atomicCAS(gave_up, 0u, where);
     return false;
 }
 __device__ __forceinline__ void report_gave_up(int* status, uint32_t gave_up) {

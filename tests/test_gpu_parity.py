@@ -572,6 +572,14 @@ def test_bounded_wait_runs_out_reports_and_leaves_the_context_usable():
     _run_training(wl, torch.bfloat16)                           # and the library is back to normal
 
 
+def test_the_wait_that_ran_out_first_is_the_one_reported():
+    """The self-test's second warp waits for its first, which waits in vain: when both have given up the status word
+    holds the first one's location, not that of the role that gave up last."""
+    for _ in range(5):
+        hmar.hmar_selftest_bounded_wait()
+        assert hmar.hmar_device_status() == (hmar.HMAR_ERR_DEVICE_TIMEOUT, 0xD1A6)
+
+
 def test_bad_workspace_is_rejected():
     wl = CONFIGS["tiny"]
     q, k, v, do = training_inputs(wl)
