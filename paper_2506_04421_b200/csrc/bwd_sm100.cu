@@ -263,7 +263,10 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     // From here on memory is read with plain loads: delta was written by the kernel before, lse, V and (where the call
     // allocates nothing) the work list by earlier ones, so none of it is read-only for the lifetime of this launch, which
     // a non-coherent load would ask for.
-    if (args.status != nullptr && *reinterpret_cast<volatile int*>(args.status) != 0) return;
+    // Whether an earlier block gave up: one answer for all threads, since the word may change between two of them and the
+    // block's barriers and its tensor-memory allocation want whole warps.
+    const int given_up = args.status != nullptr ? *reinterpret_cast<volatile int*>(args.status) : 0;
+    if (__syncthreads_or(given_up)) return;
     if (warp == MMA_WARP) {
         tmem_alloc(&sm.tmem_base, TMEM_COLS);
         tmem_relinquish();

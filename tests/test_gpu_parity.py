@@ -580,6 +580,20 @@ def test_the_wait_that_ran_out_first_is_the_one_reported():
         assert hmar.hmar_device_status() == (hmar.HMAR_ERR_DEVICE_TIMEOUT, 0xD1A6)
 
 
+def test_backward_launched_while_the_status_word_is_latched_leaves_dk_and_dv_alone():
+    wl = _Wl((3, 11, 5))
+    q, k, v, do = training_inputs(wl, bf16=True)
+    tq, tk, tv, tdo = (to_device(x, wl.B, wl.H, torch.bfloat16) for x in (q, k, v, do))
+    out, lse = hmar.hmar_attn_fwd(tq, tk, tv, wl.side_lens, wl.softmax_scale)
+    hmar.hmar_selftest_bounded_wait()
+    dk, dv = torch.full_like(tk, 7.0), torch.full_like(tv, 7.0)
+    hmar.hmar_attn_bwd(tq, tk, tv, out, lse, tdo, wl.side_lens, wl.softmax_scale, dk=dk, dv=dv)
+    torch.cuda.synchronize()
+    assert (dk == 7.0).all() and (dv == 7.0).all()
+    assert hmar.hmar_device_status()[0] == hmar.HMAR_ERR_DEVICE_TIMEOUT
+    _run_training(wl, torch.bfloat16)
+
+
 def test_bad_workspace_is_rejected():
     wl = CONFIGS["tiny"]
     q, k, v, do = training_inputs(wl)
