@@ -246,6 +246,13 @@ int hmar_schedule_tiles_window(int n_scales, const int* side_lens, int window, i
  * others the one with three variants.  Returns a negative hmar_status for a bad side list.  Host only. */
 int hmar_schedule_bwd_full_tile_share(int n_scales, const int* side_lens, int window);
 
+/* The backward's work items in the order in which its persistent blocks take them, block by block: a backward over
+ * n_heads heads run by n_blocks blocks (one per SM, or one per item where there are fewer items).  An item is 4 int32:
+ * {block, head, first key row, 128-query steps}.  Returns the number of items, or a negative hmar_status; writes at most
+ * max_items of them (pass NULL / 0 to query the count).  Host only. */
+int hmar_schedule_bwd_items(int n_scales, const int* side_lens, int window, int n_heads, int n_blocks, int32_t* items,
+                            int max_items);
+
 /* Blocks until the work queued on the current device has finished, then returns the code recorded
  * by the kernels since the last call (HMAR_OK, or HMAR_ERR_DEVICE_TIMEOUT with *detail, if not NULL,
  * telling which wait gave up first) and clears it.

@@ -38,7 +38,7 @@ HMAR_WINDOW_PREV = 3        # scale k-1 only; the first scale attends to itself
 EXPORTED_SYMBOLS = (
     "hmar_attn_fwd", "hmar_attn_fwd_f32", "hmar_attn_fwd_window", "hmar_attn_fwd_window_f32", "hmar_attn_fwd_packed", "hmar_attn_bwd_packed",
     "hmar_attn_bwd_workspace_bytes", "hmar_attn_bwd", "hmar_attn_bwd_f32", "hmar_attn_bwd_window",
-    "hmar_attn_bwd_window_f32", "hmar_schedule_tiles_window", "hmar_attn_bwd_noalloc", "hmar_attn_scale_step", "hmar_attn_scale_step_f32", "hmar_attn_scale_step_strided", "hmar_schedule_tiles", "hmar_schedule_bwd_full_tile_share",
+    "hmar_attn_bwd_window_f32", "hmar_schedule_tiles_window", "hmar_attn_bwd_noalloc", "hmar_attn_scale_step", "hmar_attn_scale_step_f32", "hmar_attn_scale_step_strided", "hmar_schedule_tiles", "hmar_schedule_bwd_full_tile_share", "hmar_schedule_bwd_items",
     "hmar_recon_accumulate", "hmar_recon_downsample", "hmar_device_status", "hmar_selftest_bounded_wait", "hmar_profile_begin", "hmar_profile_end", "hmar_debug_force_simt", "hmar_launch_count", "hmar_shutdown",
     "hmar_status_string",
 )
@@ -78,6 +78,7 @@ def lib():
     L.hmar_attn_bwd_window_f32.argtypes = L.hmar_attn_bwd_window.argtypes
     L.hmar_schedule_tiles_window.argtypes = [i, ip, i, i, ctypes.POINTER(ctypes.c_int32), i]
     L.hmar_schedule_bwd_full_tile_share.argtypes = [i, ip, i]
+    L.hmar_schedule_bwd_items.argtypes = [i, ip, i, i, i, ctypes.POINTER(ctypes.c_int32), i]
     L.hmar_attn_bwd_noalloc.argtypes = [vp] * 9 + [i, i, i, i, ip, fp, vp]
     L.hmar_attn_scale_step.argtypes = [vp] * 7 + [i, i, i, i, i, fp, vp]
     L.hmar_attn_scale_step_f32.argtypes = L.hmar_attn_scale_step.argtypes
@@ -269,6 +270,19 @@ def hmar_schedule_tiles(side_lens, direction, window=HMAR_WINDOW_MARKOV):
     lib().hmar_schedule_tiles_window(n, sides, int(window), int(direction), buf, count)
     keys = ("row_begin", "row_count", "partner_begin", "partner_end", "uniform", "cost")
     return [dict(zip(keys, buf[6 * t:6 * t + 6])) for t in range(count)]
+
+
+def hmar_schedule_bwd_items(side_lens, n_heads, n_blocks, window=HMAR_WINDOW_MARKOV):
+    """The backward's items as (block, head, first key row, steps), block by block in the order in which the blocks take
+    them (host only; needs no GPU)."""
+    sides, n = _sides(side_lens)
+    count = lib().hmar_schedule_bwd_items(n, sides, int(window), int(n_heads), int(n_blocks), None, 0)
+    if count < 0:
+        raise HmarError(count, "hmar_schedule_bwd_items")
+    buf = (ctypes.c_int32 * (4 * count))()
+    lib().hmar_schedule_bwd_items(n, sides, int(window), int(n_heads), int(n_blocks), buf, count)
+    flat = list(buf)
+    return [tuple(flat[4 * t:4 * t + 4]) for t in range(count)]
 
 
 def hmar_schedule_bwd_full_tile_share(side_lens, window=HMAR_WINDOW_MARKOV):

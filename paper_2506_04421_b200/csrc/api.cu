@@ -367,6 +367,15 @@ int hmar_schedule_bwd_full_tile_share(int n_scales, const int* side_lens, int wi
     return tc_bwd_full_tile_permille(st);
 }
 
+int hmar_schedule_bwd_items(int n_scales, const int* side_lens, int window, int n_heads, int n_blocks, int32_t* items,
+                            int max_items) {
+    ScaleTable st;
+    int rc = check_sides(n_scales, side_lens, window, &st);
+    if (rc != HMAR_OK) return rc;
+    if (n_heads <= 0 || n_heads > 65535 || n_blocks <= 0 || n_blocks > 65535) return HMAR_ERR_BAD_ARG;
+    return tc_bwd_items(st, n_heads, n_blocks, items, max_items);
+}
+
 int hmar_device_status(int* detail) {
     if (cudaDeviceSynchronize() != cudaSuccess) { cudaGetLastError(); return HMAR_ERR_CUDA; }
     int host[2] = {0, 0};

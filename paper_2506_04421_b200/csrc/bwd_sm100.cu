@@ -290,28 +290,16 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         reg_dec<REGS_MISC>();
         if (warp == SCHED_WARP) {
             // ================================================================== item scheduler
-            // A head's tiles are ordered by cost; tiles of equal cost are one class.  The launch works class by class,
-            // head by head inside a class, and the items are dealt to the blocks round by round, back and forth.  The
-            // blocks' sums then differ by 0.6 % (L = 9451, 192 heads) where a stretch or several runs of heads per block
-            // differed by 12 %, and the blocks work on few heads at a time: at L = 2240 18, whose dQ accumulators stay
-            // in L2.  (by_head: one class, see the launcher.)  The last records say that there are no more (the readers look up to two items ahead).
-            const int total = args.n_heads * args.n_work;
+            // The last records say that there are no more (the readers look up to two items ahead).
             int extra = 0;
             for (int n = 0; extra < 3; ++n) {
                 const int slot = n % ITEM_STAGES;
                 if (n >= ITEM_STAGES && !wait(AT(item_empty) + slot * 8, ((n / ITEM_STAGES) & 1) ^ 1)) break;
-                int pos = n * (int)gridDim.x + ((n & 1) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x);
                 Item it;
                 it.steps_uniform = 0;
-                if (pos < total) {
-                    int t = 0, count = args.by_head ? args.n_work : args.work[0].class_count;
-                    while (pos >= args.n_heads * count) {
-                        pos -= args.n_heads * count;
-                        t += count;
-                        count = args.work[t].class_count;
-                    }
-                    it.bh = pos / count;
-                    const BwdWork w = args.work[t + pos - it.bh * count];
+                const int tile = bwd_deal(args.work, args.n_work, args.n_heads, args.by_head, (int)gridDim.x, (int)blockIdx.x, n, it.bh);
+                if (tile >= 0) {
+                    const BwdWork w = args.work[tile];
                     it.batch = STRIDED ? it.bh / args.heads_per_batch : 0;
                     it.head = it.bh - it.batch * args.heads_per_batch * (STRIDED ? 1 : 0);
                     it.row_begin = w.row_begin;
@@ -898,8 +886,6 @@ static int sm_count() {
     return cached[dev];
 }
 
-constexpr size_t kL2Bytes = 126u << 20;
-
 // Side lists with fewer than this share (in thousandths) of their steps in full tiles run the one-variant
 // instantiation (L = 680 has 42 %, L = 2240 has 82 %).
 constexpr int kOneMaskBelowPermille = 600;
@@ -922,12 +908,7 @@ static cudaError_t launch_bwd_tc_layout(const CUtensorMap& q, const CUtensorMap&
         const long long items = (long long)BH * args.n_work;
         const unsigned grid = (unsigned)(items < sm_count() ? items : sm_count());
         BwdArgs a = args;
-        // Class by class a head's rows are read once per class.  Where its items are short (a mean of fewer than four steps) and
-        // the tensors do not stay in L2, that costs more than the balance gives, and the items go head by head: L = 680
-        // 960 heads 311 -> 285 us, L = 395 768 heads 148 -> 132.  Otherwise it is the other way round: L = 680 128 heads
-        // 53.3 against 49.5, L = 1000 192 heads 100 against 96.6, L = 2240 96 heads 200 against 185.
-        const size_t row_bytes = 4 * D * sizeof(__nv_bfloat16) + D * sizeof(float);     // Q, K, V, dO and the dQ accumulator
-        a.by_head = args.head_steps < 4 * args.n_work && n_rows * row_bytes > kL2Bytes + kL2Bytes / 4;
+        a.by_head = bwd_by_head(args.head_steps, args.n_work, n_rows);
         static SmemOptIn opt_in[2];
         const bool one_mask = args.plain_permille < kOneMaskBelowPermille;
         auto kernel = one_mask ? hmar_bwd_tc_kernel<STRIDED, true> : hmar_bwd_tc_kernel<STRIDED, false>;

@@ -72,13 +72,42 @@ inline int bwd_plain_permille(const BwdWork* work, int n) {
     return total > 0 ? (int)(plain * 1000 / total) : 1000;
 }
 
+constexpr size_t kL2Bytes = 126u << 20;
+
+// Whether the backward's items go head by head instead of class by class.  Class by class a head's rows are read once per
+// class.  Where its items are short (a mean of fewer than four steps) and the tensors do not stay in L2, that costs more than
+// the balance gives: head by head L = 680 960 heads 311 -> 285 us, L = 395 768 heads 148 -> 132.  Otherwise it is the other
+// way round: L = 680 128 heads 53.3 against 49.5, L = 1000 192 heads 100 against 96.6, L = 2240 96 heads 200 against 185.
+inline bool bwd_by_head(int head_steps, int n_work, size_t n_rows) {
+    const size_t row_bytes = 4 * kHeadDim * sizeof(__nv_bfloat16) + kHeadDim * sizeof(float);     // Q, K, V, dO and the dQ accumulator
+    return head_steps < 4 * n_work && n_rows * row_bytes > kL2Bytes + kL2Bytes / 4;
+}
+
+// The item that a block takes in a round: returns its tile and sets its head, or returns -1 where there are no more.
+// A head's tiles are ordered by cost; tiles of equal cost are one class.  The launch works class by class, head by head
+// inside a class (by_head: all tiles are one class), and the items are dealt to the blocks round by round, back and forth.
+// The blocks' sums then differ by 0.6 % (L = 9451, 192 heads) where a stretch or several runs of heads per block differed by
+// 12 %, and the blocks work on few heads at a time: at L = 2240 18, whose dQ accumulators stay in L2.
+HMAR_HD int bwd_deal(const BwdWork* work, int n_work, int n_heads, int by_head, int n_blocks, int block, int round, int& head) {
+    int pos = round * n_blocks + ((round & 1) ? n_blocks - 1 - block : block);
+    if (pos >= n_heads * n_work) return -1;
+    int t = 0, count = by_head ? n_work : work[0].class_count;
+    while (pos >= n_heads * count) {
+        pos -= n_heads * count;
+        t += count;
+        count = work[t].class_count;
+    }
+    head = pos / count;
+    return t + pos - head * count;
+}
+
 struct BwdArgs {
     const BwdWork* work;
     int n_work;
     int n_heads;             // B * H
     int plain_permille;      // from bwd_plain_permille: picks the instantiation of the main kernel
     int head_steps;          // steps of all tiles of a head (from bwd_fill_classes)
-    int by_head;             // set by the launcher: items in head order instead of class by class
+    int by_head;             // set by the launcher (bwd_by_head)
     int L;
     float scale_log2;        // softmax_scale * log2(e)
     float softmax_scale;

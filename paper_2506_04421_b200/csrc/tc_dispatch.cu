@@ -123,6 +123,25 @@ int tc_bwd_full_tile_permille(const ScaleTable& st) {
     return bwd_plain_permille(bwork.data(), (int)bwork.size());
 }
 
+int tc_bwd_items(const ScaleTable& st, int n_heads, int n_blocks, int32_t* items, int max_items) {
+    int zb = 0, ze = 0, count = 0;
+    std::vector<BwdWork> bwork = make_bwd_work(st, zb, ze);
+    const int n_work = (int)bwork.size(), head_steps = bwd_fill_classes(bwork.data(), n_work);
+    const bool by_head = bwd_by_head(head_steps, n_work, (size_t)n_heads * st.start[st.n_scales]);
+    for (int block = 0; block < n_blocks; ++block)
+        for (int round = 0;; ++round) {
+            int head = 0;
+            const int tile = bwd_deal(bwork.data(), n_work, n_heads, by_head, n_blocks, block, round, head);
+            if (tile < 0) break;
+            if (items != nullptr && count < max_items) {
+                const int32_t item[4] = {block, head, bwork[tile].row_begin, (bwork[tile].q_end - bwork[tile].q_begin + 127) / 128};
+                std::copy(item, item + 4, items + 4 * (size_t)count);
+            }
+            ++count;
+        }
+    return count;
+}
+
 static const Plan* get_plan(const ScaleTable& st) {
     PlanKey key;
     if (cudaGetDevice(&key.device) != cudaSuccess) return nullptr;

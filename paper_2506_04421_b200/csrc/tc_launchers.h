@@ -16,6 +16,8 @@ int tc_bwd(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* 
            int* status, cudaStream_t stream);
 // Share (thousandths) of a head's backward steps that lie in full tiles; picks the main kernel's instantiation.  Host only.
 int tc_bwd_full_tile_permille(const ScaleTable& st);
+// The backward's items block by block, in the order in which a block takes them; see hmar_schedule_bwd_items.  Host only.
+int tc_bwd_items(const ScaleTable& st, int n_heads, int n_blocks, int32_t* items, int max_items);
 int tc_bwd_packed(const __nv_bfloat16* qkv, const __nv_bfloat16* out, const float* lse, const __nv_bfloat16* dout,
                   __nv_bfloat16* dqkv, float* delta, float* dq_acc, int B, int H, const ScaleTable& st, float scale,
                   int* status, cudaStream_t stream);

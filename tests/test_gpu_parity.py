@@ -343,24 +343,24 @@ def _sample_heads(BH, n=6):
 
 
 def _partition_heads(wl, n, window=hmar.HMAR_WINDOW_MARKOV):
-    """Heads for the full-size comparisons, taken from the backward's own partition of the work.
+    """Heads for the full-size comparisons, taken from the backward's own dealing of the work.
 
-    The backward runs one persistent block per SM; block b takes the items (head, key tile) whose cost, in the
-    head-by-head order of the item list, lies in [total * b / blocks, total * (b + 1) / blocks), a tile costing
-    its 128-query steps plus two.  The hand-over between two items of different heads, and the first and last
-    item of a block, are the places where a mistake would hide from a comparison of whole heads chosen at
-    random, so the heads picked are those in which a block's run starts strictly inside the head, spread over
-    the blocks, always with the first and the last head.  (For sequences cut into several runs per head every
-    head has such boundaries.)"""
+    The backward runs one persistent block per SM and deals its items (head, key tile) to the blocks round by round, in
+    the library's own order.  The first and the last item of a block, its hand-overs from a class of equal cost to the
+    next, and the last round, which not every block has, are the places where a mistake would hide from a comparison of
+    whole heads chosen at random, so the heads picked are those of such items, spread over the list, always with the
+    first and the last head."""
     BH = wl.B * wl.H
-    tiles = hmar.hmar_schedule_tiles(wl.side_lens, 1, window)
-    head_cost = sum((t["partner_end"] - t["partner_begin"] + 127) // 128 + 2 for t in tiles)
     blocks = torch.cuda.get_device_properties(0).multi_processor_count
-    total = BH * head_cost
-    inside = sorted({(total * b // blocks) // head_cost for b in range(1, blocks) if (total * b // blocks) % head_cost})
-    inside = [h for h in inside if 0 < h < BH - 1] or list(range(1, BH - 1))
-    step = max(1, len(inside) // max(1, n - 2))
-    return sorted({0, BH - 1} | set(inside[::step][:max(0, n - 2)]))
+    items = hmar.hmar_schedule_bwd_items(wl.side_lens, BH, blocks, window)
+    heads = set()
+    for (before, h0, _, steps0), (block, h1, _, steps1) in zip([(-1, 0, 0, 0)] + items, items + [(blocks, 0, 0, 0)]):
+        if before != block or steps0 != steps1:                # an item that ends a run and the one that begins the next
+            heads |= ({h0} if before >= 0 else set()) | ({h1} if block < blocks else set())
+    inside = [h for h in sorted(heads) if 0 < h < BH - 1]
+    assert inside
+    picked = [inside[k * (len(inside) - 1) // max(1, n - 3)] for k in range(n - 2)]
+    return sorted({0, BH - 1} | set(picked))
 
 
 def _check_sampled(wl, heads, window_id, window_name, backward, chunk):
@@ -400,7 +400,7 @@ def test_block_causal_full_size_sampled_heads():
 def test_full_size_configs_sampled_heads(name):
     """Configs 2-4 (and the 1024 shape) at their full sizes, in the launch shape the benchmark times; the oracle
     checks a sample of heads element by element: at least 32 (8 at L = 9451, where one head costs the oracle
-    several seconds and gigabytes), chosen where the backward's blocks change heads."""
+    several seconds and gigabytes), taken from the items with which the backward's blocks begin, end or change class."""
     wl = CONFIGS[name]
     backward = "bwd" in wl.passes
     n_heads = 8 if wl.L > 4000 else 32

@@ -309,3 +309,41 @@ def test_first_calls_of_several_threads_load_the_module_once(monkeypatch):
     for t in threads:
         t.join()
     assert len(built) == 1 and len(got) == 4 and all(m is got[0] for m in got)
+
+
+@pytest.mark.parametrize("window", WINDOWS, ids=[w[0] for w in WINDOWS])
+@pytest.mark.parametrize("sides, n_heads, n_blocks", [
+    ((1,), 1, 1), ((1,), 3, 148), ((1, 1), 149, 148), ((3, 11), 7, 5), ((2, 1, 3, 1, 2), 37, 4), ((1, 2, 4, 8, 16, 32, 64), 3, 148),
+    (CONFIGS["256_d30_train"].side_lens, 31, 148), (CONFIGS["256_d30_train"].side_lens, 960, 148), (CONFIGS["512_d24_train"].side_lens, 2, 148),
+    (CONFIGS["512_d24_train"].side_lens, 47, 147), ((13, 17, 19), 5, 3)])
+def test_backward_deals_every_item_once(sides, n_heads, n_blocks, window):
+    """What the blocks of the backward take, from the function the kernel calls: every (head, key tile) with queries exactly
+    once, in either order (class by class, head by head), with fewer items than blocks, one block, and a last round that
+    only some blocks have."""
+    items = hmar.hmar_schedule_bwd_items(sides, n_heads, n_blocks, window[1])
+    tiles = {t["row_begin"]: t["cost"] for t in hmar.hmar_schedule_tiles(sides, 1, window[1]) if t["cost"] > 0}
+    assert sorted((h, r) for _, h, r, _ in items) == sorted((h, r) for h in range(n_heads) for r in tiles)
+    assert all(steps == tiles[r] for _, _, r, steps in items)
+    blocks = [b for b, _, _, _ in items]
+    assert blocks == sorted(blocks) and 0 <= min(blocks) and max(blocks) < n_blocks
+    counts = np.bincount(blocks, minlength=n_blocks)
+    assert counts.max() - counts.min() <= 1
+
+
+def test_backward_order_of_items():
+    """Lists of short items whose tensors exceed L2 go head by head, the others class by class, costliest first; dealt back
+    and forth, the blocks' sums of steps stay within a percent of one another where there are many items."""
+    def first_round(sides, n_heads):
+        items = hmar.hmar_schedule_bwd_items(sides, n_heads, 148)
+        return [next(it for it in items if it[0] == b) for b in range(148)], items
+    short, long_ = CONFIGS["256_d30_train"].side_lens, (1, 2, 3, 4, 5, 7, 9, 12, 16, 21, 27, 36, 48, 64)
+    first, _ = first_round(short, 960)
+    per_head = len(set(r for _, _, r, _ in first))
+    assert [h for _, h, _, _ in first] == [b // per_head for b in range(148)]
+    first, _ = first_round(short, 128)
+    assert len({steps for _, _, _, steps in first}) == 1
+    first, items = first_round(long_, 192)
+    sums = np.zeros(148)
+    for b, _, _, steps in items:
+        sums[b] += steps
+    assert sums.max() - sums.min() <= 0.01 * sums.mean()
