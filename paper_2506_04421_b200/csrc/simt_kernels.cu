@@ -3,7 +3,8 @@
 // are float or bf16.
 //
 // A block of 128 threads owns a tile of up to 64 rows of ONE scale, so all of its rows see the same contiguous range of
-// the other operand (mask: paper Sec. 4.1, Fig. attn-mask) and no element needs a mask but the ragged end of that range.
+// the other operand (mask: paper Sec. 4.1, Fig. attn-mask) and no element needs a mask but the ragged end of that range
+// (calls of small scales: one warp, 16 rows; see tile_height).
 // It walks the range 64 rows at a time, as small dense products from shared memory with 8 x 4 results per thread: 12
 // 16-byte shared-memory loads feed 128 FMAs, which leaves the FMA pipe as the bound (a warp's loads take half of the
 // shared-memory cycles its FMAs last).  One row per thread pair, an operand of every FMA from shared memory, was bound
@@ -12,14 +13,18 @@
 // start first and spread over the SMs (head by head, an SM could get three of them and another none).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+
+#include <algorithm>
+
 #include "hmar_common.h"
 #include "launchers.h"
 
 namespace hmar {
 namespace {
 
-constexpr int TR = 64;             // rows of a tile, on either side
-constexpr int THREADS = 128;       // thread t: rows 8 (t / 16) .. + 7, columns t % 16 + {0, 16, 32, 48} of a 64 x 64 product
+// A tile has TR rows on either side, 64 or 16, and 2 TR threads: thread t has rows 8 (t / 16) .. + 7 and columns
+// t % 16 + 16 j, j < TR / 16, of a TR x TR product.
+constexpr int DELTA_THREADS = 128;
 
 __device__ __forceinline__ float to_f(float x) { return x; }
 __device__ __forceinline__ float to_f(__nv_bfloat16 x) { return __bfloat162float(x); }
@@ -35,14 +40,14 @@ __device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
 }
 
 // Rows in shared memory are padded by four floats: 16-byte loads of eight consecutive rows then hit 32 distinct banks.
-template <int D> struct RowTile { float v[TR][D + 4]; };
-struct SquareTile { float v[TR][TR + 4]; };
+template <int D, int TR> struct RowTile { float v[TR][D + 4]; };
+template <int TR> struct SquareTile { float v[TR][TR + 4]; };
 
 // dst rows [0, TR) = src rows [0, n) as float; the rest zeros.
-template <typename T, int D>
-__device__ __forceinline__ void stage(RowTile<D>& dst, const T* src, int n) {
+template <typename T, int D, int TR>
+__device__ __forceinline__ void stage(RowTile<D, TR>& dst, const T* src, int n) {
 #pragma unroll 8
-    for (int idx = threadIdx.x; idx < TR * (D / 4); idx += THREADS) {
+    for (int idx = threadIdx.x; idx < TR * (D / 4); idx += 2 * TR) {
         const int r = idx / (D / 4), c = idx % (D / 4) * 4;
         *reinterpret_cast<float4*>(&dst.v[r][c]) = r < n ? load4(src + (size_t)r * D + c) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
@@ -51,20 +56,21 @@ __device__ __forceinline__ void stage(RowTile<D>& dst, const T* src, int n) {
 // acc[i][j] = sum_d a[r0 + i][d] b[tx + 16 j][d].  Sums of eight products are added up: one chain over all of d doubles
 // the rounding error of large logits (LSE at |logits| = 30, D = 64: 1.1e-5 against 0.6e-5), and an addition per eight
 // FMAs costs less than that.
-template <int D>
-__device__ __forceinline__ void product_nt(const RowTile<D>& a, const RowTile<D>& b, int r0, int tx, float (&acc)[8][4]) {
+template <int D, int TR>
+__device__ __forceinline__ void product_nt(const RowTile<D, TR>& a, const RowTile<D, TR>& b, int r0, int tx, float (&acc)[8][TR / 16]) {
+    constexpr int J = TR / 16;
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+        for (int j = 0; j < J; ++j) acc[i][j] = 0.f;
     // two chunks of d per round for D = 128 (bf16, 32 heads of L = 680: forward 190 -> 132 us, backward 558 -> 542); D = 64 is
     // the same either way, and D = 32 1 % slower
     constexpr int UNROLL = D == 128 ? 2 : 1;
 #pragma unroll UNROLL
     for (int d = 0; d < D; d += 8) {
-        float4 b0[4], b1[4];
+        float4 b0[J], b1[J];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < J; ++j) {
             b0[j] = *reinterpret_cast<const float4*>(&b.v[tx + 16 * j][d]);
             b1[j] = *reinterpret_cast<const float4*>(&b.v[tx + 16 * j][d + 4]);
         }
@@ -73,7 +79,7 @@ __device__ __forceinline__ void product_nt(const RowTile<D>& a, const RowTile<D>
             const float4 a0 = *reinterpret_cast<const float4*>(&a.v[r0 + i][d]);
             const float4 a1 = *reinterpret_cast<const float4*>(&a.v[r0 + i][d + 4]);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < J; ++j) {
                 float t = fmaf(a0.w, b0[j].w, fmaf(a0.z, b0[j].z, fmaf(a0.y, b0[j].y, a0.x * b0[j].x)));
                 t = fmaf(a1.w, b1[j].w, fmaf(a1.z, b1[j].z, fmaf(a1.y, b1[j].y, fmaf(a1.x, b1[j].x, t))));
                 acc[i][j] += t;
@@ -88,8 +94,8 @@ template <int D> struct Cols {
 };
 
 // acc[i][.] += sum_k p[r0 + i][k] b[k][columns of the thread], k < n (a multiple of 4)
-template <int D>
-__device__ __forceinline__ void product_nn(const SquareTile& p, const RowTile<D>& b, int r0, int tx, int n, float (&acc)[8][Cols<D>::N]) {
+template <int D, int TR>
+__device__ __forceinline__ void product_nn(const SquareTile<TR>& p, const RowTile<D, TR>& b, int r0, int tx, int n, float (&acc)[8][Cols<D>::N]) {
     constexpr int W = Cols<D>::W, G = Cols<D>::GROUPS;
 #pragma unroll 2
     for (int k = 0; k < n; k += 4) {
@@ -136,6 +142,7 @@ __device__ __forceinline__ void store_rows(T* dst, const float (&acc)[8][Cols<D>
 
 // Tile number `t` of a head: rows [row0, row0 + n) of scale s.  Tiles of the last scale come first.
 struct TileRows { int s, row0, n; };
+template <int TR>
 __device__ __forceinline__ TileRows tile_rows(const ScaleTable& st, int t) {
     int s = st.n_scales - 1;
     while (true) {
@@ -149,18 +156,19 @@ __device__ __forceinline__ TileRows tile_rows(const ScaleTable& st, int t) {
 // ---------------------------------------------------------------------------------------------
 // Forward and inference step.  The keys are rows [lo, hi) of one sequence, or (inference step: st has one scale, the
 // queries) n0 rows of the previous scale followed by n1 of the current one.
-template <int D> struct FwdSmem { RowTile<D> q, k, v; SquareTile p; };
+template <int D, int TR> struct FwdSmem { RowTile<D, TR> q, k, v; SquareTile<TR> p; };
 
-template <typename T, int D>
-__global__ void __launch_bounds__(THREADS)
+template <typename T, int D, int TR>
+__global__ void __launch_bounds__(2 * TR)
 simt_fwd_kernel(const T* __restrict__ q, const T* __restrict__ k0, const T* __restrict__ v0,
                 const T* __restrict__ k1, const T* __restrict__ v1,
                 T* __restrict__ out, float* __restrict__ lse,
                 const __grid_constant__ ScaleTable st, int n_heads, int n_q, int n0, int n1, int dense, float scale) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    FwdSmem<D>& sm = *reinterpret_cast<FwdSmem<D>*>(smem_raw);
+    FwdSmem<D, TR>& sm = *reinterpret_cast<FwdSmem<D, TR>*>(smem_raw);
+    constexpr int J = TR / 16;
     const int bh = blockIdx.x % n_heads;
-    const TileRows tile = tile_rows(st, blockIdx.x / n_heads);
+    const TileRows tile = tile_rows<TR>(st, blockIdx.x / n_heads);
     const int tx = threadIdx.x & 15, r0 = (threadIdx.x >> 4) * 8;
     const bool live = (threadIdx.x >> 5) * 16 < tile.n;     // the warp has rows of the tile
     const int lo = dense ? 0 : st.start[first_key_scale(st.window, tile.s)];
@@ -188,13 +196,13 @@ simt_fwd_kernel(const T* __restrict__ q, const T* __restrict__ k0, const T* __re
         stage(sm.v, vs, n);
         __syncthreads();
         if (live) {
-            float s[8][4];
+            float s[8][J];
             product_nt(sm.q, sm.k, r0, tx, s);
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 float mx = -INFINITY;
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
+                for (int j = 0; j < J; ++j) {
                     s[i][j] = tx + 16 * j < n ? s[i][j] * scale : -INFINITY;
                     mx = fmaxf(mx, s[i][j]);
                 }
@@ -206,7 +214,7 @@ simt_fwd_kernel(const T* __restrict__ q, const T* __restrict__ k0, const T* __re
 #pragma unroll
                 for (int e = 0; e < Cols<D>::N; ++e) o[i][e] *= corr;
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
+                for (int j = 0; j < J; ++j) {
                     const float p = expf(s[i][j] - m_new);
                     l[i] += p;
                     sm.p.v[r0 + i][tx + 16 * j] = p;
@@ -232,11 +240,11 @@ simt_fwd_kernel(const T* __restrict__ q, const T* __restrict__ k0, const T* __re
 // ---------------------------------------------------------------------------------------------
 // delta_i = sum_d dO_id * O_id, two threads per row
 template <typename T, int D>
-__global__ void __launch_bounds__(THREADS)
+__global__ void __launch_bounds__(DELTA_THREADS)
 simt_delta_kernel(const T* __restrict__ out, const T* __restrict__ dout, float* __restrict__ delta,
                   size_t n_rows) {
     constexpr int DH = D / 2;          // dimensions per thread
-    const size_t row = (size_t)blockIdx.x * (THREADS / 2) + (threadIdx.x >> 1);
+    const size_t row = (size_t)blockIdx.x * (DELTA_THREADS / 2) + (threadIdx.x >> 1);
     const int half = threadIdx.x & 1;
     float acc = 0.f;
     if (row < n_rows) {
@@ -256,20 +264,21 @@ simt_delta_kernel(const T* __restrict__ out, const T* __restrict__ dout, float* 
 // Backward: a tile's first block owns it as a key tile (dK, dV over the queries that see it), its second as a query tile
 // (dQ over its keys); one launch, so that both kinds fill the chip together.  Each result has one owner that
 // adds in a fixed order: the gradients are bit-reproducible.
-template <int D> struct BwdSmem { RowTile<D> a, b, x, y; SquareTile p; float lse[TR], delta[TR]; };
+template <int D, int TR> struct BwdSmem { RowTile<D, TR> a, b, x, y; SquareTile<TR> p; float lse[TR], delta[TR]; };
 
-template <typename T, int D>
-__global__ void __launch_bounds__(THREADS)
+template <typename T, int D, int TR>
+__global__ void __launch_bounds__(2 * TR)
 simt_bwd_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
                 const T* __restrict__ dout, const float* __restrict__ lse, const float* __restrict__ delta,
                 T* __restrict__ dq, T* __restrict__ dk, T* __restrict__ dv,
                 const __grid_constant__ ScaleTable st, int n_heads, int L, float scale) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    BwdSmem<D>& sm = *reinterpret_cast<BwdSmem<D>*>(smem_raw);
+    BwdSmem<D, TR>& sm = *reinterpret_cast<BwdSmem<D, TR>*>(smem_raw);
+    constexpr int J = TR / 16;
     const int unit = blockIdx.x / n_heads;
     const size_t head = (size_t)(blockIdx.x - unit * n_heads) * L;
     const bool keys = (unit & 1) == 0;                      // the block owns a key tile
-    const TileRows tile = tile_rows(st, unit >> 1);
+    const TileRows tile = tile_rows<TR>(st, unit >> 1);
     const int tx = threadIdx.x & 15, r0 = (threadIdx.x >> 4) * 8;
     const bool live = (threadIdx.x >> 5) * 16 < tile.n;     // the warp has rows of the tile
     // Own rows a, b against partner rows x, y: keys own K, V and walk Q, dO; queries own Q, dO and walk K, V.
@@ -308,12 +317,12 @@ simt_bwd_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
         }
         __syncthreads();
         if (!live) continue;
-        float s[8][4], dp[8][4];
+        float s[8][J], dp[8][J];
         product_nt(sm.a, sm.x, r0, tx, s);
 #pragma unroll
         for (int i = 0; i < 8; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < J; ++j) {
                 const int c = tx + 16 * j;
                 s[i][j] = c < n ? expf(s[i][j] * scale - (keys ? sm.lse[c] : row_lse[i])) : 0.f;
             }
@@ -321,7 +330,7 @@ simt_bwd_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
 #pragma unroll
             for (int i = 0; i < 8; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) sm.p.v[r0 + i][tx + 16 * j] = s[i][j];
+                for (int j = 0; j < J; ++j) sm.p.v[r0 + i][tx + 16 * j] = s[i][j];
             __syncwarp();                     // a row of P is written and read by the same 16 lanes
             product_nn(sm.p, sm.y, r0, tx, (n + 3) & ~3, acc2);
             __syncwarp();
@@ -330,7 +339,7 @@ simt_bwd_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
 #pragma unroll
         for (int i = 0; i < 8; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < J; ++j) {
                 const int c = tx + 16 * j;
                 sm.p.v[r0 + i][c] = s[i][j] * (dp[i][j] - (keys ? sm.delta[c] : row_delta[i]));
             }
@@ -350,22 +359,42 @@ simt_bwd_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
 // ---------------------------------------------------------------------------------------------
 // Launchers
 
-static int count_tiles(const ScaleTable& st) {
+static int count_tiles(const ScaleTable& st, int tile) {
     int n = 0;
-    for (int s = 0; s < st.n_scales; ++s) n += (st.start[s + 1] - st.start[s] + TR - 1) / TR;
+    for (int s = 0; s < st.n_scales; ++s) n += (st.start[s + 1] - st.start[s] + tile - 1) / tile;
     return n;
+}
+
+// Height of a call's tiles.  A block of 64 rows of which a scale fills one to sixteen spends its time on rows that are not
+// there, and its 53 to 153 KB of shared memory keep an SM at one to four blocks; a block of 16 rows is one warp in 14 to 34 KB.
+// us with 64 and 16 rows: fp32 forward + backward of sides (1, 2), 960 heads 152 and 39, of (1, 2, 3, 4) 312 and 80; bf16
+// D = 128 (1, 2, 3), 256 heads 256 and 45; fp32 step 1 -> 2, 1536 heads 41 and 12.  At 17 to 36 rows the many products
+// per load of a high tile count for more until the chip is full: (1, 2, 4, 6) 4 heads 28.7 and 39, 64 heads 41 and 39, 512
+// heads 207 and 115; (5, 6) 64 heads 37 and 43, 512 heads 155 and 127.  Beyond that the high tiles win at any number of heads
+// ((7, 8), 512 heads 252 and 319).
+static int tile_height(const ScaleTable& st, int BH, int n_prev) {
+    int rows = n_prev;                  // inference step: the previous scale, walked as far as the current one
+    for (int s = 0; s < st.n_scales; ++s) rows = std::max(rows, st.start[s + 1] - st.start[s]);
+    return rows <= 16 || (rows <= 36 && (long long)count_tiles(st, 64) * BH >= 512) ? 16 : 64;
+}
+
+template <typename T, int D, int TR>
+static cudaError_t simt_fwd_tiles(const T* q, const T* k0, const T* v0, const T* k1, const T* v1, T* out, float* lse, int BH,
+                                const ScaleTable& st, int n_q, int n0, int n1, int dense, float scale, cudaStream_t stream) {
+    static SmemOptIn opt_in;
+    const cudaError_t e = opt_in((const void*)simt_fwd_kernel<T, D, TR>, sizeof(FwdSmem<D, TR>));
+    if (e != cudaSuccess) return e;
+    simt_fwd_kernel<T, D, TR><<<(unsigned)count_tiles(st, TR) * BH, 2 * TR, sizeof(FwdSmem<D, TR>), stream>>>(q, k0, v0, k1, v1, out, lse, st, BH,
+                                                                                                           n_q, n0, n1, dense, scale);
+    count_launch(1);
+    return cudaGetLastError();
 }
 
 template <typename T, int D>
 static cudaError_t simt_fwd_any(const T* q, const T* k0, const T* v0, const T* k1, const T* v1, T* out, float* lse, int BH,
                                 const ScaleTable& st, int n_q, int n0, int n1, int dense, float scale, cudaStream_t stream) {
-    static SmemOptIn opt_in;
-    const cudaError_t e = opt_in((const void*)simt_fwd_kernel<T, D>, sizeof(FwdSmem<D>));
-    if (e != cudaSuccess) return e;
-    simt_fwd_kernel<T, D><<<(unsigned)count_tiles(st) * BH, THREADS, sizeof(FwdSmem<D>), stream>>>(q, k0, v0, k1, v1, out, lse, st, BH, n_q,
-                                                                                                 n0, n1, dense, scale);
-    count_launch(1);
-    return cudaGetLastError();
+    return tile_height(st, BH, dense ? n0 : 0) == 16 ? simt_fwd_tiles<T, D, 16>(q, k0, v0, k1, v1, out, lse, BH, st, n_q, n0, n1, dense, scale, stream)
+                                                     : simt_fwd_tiles<T, D, 64>(q, k0, v0, k1, v1, out, lse, BH, st, n_q, n0, n1, dense, scale, stream);
 }
 
 template <typename T, int D>
@@ -387,20 +416,29 @@ static cudaError_t simt_scale_step_d(const T* q, const T* k_prev, const T* v_pre
     return simt_fwd_any<T, D>(q, k_cur, v_cur, nullptr, nullptr, out, lse, BH, st, n_cur, n_cur, 0, 1, scale, stream);
 }
 
+template <typename T, int D, int TR>
+static cudaError_t simt_bwd_tiles(const T* q, const T* k, const T* v, const float* lse, const T* dout, T* dq, T* dk, T* dv,
+                                  const float* delta, int BH, const ScaleTable& st, float scale, cudaStream_t stream) {
+    static SmemOptIn opt_in;
+    const cudaError_t e = opt_in((const void*)simt_bwd_kernel<T, D, TR>, sizeof(BwdSmem<D, TR>));
+    if (e != cudaSuccess) return e;
+    simt_bwd_kernel<T, D, TR><<<2u * count_tiles(st, TR) * BH, 2 * TR, sizeof(BwdSmem<D, TR>), stream>>>(q, k, v, dout, lse, delta, dq, dk, dv, st, BH,
+                                                                                                      st.start[st.n_scales], scale);
+    return cudaGetLastError();
+}
+
 template <typename T, int D>
 static cudaError_t simt_bwd_d(const T* q, const T* k, const T* v, const T* out, const float* lse, const T* dout,
                               T* dq, T* dk, T* dv, float* delta, int BH, const ScaleTable& st, float scale,
                               cudaStream_t stream) {
-    const int L = st.start[st.n_scales];
-    const size_t n_rows = (size_t)BH * L;
-    static SmemOptIn opt_in;
-    const cudaError_t e = opt_in((const void*)simt_bwd_kernel<T, D>, sizeof(BwdSmem<D>));
-    if (e != cudaSuccess) return e;
-    simt_delta_kernel<T, D><<<(unsigned)((n_rows + THREADS / 2 - 1) / (THREADS / 2)), THREADS, 0, stream>>>(out, dout, delta, n_rows);
-    simt_bwd_kernel<T, D><<<2u * count_tiles(st) * BH, THREADS, sizeof(BwdSmem<D>), stream>>>(q, k, v, dout, lse, delta, dq, dk, dv, st, BH, L,
-                                                                                            scale);
-    count_launch(2);
-    return cudaGetLastError();
+    const size_t n_rows = (size_t)BH * st.start[st.n_scales];
+    simt_delta_kernel<T, D><<<(unsigned)((n_rows + DELTA_THREADS / 2 - 1) / (DELTA_THREADS / 2)), DELTA_THREADS, 0, stream>>>(out, dout, delta, n_rows);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess)
+        e = tile_height(st, BH, 0) == 16 ? simt_bwd_tiles<T, D, 16>(q, k, v, lse, dout, dq, dk, dv, delta, BH, st, scale, stream)
+                                         : simt_bwd_tiles<T, D, 64>(q, k, v, lse, dout, dq, dk, dv, delta, BH, st, scale, stream);
+    if (e == cudaSuccess) count_launch(2);
+    return e;
 }
 
 // The public launchers pick the instantiation for the head dimension (32, 64 or 128; checked by the caller).

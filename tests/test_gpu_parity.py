@@ -170,6 +170,24 @@ def test_other_head_dimensions_through_the_plain_kernels(sides, dtype, D):
     _no_device_error()
 
 
+@pytest.mark.parametrize("D", [32, 64, 128])
+@pytest.mark.parametrize("sides, B, H", [((1,), 1, 3), ((4, 4), 2, 3), ((2, 2, 2, 2, 2, 2), 1, 5), ((4, 1, 3), 3, 1), ((1, 5), 1, 3), ((6, 5), 1, 3),
+                                         ((6, 5), 4, 64), ((1, 2, 4, 6), 2, 64), ((6, 7), 4, 64), ((3, 4, 9), 1, 2)])
+def test_plain_kernels_low_and_high_tiles(sides, B, H, D):
+    """fp32 at both tile heights of the plain kernels: scales of at most 16 tokens (16 rows), of 17 to 36 with few heads
+    (64) and with many (16), and larger ones; forward, backward and the inference step of the last scale."""
+    wl = _Wl(sides, B=B, H=H, D=D)
+    wl.softmax_scale = D ** -0.5
+    _run_training(wl, torch.float32)
+    q, kp, vp, kc, vc = scale_step_inputs(wl, len(sides) - 1, 0, bf16=False)
+    dev = [None if x is None else to_device(x, B, H, torch.float32) for x in (q, kp, vp, kc, vc)]
+    out, lse = hmar.hmar_attn_scale_step(*dev, sides[-2] if len(sides) > 1 else 0, sides[-1], wl.softmax_scale)
+    ref_out, ref_lse = orc.scale_step(q, kp, vp, kc, vc, wl.softmax_scale)
+    _assert_close("step out", out, ref_out, True)
+    _assert_lse(lse, ref_lse, True)
+    _no_device_error()
+
+
 def test_large_logits_exercise_running_max():
     # q scaled by 8: logits ~ N(0, 8^2), the running maximum moves often and P is peaked
     _run_training(_Wl((1, 2, 3, 4, 6, 9, 13, 18)), torch.bfloat16, gain=8.0)
