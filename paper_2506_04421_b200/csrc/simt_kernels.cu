@@ -238,26 +238,27 @@ simt_fwd_kernel(const T* __restrict__ q, const T* __restrict__ k0, const T* __re
 }
 
 // ---------------------------------------------------------------------------------------------
-// delta_i = sum_d dO_id * O_id, two threads per row
+// delta_i = sum_d dO_id * O_id, in the very order in which product_nt sums a dot product: where a query has a single key,
+// O is that key's V and dP - delta is exactly zero.  D / 8 threads per row, eight products each.
 template <typename T, int D>
 __global__ void __launch_bounds__(DELTA_THREADS)
 simt_delta_kernel(const T* __restrict__ out, const T* __restrict__ dout, float* __restrict__ delta,
                   size_t n_rows) {
-    constexpr int DH = D / 2;          // dimensions per thread
-    const size_t row = (size_t)blockIdx.x * (DELTA_THREADS / 2) + (threadIdx.x >> 1);
-    const int half = threadIdx.x & 1;
-    float acc = 0.f;
+    constexpr int PARTS = D / 8;
+    const size_t row = ((size_t)blockIdx.x * DELTA_THREADS + threadIdx.x) / PARTS;
+    const int part = threadIdx.x % PARTS;
+    float t = 0.f;
     if (row < n_rows) {
-        const T* a = out + row * D + half * DH;
-        const T* b = dout + row * D + half * DH;
-#pragma unroll
-        for (int d = 0; d < DH; d += 4) {
-            const float4 x = load4(a + d), y = load4(b + d);
-            acc = fmaf(x.w, y.w, fmaf(x.z, y.z, fmaf(x.y, y.y, fmaf(x.x, y.x, acc))));
-        }
+        const T* a = dout + row * D + part * 8;
+        const T* b = out + row * D + part * 8;
+        const float4 a0 = load4(a), a1 = load4(a + 4), b0 = load4(b), b1 = load4(b + 4);
+        t = fmaf(a0.w, b0.w, fmaf(a0.z, b0.z, fmaf(a0.y, b0.y, a0.x * b0.x)));
+        t = fmaf(a1.w, b1.w, fmaf(a1.z, b1.z, fmaf(a1.y, b1.y, fmaf(a1.x, b1.x, t))));
     }
-    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-    if (row < n_rows && half == 0) delta[row] = acc;
+    float acc = 0.f;
+#pragma unroll
+    for (int c = 0; c < PARTS; ++c) acc += __shfl_sync(0xffffffffu, t, c, PARTS);
+    if (row < n_rows && part == 0) delta[row] = acc;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -432,7 +433,8 @@ static cudaError_t simt_bwd_d(const T* q, const T* k, const T* v, const T* out, 
                               T* dq, T* dk, T* dv, float* delta, int BH, const ScaleTable& st, float scale,
                               cudaStream_t stream) {
     const size_t n_rows = (size_t)BH * st.start[st.n_scales];
-    simt_delta_kernel<T, D><<<(unsigned)((n_rows + DELTA_THREADS / 2 - 1) / (DELTA_THREADS / 2)), DELTA_THREADS, 0, stream>>>(out, dout, delta, n_rows);
+    constexpr int ROWS = DELTA_THREADS / (D / 8);
+    simt_delta_kernel<T, D><<<(unsigned)((n_rows + ROWS - 1) / ROWS), DELTA_THREADS, 0, stream>>>(out, dout, delta, n_rows);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess)
         e = tile_height(st, BH, 0) == 16 ? simt_bwd_tiles<T, D, 16>(q, k, v, lse, dout, dq, dk, dv, delta, BH, st, scale, stream)

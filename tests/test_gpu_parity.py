@@ -188,6 +188,21 @@ def test_plain_kernels_low_and_high_tiles(sides, B, H, D):
     _no_device_error()
 
 
+@pytest.mark.parametrize("D, dtype", [(32, torch.bfloat16), (32, torch.float32), (64, torch.float32), (128, torch.float32), (128, torch.bfloat16)])
+@pytest.mark.parametrize("sides, H", [((1, 2), 3), ((1, 9), 2), ((1, 3), 700)])
+def test_plain_backward_of_a_query_with_one_key_is_exactly_zero(sides, H, D, dtype):
+    """The first token sees itself alone: P = 1 and O = V whatever Q and K are, so its dQ is zero, and under the
+    block-diagonal mask its dK too; not merely small."""
+    L = sum(s * s for s in sides)
+    q, k, v, do = torch.randn((4, 1, H, L, D), generator=torch.Generator().manual_seed(H)).to("cuda", dtype)
+    for window in (hmar.HMAR_WINDOW_MARKOV, hmar.HMAR_WINDOW_SELF):
+        out, lse = hmar.hmar_attn_fwd(q, k, v, sides, D ** -0.5, window=window)
+        assert torch.equal(out[:, :, 0], v[:, :, 0])
+        dq, dk, _ = hmar.hmar_attn_bwd(q, k, v, out, lse, do, sides, D ** -0.5, window=window)
+        assert not dq[:, :, 0].any()
+        assert window == hmar.HMAR_WINDOW_MARKOV or not dk[:, :, 0].any()
+
+
 def test_large_logits_exercise_running_max():
     # q scaled by 8: logits ~ N(0, 8^2), the running maximum moves often and P is peaked
     _run_training(_Wl((1, 2, 3, 4, 6, 9, 13, 18)), torch.bfloat16, gain=8.0)
