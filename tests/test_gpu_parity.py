@@ -726,6 +726,25 @@ def test_recon_accumulate_strips_and_equal_sizes(side, out_side, C):
     assert all(intact() for intact in guards)
 
 
+@pytest.mark.parametrize("side,out_side,C", [(33, 33, 5), (36, 64, 5), (47, 63, 9), (33, 64, 1), (64, 64, 7), (40, 41, 13)])
+def test_recon_accumulate_strips_with_a_channel_group_cut_short(side, out_side, C):
+    """Maps past 32 x 32 whose channels are no multiple of four: the strips' gather takes one value at a time, four of a
+    thread's loads together, with a last round that is not full.  1e-5 relative, as above."""
+    rng = np.random.default_rng(1000 * side + 10 * out_side + C)
+    B, V = 3, 90
+    codebook = rng.standard_normal((V, C)).astype(np.float32)
+    new = rng.integers(0, V, (B, side, side)).astype(np.int32)
+    x0 = rng.standard_normal((B, C, out_side, out_side)).astype(np.float32)
+    guards = []
+    xhat = _guarded(x0.shape, torch.float32, guards)
+    xhat.copy_(torch.from_numpy(x0))
+    hmar.hmar_recon_accumulate(xhat, torch.from_numpy(codebook).cuda(), torch.from_numpy(new).cuda())
+    ref = orc.recon_accumulate(x0, codebook, new, out_side)
+    err = np.abs(xhat.double().cpu().numpy() - ref)
+    assert err.max() <= 1e-5 * max(1.0, np.abs(ref).max()), f"max abs err {err.max():.3e}"
+    assert all(intact() for intact in guards)
+
+
 def test_recon_accumulate_codebook_off_16_byte_alignment():
     """A codebook whose base address is not a multiple of 16 bytes takes the staged kernel's one-value-at-a-time
     gather; same result as the oracle."""
