@@ -113,6 +113,7 @@ def _sides_array(sides):
 
 def _sides(side_lens):
     """(C array, length) of a side list; the arrays are read-only and shared by all calls with equal lists."""
+    len(side_lens)                         # a generator has none, and is refused: a second call would find it used up
     return _sides_array(tuple(map(int, side_lens)))
 
 

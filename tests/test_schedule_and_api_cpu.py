@@ -283,6 +283,9 @@ def test_side_lists_have_a_length():
     q = _cuda_tensor_without_memory(1, 1, 4, 64, dtype=torch.bfloat16)
     with pytest.raises(TypeError):
         hmar.hmar_attn_fwd(q, q, q, (s for s in (2,)), 0.125, out=q, lse=q)
+    with pytest.raises(TypeError):
+        hmar.hmar_schedule_tiles((s for s in (2,)), 0)
+    assert hmar.hmar_schedule_tiles(np.array([2, 3]), 0) == hmar.hmar_schedule_tiles([2, 3], 0)
 
 
 def test_softmax_scale_is_whatever_float_takes():
