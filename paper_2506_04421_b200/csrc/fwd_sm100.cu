@@ -513,8 +513,6 @@ cudaError_t launch_selftest_wait(int* status, cudaStream_t stream) {
     return cudaGetLastError();
 }
 
-constexpr size_t kGroupBytes = 128000000;      // L2 holds 126 MiB
-
 size_t fwd_tc_smem_bytes() { return sizeof(SharedStorage); }
 
 cudaError_t launch_fwd_tc(const CUtensorMap& q, const CUtensorMap& k0, const CUtensorMap& v0, const CUtensorMap& k1,
@@ -533,7 +531,7 @@ cudaError_t launch_fwd_tc(const CUtensorMap& q, const CUtensorMap& k0, const CUt
     // heads and L = 395 768 heads equal.  Groups of 48 MB are 1 to 4 % slower than these, of 96 or 160 MB equal.
     // The tiles of an inference step all cost the same, and stay head by head (groups: 0 to 15 % slower).
     FwdArgs a = args;
-    const size_t groups = (BH * args.head_bytes + kGroupBytes - 1) / kGroupBytes;
+    const size_t groups = (BH * args.head_bytes + kL2Bytes - 1) / kL2Bytes;
     a.n_heads = BH;
     a.group_heads = (int)((BH + groups - 1) / groups);
     {

@@ -72,7 +72,7 @@ inline int bwd_plain_permille(const BwdWork* work, int n) {
     return total > 0 ? (int)(plain * 1000 / total) : 1000;
 }
 
-constexpr size_t kL2Bytes = 126u << 20;
+constexpr size_t kL2Bytes = 126u << 20;      // L2 of the one part this library is built for
 
 // Whether the backward's items go head by head instead of class by class.  Class by class a head's rows are read once per
 // class.  Where its items are short (a mean of fewer than four steps) and the tensors do not stay in L2, that costs more than
