@@ -34,7 +34,8 @@
 // two warpgroups lower theirs (setmaxnreg) within the same total.
 // The SMs of a cluster share the instruction cache behind the small per-partition one, and this kernel's
 // speed depends on how much code it streams through it: changes that only add instructions (more unrolled
-// variants, code that never runs) have cost up to a tenth of the time, so variants are kept few.
+// variants, code that never runs) have cost up to a tenth of the time, so variants are kept few.  (94 to 96 % of the
+// requests hit now, 67 to 92 % while each wait carried a timer and a report of its own.)
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -152,7 +153,7 @@ __device__ __forceinline__ void load_swizzled_row(const uint8_t* tile, int r, ui
 // MODE 0: all rows see all columns.
 // ROLLED: the two halves of the rows are iterations of a loop and not two copies of the code.  Less code, but the compiler
 // no longer mixes one half's stores with the next half's loads: the instantiation for partial and packed tiles is bound
-// by instruction fetch and gains (L = 680: 332 -> 295 us), the one for full tiles loses (L = 2240: 832 -> 849 us).
+// by the code at its many item boundaries and gains (L = 680: 332 -> 295 us), the one for full tiles loses (L = 2240: 832 -> 849 us).
 template <int MODE, bool ROLLED>
 __device__ __forceinline__ void softmax_grad_half(uint32_t lane_base, int cbase, const uint64_t (&nls)[8], const uint64_t (&nde)[8],
                                                   float sl2, const int (&c_lo)[4], const int (&c_hi)[4], uint8_t* ds_tile,
@@ -206,9 +207,8 @@ __device__ __forceinline__ void softmax_grad_half(uint32_t lane_base, int cbase,
 // benchmarks run: the extra address arithmetic and code of the strided one cost it a tenth of its speed).
 // ONE_MASK: every tile goes through the variant of the softmax-gradient code with per-element bounds, so that the
 // block's code holds one variant instead of three.  It is the instantiation for side lists whose tiles are mostly
-// partial or packed (L = 680: 11 % faster, a third of the instruction-cache requests of the three-variant code
-// miss there); where most steps belong to full tiles the plain variant's shorter arithmetic wins (L = 2240: the
-// one-variant code is 4 % slower).
+// partial or packed (L = 680, 960 heads: 258 us, 322 with three variants); where most steps belong to full tiles the
+// plain variant's shorter arithmetic wins (L = 2240, 384 heads: 879 us, 740 with three).  See kOneMaskBelowPermille.
 template <bool STRIDED, bool ONE_MASK>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -887,7 +887,10 @@ static int sm_count() {
 }
 
 // Side lists with fewer than this share (in thousandths) of their steps in full tiles run the one-variant
-// instantiation (L = 680 has 42 %, L = 2240 has 82 %).
+// instantiation.  Main kernel, one variant / three: 0.71 at 200 (L = 399, 768 heads), 0.80 and 0.97 at 421 (L = 680, 960 and
+// 128 heads), 1.07 at 500 (L = 900, four scales of 15), 1.04 at 512 (L = 1060), 1.13 at 709 and 714, 1.15 at 824
+// (L = 2240, 96 heads), 1.22 at 973.  The line was drawn before both instantiations became faster; the crossing is now
+// between 421 and 500.  (Twelve scales of 11 have no full tile and 1.04: their tiles are all cut short alike.)
 constexpr int kOneMaskBelowPermille = 600;
 
 template <bool STRIDED>

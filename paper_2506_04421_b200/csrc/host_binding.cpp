@@ -1,7 +1,9 @@
 // The Python side of the calls, in native code: checks of the tensors, allocation of the results, the stream and the call
-// of the C entry point.  A call of a small scale is host time only.  In Python (tensor attributes, allocations through the
-// interpreter, a ctypes call of a dozen arguments) it took 9.0 us for a step and 7.2 to 7.8 for the sampler's two calls;
-// here 6.1 and 4.1, of which the launch is 2.5 and a step's two allocations 2.3.
+// of the C entry point.  In Python (tensor attributes, allocations through the interpreter, a ctypes call of a dozen
+// arguments) a call of a small scale was host time only: 9.0 us for a step and 7.2 to 7.8 for the sampler's two calls.
+// Here the host needs 5.1 us for a step without LSE, 6.1 with it, 3.7 where both outputs are given (an allocation is 1.3
+// and the rest mostly the launch), 2.8 for an accumulation; the GPU needs 3.4 to 3.8 in a graph, and takes plain
+// launches in a row every 5.2 to 6.2.
 //
 // The module holds no reference to the library: bind() takes the handle of the one the package loaded.  Every function
 // returns its results, or the entry point's status as an int where that is not HMAR_OK.
