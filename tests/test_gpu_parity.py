@@ -658,9 +658,10 @@ def test_repeat_calls_are_stable():
 @pytest.mark.parametrize("masked", [False, True])
 def test_recon_accumulate_matches_oracle(side, out_side, B, C, V, masked):
     """The sampler's neighbour step (Alg. 2 lines 7-8 with the sub-step's token selection, Sec. 4.2) on a synthetic
-    codebook: fp32 on the GPU against the fp64 oracle, and the selected token map bit for bit.  Maps of at most
-    32 x 32 tokens and reconstructions of at most 64 x 64 take the staged kernel (also with more than 32 channels,
-    and with more than 32 output columns), the 40 x 40 map and the 80 x 80 reconstruction the plain one."""
+    codebook: fp32 on the GPU against the fp64 oracle, and the selected token map bit for bit.
+    Reconstructions of at most 64 x 64 take the staged kernel (also with more than 32 channels, with more than 32
+    output columns and, in strips, the 40 x 40 map), equal sizes the one without interpolation, the 80 x 80
+    reconstruction the plain one."""
     rng = np.random.default_rng(1000 * side + out_side + int(masked))
     codebook = rng.standard_normal((V, C)).astype(np.float32)
     old = rng.integers(0, V, (B, side, side)).astype(np.int32)
