@@ -738,12 +738,22 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             for (int i = 0; i < 4; ++i) {
                 const int rr = quarter * 32 + (i >> 1) * 16 + (lane >> 2) + (i & 1) * 8;
                 qlo[i] = w.q_begin; qhi[i] = w.q_end;
-                if (tile_masked) {
-                    if (rr >= w.row_count) { qlo[i] = 0; qhi[i] = 0; }
-                    else if (!w.uniform()) {
-                        const int sc = scale_of_row(args.st, w.row_begin + rr);
-                        qlo[i] = args.st.start[first_query_scale(args.st.window, sc)];
-                        qhi[i] = args.st.start[last_query_scale(args.st.window, sc, args.st.n_scales) + 1];
+                if (tile_masked && rr >= w.row_count) { qlo[i] = 0; qhi[i] = 0; }
+            }
+            if (!w.uniform()) {
+                // Scale by scale and not row by row: the table lies in constant memory, where lanes that read different
+                // entries are served one after the other (a packed tile's search took 3 000 clocks at L = 680; 960 heads
+                // 346.0 -> 341.3 us, 128 heads 60.7 -> 59.3).
+                for (int s = 0; s < args.st.n_scales; ++s) {
+                    const int begin = args.st.start[s] - w.row_begin, end = args.st.start[s + 1] - w.row_begin;
+                    if (end <= 0) continue;
+                    if (begin >= w.row_count) break;
+                    const int first = args.st.start[first_query_scale(args.st.window, s)];
+                    const int last = args.st.start[last_query_scale(args.st.window, s, args.st.n_scales) + 1];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int rr = quarter * 32 + (i >> 1) * 16 + (lane >> 2) + (i & 1) * 8;
+                        if (rr >= begin && rr < end && rr < w.row_count) { qlo[i] = first; qhi[i] = last; }
                     }
                 }
             }
