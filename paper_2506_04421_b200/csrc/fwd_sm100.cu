@@ -119,17 +119,17 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     }
     // ---- which tile of which head
     int bh, wi;
+    const int group = args.by_group((int)blockIdx.x);
     if (args.work != nullptr) {
-        const int group = blockIdx.x / (args.group_heads * args.n_work);
-        const int first_head = group * args.group_heads, in_group = blockIdx.x - first_head * args.n_work;
-        const int heads = min(args.group_heads, args.n_heads - first_head);
-        wi = in_group / heads;
-        bh = first_head + in_group - wi * heads;
+        const int first_head = group * args.group_heads, in_group = (int)blockIdx.x - first_head * args.n_work;
+        const bool whole = first_head + args.group_heads <= args.n_heads;
+        wi = whole ? args.by_group_heads(in_group) : args.by_last_heads(in_group);
+        bh = first_head + in_group - wi * (whole ? args.group_heads : args.n_heads - first_head);
     } else {
-        bh = blockIdx.x / args.n_work;
-        wi = blockIdx.x - bh * args.n_work;
+        bh = group;
+        wi = (int)blockIdx.x - bh * args.n_work;
     }
-    const int batch = bh / args.heads_per_batch, head = bh - batch * args.heads_per_batch;
+    const int batch = args.by_batch(bh), head = bh - batch * args.heads_per_batch;
     FwdWork w;
     if (args.work != nullptr) {
         w = args.work[wi];
@@ -534,6 +534,10 @@ cudaError_t launch_fwd_tc(const CUtensorMap& q, const CUtensorMap& k0, const CUt
     const size_t groups = (BH * args.head_bytes + kL2Bytes - 1) / kL2Bytes;
     a.n_heads = BH;
     a.group_heads = (int)((BH + groups - 1) / groups);
+    a.by_group = FastDiv(args.work != nullptr ? (uint32_t)a.group_heads * (uint32_t)a.n_work : (uint32_t)a.n_work);
+    a.by_group_heads = FastDiv((uint32_t)a.group_heads);
+    a.by_last_heads = FastDiv((uint32_t)((BH - 1) % a.group_heads + 1));
+    a.by_batch = FastDiv((uint32_t)a.heads_per_batch);
     {
         KernelTimer timer(args.work != nullptr ? "hmar_fwd_tc_kernel" : "hmar_fwd_tc_kernel/scale_step", stream);
         const cudaError_t launched = launch_overlapped(hmar_fwd_tc_kernel, grid, NUM_THREADS, smem, stream, q, k0, v0, k1, v1, a);

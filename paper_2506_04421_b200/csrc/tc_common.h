@@ -18,6 +18,26 @@ struct FwdWork {
     int32_t pad;
 };
 
+// Division of numbers below 2^31 by a number that the host knows: q = (hi(n * mul) + n) >> shift with mul = 2^32 * (2^shift / d - 1)
+// rounded up and shift = ceil(log2(d)) (Granlund and Montgomery, "Division by invariant integers using multiplication").
+// A division by a variable is some forty instructions, and every block of the forward began with three of them, in all of its
+// warps: 1 100 clocks of a block's 11 000 to 69 000.  L = 680 960 heads 127 -> 121 us, L = 2240 384 heads 346 -> 338, L = 384 128
+// heads 17.7 -> 16.6, inference step 13 -> 18 1536 heads 143 -> 139, 24 -> 32 384 heads 224 -> 219.5.
+struct FastDiv {
+    uint32_t mul = 0, shift = 0;
+    FastDiv() = default;
+    constexpr explicit FastDiv(uint32_t d) {
+        while ((1ull << shift) < d) ++shift;
+        mul = (uint32_t)(((1ull << 32) * ((1ull << shift) - d) + d - 1) / d);
+    }
+    HMAR_HD constexpr int operator()(int n) const {
+        return (int)(((uint32_t)(((uint64_t)(uint32_t)n * mul) >> 32) + (uint32_t)n) >> shift);
+    }
+};
+static_assert(FastDiv(1)(0x7fffffff) == 0x7fffffff && FastDiv(2)(0x7fffffff) == 0x3fffffff && FastDiv(3)(0x7ffffffd) == 0x2aaaaaa9 &&
+              FastDiv(7)(0x7ffffffe) == 306783378 && FastDiv(7)(306783378 * 7 - 1) == 306783377 && FastDiv(641)(640) == 0 &&
+              FastDiv(0x7fffffff)(0x7fffffff) == 1 && FastDiv(0x7fffffff)(0x7ffffffe) == 0, "division at the ends of its range");
+
 struct FwdArgs {
     const FwdWork* work;     // n_work tiles per head; nullptr = inference step (tiles derived in-kernel)
     int n_work;
@@ -26,6 +46,8 @@ struct FwdArgs {
     int n_heads;             // set by the launcher, as group_heads: the blocks go group by group of this many heads, and
     int group_heads;         // tile by tile over the heads of a group
     int heads_per_batch;     // H: head bh is head bh % H of batch bh / H (the tensor maps are 4-D: D, rows, H, B)
+    FastDiv by_group, by_group_heads, by_last_heads, by_batch;      // set by the launcher: group_heads * n_work (an inference step: n_work),
+                             // heads of a group, heads of the last group, heads_per_batch
     long long out_row_stride, out_head_stride, out_batch_stride;   // of `out`, in elements (lse is always [B*H, rows])
     long long out_extent, lse_extent;   // elements reachable through out / lse (read by the checking build only)
     int n0, n1;              // inference step: rows of the previous / current scale's keys

@@ -784,6 +784,21 @@ def test_last_query_tiles_with_one_to_four_softmax_warps(side):
     _no_device_error()
 
 
+@pytest.mark.parametrize("B, H", [(1, 1111), (101, 11)])
+def test_forward_in_groups_of_heads_with_a_smaller_last_group(B, H):
+    """Q, K, V of 1111 heads are more than two L2s: three groups of heads, the last one smaller.  Every head's rows are those of a
+    call on that head alone, bit for bit."""
+    sides = (1, 2, 3, 4, 5, 6, 8, 10, 13, 16)
+    L = sum(s * s for s in sides)
+    g = torch.Generator(device="cuda").manual_seed(11)
+    q, k, v = (torch.randn((B, H, L, 64), generator=g, device="cuda").to(torch.bfloat16) for _ in range(3))
+    out, lse = hmar.hmar_attn_fwd(q, k, v, sides, 0.125)
+    flat = [t.view(B * H, L, 64) for t in (q, k, v, out)]
+    for head in (0, 1, 369, 370, 371, 372, 740, 741, 742, 743, 1109, 1110):
+        o1, l1 = hmar.hmar_attn_fwd(*(t[head].view(1, 1, L, 64) for t in flat[:3]), sides, 0.125)
+        assert torch.equal(o1.view(L, 64), flat[3][head]) and torch.equal(l1.view(L), lse.view(B * H, L)[head]), head
+
+
 @pytest.mark.parametrize("noalloc", [False, True])
 def test_overlapped_launches_see_what_the_calls_before_wrote(noalloc):
     """Calls in a row on the same buffers, none waited for: each launch starts while the one before it ends, and has to
