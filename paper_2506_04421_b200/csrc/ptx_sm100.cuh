@@ -280,6 +280,13 @@ __device__ __forceinline__ float ex2(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+// Bits of the columns [lo, hi) of a tile's 64, the first 32 and the others.
+__device__ __forceinline__ void visible_columns(int lo, int hi, uint32_t& first, uint32_t& others) {
+    auto below = [](int n) -> uint32_t { return n >= 32 ? 0xffffffffu : n <= 0 ? 0u : (1u << n) - 1u; };
+    first = below(hi) & ~below(lo);
+    others = below(hi - 32) & ~below(lo - 32);
+}
+
 // Packed fp32 pairs (one instruction works on two floats held in a 64-bit register).
 __device__ __forceinline__ uint64_t f32x2(float lo, float hi) {
     uint64_t r;
