@@ -165,6 +165,17 @@ __device__ __forceinline__ void softmax_grad_half(uint32_t lane_base, int cbase,
 #pragma unroll (ROLLED ? 1 : 2)
     for (int hl = 0; hl < 2; ++hl) {                    // lanes 0-15, then 16-31 of the warp's quarter
         const int lo2[2] = {hl ? c_lo[2] : c_lo[0], hl ? c_lo[3] : c_lo[1]}, hi2[2] = {hl ? c_hi[2] : c_hi[0], hl ? c_hi[3] : c_hi[1]};
+        // MODE 2: a bit per column of the half, moved so that this thread's pairs are the lowest two of each byte (bounds compared
+        // column by column: L = 680 960 heads, main kernel 253 -> 245 us, L = 384 128 heads 31.3 -> 29.2)
+        uint32_t seen[2][2];
+        if (MODE == 2) {
+#pragma unroll
+            for (int rs = 0; rs < 2; ++rs) {
+                visible_columns(lo2[rs] - cbase, hi2[rs] - cbase, seen[rs][0], seen[rs][1]);
+                seen[rs][0] >>= 2 * tq;
+                seen[rs][1] >>= 2 * tq;
+            }
+        }
         const uint32_t taddr = lane_base + ((uint32_t)(hl * 16) << 16);
         uint32_t s_buf[32], dp_buf[32];
         tmem_ld_16x256b_x8(taddr + COL_ST + cbase, s_buf);
@@ -182,9 +193,8 @@ __device__ __forceinline__ void softmax_grad_half(uint32_t lane_base, int cbase,
                                   sl2_2, nls[k]), x0, x1);
                 float p0 = ex2(x0), p1 = ex2(x1);
                 if (MODE == 2) {
-                    const int c = cbase + 8 * k + 2 * tq;
-                    p0 = (c >= lo2[rs] && c < hi2[rs]) ? p0 : 0.f;
-                    p1 = (c + 1 >= lo2[rs] && c + 1 < hi2[rs]) ? p1 : 0.f;
+                    if (!(seen[rs][k >> 2] >> (8 * (k & 3)) & 1u)) p0 = 0.f;
+                    if (!(seen[rs][k >> 2] >> (8 * (k & 3)) & 2u)) p1 = 0.f;
                 }
                 float d0, d1;
                 f32x2_split(fmul2(f32x2(p0, p1),
