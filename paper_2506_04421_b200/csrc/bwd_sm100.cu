@@ -834,11 +834,13 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 struct RowLayout {
     int L, heads_per_batch;
     long long row, head, batch;
+    FastDiv by_L, by_heads;
     template <bool STRIDED>
     __device__ __forceinline__ long long offset(size_t r) const {
         if (!STRIDED) return (long long)r * D;
-        const int bh = (int)(r / (size_t)L), l = (int)(r - (size_t)bh * L);
-        const int b = bh / heads_per_batch, h = bh - b * heads_per_batch;
+        // (a tensor of 2^31 rows of 128 bytes would be larger than the memory)
+        const int bh = by_L((int)r), l = (int)r - bh * L;
+        const int b = by_heads(bh), h = bh - b * heads_per_batch;
         return b * batch + h * head + l * row;
     }
 };
@@ -921,7 +923,7 @@ static cudaError_t launch_bwd_tc_layout(const CUtensorMap& q, const CUtensorMap&
     const size_t n_rows = (size_t)BH * args.L;
     {
         KernelTimer timer("hmar_bwd_delta_kernel", stream);
-        const RowLayout lay{args.L, args.heads_per_batch, args.od_row, args.od_head, args.od_batch};
+        const RowLayout lay{args.L, args.heads_per_batch, args.od_row, args.od_head, args.od_batch, FastDiv(args.L), FastDiv(args.heads_per_batch)};
         const cudaError_t e = launch_overlapped(hmar_bwd_delta_kernel<STRIDED>, (unsigned)((n_rows * 8 + 255) / 256), 256, 0, stream, out, dout,
                                                 args.delta_w, args.dq_acc, n_rows, lay);
         if (e != cudaSuccess) return e;
@@ -942,7 +944,7 @@ static cudaError_t launch_bwd_tc_layout(const CUtensorMap& q, const CUtensorMap&
     const size_t n8 = n_rows * D / 8;
     {
         KernelTimer timer("hmar_bwd_dq_convert_kernel", stream);
-        const RowLayout lay{args.L, args.heads_per_batch, args.g_row, args.g_head, args.g_batch};
+        const RowLayout lay{args.L, args.heads_per_batch, args.g_row, args.g_head, args.g_batch, FastDiv(args.L), FastDiv(args.heads_per_batch)};
         const cudaError_t e = launch_overlapped(hmar_bwd_dq_convert_kernel<STRIDED>, (unsigned)((n8 + 255) / 256), 256, 0, stream, args.dq_acc, dq,
                                                 args.softmax_scale, n8, lay);
         if (e != cudaSuccess) return e;
