@@ -19,7 +19,8 @@
 //   warps 8-11  per step: drain dQ_i from TMEM through a staging buffer into the fp32 accumulator with
 //               bulk tensor reductions (cp.reduce.async.bulk.tensor).  Per item: copy the next item's K
 //               and V rows into TMEM as soon as the current item's last scores are done, and write the
-//               finished dK, dV (scaled, bf16), V, dK and dV as whole rows per instruction
+//               finished dK, dV (scaled, bf16; by bulk tensor stores where a warp's 32 rows are all the tile's), V, dK and dV
+//               as whole rows per instruction
 //   warp 12     TMA producer: K per item (two buffers); Q_i, dO_i through a 3-stage ring
 //   warp 13     issues tcgen05.mma.  K and V in TMEM are the A operands of S^T = K Q_i^T and
 //               dP^T = V dO_i^T; dV += P^T dO_i and dK += dS^T Q_i read their A operand from TMEM too;
@@ -113,6 +114,12 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 __device__ __forceinline__ void tma_reduce_add_2d(const CUtensorMap* m, const void* smem_src, int c0, int c1) {
     asm volatile("cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3}], [%1];"
                  ::"l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(smem_src)), "r"(c0), "r"(c1)
+                 : "memory");
+}
+// Writes [32 rows x 64 bf16] from shared memory (128-byte swizzle) to rows c1.. of head c2 of batch c3.
+__device__ __forceinline__ void tma_store_4d(const CUtensorMap* m, const void* smem_src, int c1, int c2, int c3) {
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];"
+                 ::"l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(smem_src)), "r"(0), "r"(c1), "r"(c2), "r"(c3)
                  : "memory");
 }
 __device__ __forceinline__ void bulk_commit_group() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
@@ -223,7 +230,8 @@ template <bool STRIDED, bool ONE_MASK>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                    const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do,
-                   const __grid_constant__ CUtensorMap map_dq, const BwdArgs args) {
+                   const __grid_constant__ CUtensorMap map_dq, const __grid_constant__ CUtensorMap map_dk,
+                   const __grid_constant__ CUtensorMap map_dv, const BwdArgs args) {
     // aligned by its declaration, so that every shared-memory address is a constant of the code (one added at run time
     // costs a register in every role and about 5 % of the code); checked below
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -671,7 +679,16 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                             o.w = pack_bf16(__uint_as_float(buf[8 * t + 6]) * mul, __uint_as_float(buf[8 * t + 7]) * mul);
                             *reinterpret_cast<uint4*>(stage_row + ((((part & 1) * 4 + t) ^ (lane & 7)) << 4)) = o;
                         }
-                        if ((part & 1) == 1) {
+                        // A warp whose 32 rows are all the tile's sends them with one copy; other rows belong to another tile.
+                        // (Always with stores: packed layout, 96 heads of L = 2240, 215 -> 210 us; L = 680 960 heads 333.5 -> 331.)
+                        if ((part & 1) == 1 && quarter * 32 + 32 <= w.row_count) {
+                            fence_proxy_async_smem();
+                            __syncwarp();
+                            if (lane == 0) {
+                                tma_store_4d(part < 2 ? &map_dk : &map_dv, stage, w.row_begin + quarter * 32, w.head, w.batch);
+                                bulk_commit_group();
+                            }
+                        } else if ((part & 1) == 1) {
                             __syncwarp();
                             __nv_bfloat16* base = part < 2 ? args.dk : args.dv;
                             const int row0 = quarter * 32 + sub_row;
@@ -721,7 +738,7 @@ hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             }
             if (ok) done(item);
         }
-        if (lane == 0) bulk_wait_all();         // the staging buffer must outlive the last reduction's read
+        if (lane == 0) bulk_wait_all();         // the staging buffer must outlive the last copy's read
     } else {
         // ================================================================== compute warpgroups
         reg_inc<REGS_COMPUTE>();
@@ -917,8 +934,8 @@ constexpr int kOneMaskBelowPermille = 600;
 
 template <bool STRIDED>
 static cudaError_t launch_bwd_tc_layout(const CUtensorMap& q, const CUtensorMap& k, const CUtensorMap& v, const CUtensorMap& dout_map,
-                                        const CUtensorMap& dq_acc_map, const BwdArgs& args, const __nv_bfloat16* out,
-                                        const __nv_bfloat16* dout, __nv_bfloat16* dq, int BH, cudaStream_t stream) {
+                                        const CUtensorMap& dq_acc_map, const CUtensorMap& dk_map, const CUtensorMap& dv_map, const BwdArgs& args,
+                                        const __nv_bfloat16* out, const __nv_bfloat16* dout, __nv_bfloat16* dq, int BH, cudaStream_t stream) {
     const size_t smem = sizeof(SharedStorage);
     const size_t n_rows = (size_t)BH * args.L;
     {
@@ -938,7 +955,7 @@ static cudaError_t launch_bwd_tc_layout(const CUtensorMap& q, const CUtensorMap&
         const bool one_mask = args.plain_permille < kOneMaskBelowPermille;
         auto kernel = one_mask ? hmar_bwd_tc_kernel<STRIDED, true> : hmar_bwd_tc_kernel<STRIDED, false>;
         cudaError_t e = opt_in[one_mask]((const void*)kernel, smem);
-        if (e == cudaSuccess) e = launch_overlapped(kernel, grid, NUM_THREADS, smem, stream, q, k, v, dout_map, dq_acc_map, a);
+        if (e == cudaSuccess) e = launch_overlapped(kernel, grid, NUM_THREADS, smem, stream, q, k, v, dout_map, dq_acc_map, dk_map, dv_map, a);
         if (e != cudaSuccess) return e;
     }
     const size_t n8 = n_rows * D / 8;
@@ -954,16 +971,16 @@ static cudaError_t launch_bwd_tc_layout(const CUtensorMap& q, const CUtensorMap&
 }
 
 cudaError_t launch_bwd_tc(const CUtensorMap& q, const CUtensorMap& k, const CUtensorMap& v, const CUtensorMap& dout_map,
-                          const CUtensorMap& dq_acc_map, const BwdArgs& args, const __nv_bfloat16* out, const __nv_bfloat16* dout,
-                          __nv_bfloat16* dq, int BH, cudaStream_t stream) {
+                          const CUtensorMap& dq_acc_map, const CUtensorMap& dk_map, const CUtensorMap& dv_map, const BwdArgs& args,
+                          const __nv_bfloat16* out, const __nv_bfloat16* dout, __nv_bfloat16* dq, int BH, cudaStream_t stream) {
     // dense [BH, L, 64] everywhere: the instantiation with compile-time strides
     const long long row = D, head = (long long)args.L * D;
     const bool dense = args.in_row == row && args.od_row == row && args.g_row == row && args.in_head == head &&
                        args.od_head == head && args.g_head == head &&
                        (args.heads_per_batch == BH || (args.in_batch == args.heads_per_batch * head &&
                                                        args.od_batch == args.in_batch && args.g_batch == args.in_batch));
-    return dense ? launch_bwd_tc_layout<false>(q, k, v, dout_map, dq_acc_map, args, out, dout, dq, BH, stream)
-                 : launch_bwd_tc_layout<true>(q, k, v, dout_map, dq_acc_map, args, out, dout, dq, BH, stream);
+    return dense ? launch_bwd_tc_layout<false>(q, k, v, dout_map, dq_acc_map, dk_map, dv_map, args, out, dout, dq, BH, stream)
+                 : launch_bwd_tc_layout<true>(q, k, v, dout_map, dq_acc_map, dk_map, dv_map, args, out, dout, dq, BH, stream);
 }
 
 }  // namespace hmar

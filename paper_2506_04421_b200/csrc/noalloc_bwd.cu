@@ -65,7 +65,7 @@ static __global__ void noalloc_fill_work_kernel(const WorkChunk chunk, int first
     for (int i = threadIdx.x; i < count; i += blockDim.x) dst[first + i] = chunk.w[i];
 }
 
-bool make_rows_map_bf16(CUtensorMap* map, const void* base, int heads, int rows);
+bool make_rows_map_bf16(CUtensorMap* map, const void* base, int heads, int rows, bool gradient = false);
 bool make_dq_acc_map(CUtensorMap* map, const float* base, size_t rows);
 
 }  // namespace hmar
@@ -128,9 +128,10 @@ extern "C" int hmar_attn_bwd_noalloc(const void* q, const void* k, const void* v
     count_launch((int)((tiles.size() + kFillChunk - 1) / kFillChunk));
 
     const int BH = B * H;
-    CUtensorMap mq, mk, mv, mdo, macc;
+    CUtensorMap mq, mk, mv, mdo, macc, mdk, mdv;
     if (!make_rows_map_bf16(&mq, q, BH, (int)L) || !make_rows_map_bf16(&mk, k, BH, (int)L) ||
         !make_rows_map_bf16(&mv, v, BH, (int)L) || !make_rows_map_bf16(&mdo, dout, BH, (int)L) ||
+        !make_rows_map_bf16(&mdk, dk, BH, (int)L, true) || !make_rows_map_bf16(&mdv, dv, BH, (int)L, true) ||
         !make_dq_acc_map(&macc, reinterpret_cast<const float*>(scratch + kWorkBytes + kDeltaBytes), (size_t)BH * L))
         return HMAR_ERR_CUDA;
     BwdArgs a{};
@@ -156,6 +157,6 @@ extern "C" int hmar_attn_bwd_noalloc(const void* q, const void* k, const void* v
     a.dv = static_cast<__nv_bfloat16*>(dv);
     a.status = nullptr;
     a.st = st;
-    return launch_status(launch_bwd_tc(mq, mk, mv, mdo, macc, a, static_cast<const __nv_bfloat16*>(out),
+    return launch_status(launch_bwd_tc(mq, mk, mv, mdo, macc, mdk, mdv, a, static_cast<const __nv_bfloat16*>(out),
                                        static_cast<const __nv_bfloat16*>(dout), static_cast<__nv_bfloat16*>(dq), BH, s));
 }

@@ -41,6 +41,7 @@ static EncodeTiledFn encode_fn() {
 // 4-D map (64 elements, rows, heads, batches) with the strides of the tensor in elements; boxes of `box_rows`
 // rows of one head.  Serves the contiguous [B, H, rows, 64] layout and a packed [B, rows, 3, H, 64] one alike.
 constexpr int kFwdKeyRows = 64;      // key rows per tile of the forward kernel (its query tiles are kTileRows high)
+constexpr int kGradRows = 32;        // rows of dK, dV that a warp of the backward kernel writes at a time
 static bool make_rows_map4(CUtensorMap* map, const void* base, int batches, int heads, int rows, long long row_stride,
                            long long head_stride, long long batch_stride, int box_rows) {
     EncodeTiledFn fn = encode_fn();
@@ -302,11 +303,13 @@ static int tc_bwd_strided(const bf16* q, const bf16* k, const bf16* v, const bf1
     if (plan == nullptr) return HMAR_ERR_CUDA;
     const int L = st.start[st.n_scales];
     const int BH = B * H;
-    CUtensorMap mq, mk, mv, mdo, macc;
+    CUtensorMap mq, mk, mv, mdo, macc, mdk, mdv;
     if (!make_rows_map4(&mq, q, B, H, L, in.row, in.head, in.batch, kTileRows) ||
         !make_rows_map4(&mk, k, B, H, L, in.row, in.head, in.batch, kTileRows) ||
         !make_rows_map4(&mv, v, B, H, L, in.row, in.head, in.batch, kTileRows) ||
-        !make_rows_map4(&mdo, dout, B, H, L, od.row, od.head, od.batch, kTileRows) || !make_acc_map(&macc, dq_acc, (size_t)BH * L))
+        !make_rows_map4(&mdo, dout, B, H, L, od.row, od.head, od.batch, kTileRows) ||
+        !make_rows_map4(&mdk, dk, B, H, L, g.row, g.head, g.batch, kGradRows) ||
+        !make_rows_map4(&mdv, dv, B, H, L, g.row, g.head, g.batch, kGradRows) || !make_acc_map(&macc, dq_acc, (size_t)BH * L))
         return HMAR_ERR_CUDA;
     BwdArgs a{};
     a.work = plan->bwd_work;
@@ -351,7 +354,7 @@ static int tc_bwd_strided(const bf16* q, const bf16* k, const bf16* v, const bf1
                 }
         }
     }
-    return launch_status(launch_bwd_tc(mq, mk, mv, mdo, macc, a, out, dout, dq, BH, stream));
+    return launch_status(launch_bwd_tc(mq, mk, mv, mdo, macc, mdk, mdv, a, out, dout, dq, BH, stream));
 }
 
 // Contiguous [B*H, L, 64] tensors: one "batch" of BH heads.
@@ -373,8 +376,9 @@ int tc_bwd_packed(const bf16* qkv, const bf16* out, const float* lse, const bf16
 }
 
 // The same tensor maps for code outside this file.
-bool make_rows_map_bf16(CUtensorMap* map, const void* base, int heads, int rows) {
-    return make_rows_map4(map, base, 1, heads, rows, kHeadDim, (long long)rows * kHeadDim, (long long)heads * rows * kHeadDim, kTileRows);
+bool make_rows_map_bf16(CUtensorMap* map, const void* base, int heads, int rows, bool gradient) {
+    return make_rows_map4(map, base, 1, heads, rows, kHeadDim, (long long)rows * kHeadDim, (long long)heads * rows * kHeadDim,
+                          gradient ? kGradRows : kTileRows);
 }
 bool make_dq_acc_map(CUtensorMap* map, const float* base, size_t rows) { return make_acc_map(map, base, rows); }
 
