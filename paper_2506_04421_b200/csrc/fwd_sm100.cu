@@ -567,9 +567,13 @@ cudaError_t launch_fwd_tc(const CUtensorMap& q, const CUtensorMap& k0, const CUt
     const size_t groups = (BH * args.head_bytes + kL2Bytes - 1) / kL2Bytes;
     a.n_heads = BH;
     a.group_heads = (int)((BH + groups - 1) / groups);
-    a.by_group = FastDiv(args.work != nullptr ? (uint32_t)a.group_heads * (uint32_t)a.n_work : (uint32_t)a.n_work);
-    a.by_group_heads = FastDiv((uint32_t)a.group_heads);
-    a.by_last_heads = FastDiv((uint32_t)((BH - 1) % a.group_heads + 1));
+    if (args.work != nullptr) {
+        a.by_group = FastDiv((uint32_t)a.group_heads * (uint32_t)a.n_work);
+        a.by_group_heads = FastDiv((uint32_t)a.group_heads);
+        a.by_last_heads = FastDiv((uint32_t)((BH - 1) % a.group_heads + 1));
+    } else {
+        a.by_group = FastDiv((uint32_t)a.n_work);
+    }
     a.by_batch = FastDiv((uint32_t)a.heads_per_batch);
     {
         KernelTimer timer(args.work != nullptr ? "hmar_fwd_tc_kernel" : "hmar_fwd_tc_kernel/scale_step", stream);

@@ -27,7 +27,7 @@ struct FastDiv {
     uint32_t mul = 0, shift = 0;
     FastDiv() = default;
     constexpr explicit FastDiv(uint32_t d) {
-        while ((1ull << shift) < d) ++shift;
+        shift = d > 1 ? 32 - __builtin_clz(d - 1) : 0;
         mul = (uint32_t)(((1ull << 32) * ((1ull << shift) - d) + d - 1) / d);
     }
     HMAR_HD constexpr int operator()(int n) const {
