@@ -227,8 +227,8 @@ __device__ __forceinline__ void softmax_grad_half(uint32_t lane_base, int cbase,
 // benchmarks run: the extra address arithmetic and code of the strided one cost it a tenth of its speed).
 // ONE_MASK: every tile goes through the variant of the softmax-gradient code with per-element bounds, so that the
 // block's code holds one variant instead of three.  It is the instantiation for side lists whose tiles are mostly
-// partial or packed (L = 680, 960 heads: 258 us, 322 with three variants); where most steps belong to full tiles the
-// plain variant's shorter arithmetic wins (L = 2240, 384 heads: 879 us, 740 with three).  See kOneMaskBelowPermille.
+// partial or packed (L = 680, 960 heads: whole backward 336 us, 400 with three variants); where most steps belong to full tiles
+// the plain variant's shorter arithmetic wins (share 700: 6 to 9 %).  See kOneMaskBelowPermille.
 template <bool STRIDED, bool ONE_MASK>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -929,10 +929,10 @@ static int sm_count() {
 }
 
 // Side lists with fewer than this share (in thousandths) of their steps in full tiles run the one-variant
-// instantiation.  Main kernel, one variant / three: 0.71 at 200 (L = 399, 768 heads), 0.80 and 0.97 at 421 (L = 680, 960 and
-// 128 heads), 1.07 at 500 (L = 900, four scales of 15), 1.04 at 512 (L = 1060), 1.13 at 709 and 714, 1.15 at 824
-// (L = 2240, 96 heads), 1.22 at 973.  The line was drawn before both instantiations became faster; the crossing is now
-// between 421 and 500.  (Twelve scales of 11 have no full tile and 1.04: their tiles are all cut short alike.)
+// instantiation.  Whole backward, one variant / three: 0.84 at 421 (L = 680, 960 heads; 1.00 with 128), 0.83 at 481 (L = 774, 468
+// heads), 1.00 at 526 (L = 538, 50 heads), 1.02 at 548 (L = 788, 16 heads), 1.00 at 571 (L = 958, 84 heads), 1.02 at 607 (L = 594, 725
+// heads), 1.05 at 642 (L = 875, 30 heads), 1.06 to 1.09 from 690 to 731.  (Four scales of 15, 500: 1.02; twelve of 11, which have no
+// full tile, 1.04 before the masks were bits: their tiles are all cut short alike.)
 constexpr int kOneMaskBelowPermille = 600;
 
 template <bool STRIDED>
