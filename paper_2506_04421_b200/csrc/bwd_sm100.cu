@@ -976,14 +976,8 @@ static cudaError_t launch_bwd_tc_layout(const CUtensorMap& q, const CUtensorMap&
 cudaError_t launch_bwd_tc(const CUtensorMap& q, const CUtensorMap& k, const CUtensorMap& v, const CUtensorMap& dout_map,
                           const CUtensorMap& dq_acc_map, const CUtensorMap& dk_map, const CUtensorMap& dv_map, const BwdArgs& args,
                           const __nv_bfloat16* out, const __nv_bfloat16* dout, __nv_bfloat16* dq, int BH, cudaStream_t stream) {
-    // dense [BH, L, 64] everywhere: the instantiation with compile-time strides
-    const long long row = D, head = (long long)args.L * D;
-    const bool dense = args.in_row == row && args.od_row == row && args.g_row == row && args.in_head == head &&
-                       args.od_head == head && args.g_head == head &&
-                       (args.heads_per_batch == BH || (args.in_batch == args.heads_per_batch * head &&
-                                                       args.od_batch == args.in_batch && args.g_batch == args.in_batch));
-    return dense ? launch_bwd_tc_layout<false>(q, k, v, dout_map, dq_acc_map, dk_map, dv_map, args, out, dout, dq, BH, stream)
-                 : launch_bwd_tc_layout<true>(q, k, v, dout_map, dq_acc_map, dk_map, dv_map, args, out, dout, dq, BH, stream);
+    return bwd_dense(args) ? launch_bwd_tc_layout<false>(q, k, v, dout_map, dq_acc_map, dk_map, dv_map, args, out, dout, dq, BH, stream)
+                           : launch_bwd_tc_layout<true>(q, k, v, dout_map, dq_acc_map, dk_map, dv_map, args, out, dout, dq, BH, stream);
 }
 
 }  // namespace hmar

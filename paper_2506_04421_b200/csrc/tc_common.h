@@ -153,6 +153,29 @@ struct BwdArgs {
     ScaleTable st;
 };
 
+// Whether the backward's tensors are all dense [B*H, L, 64]: the instantiation with compile-time strides.  It takes a head by its
+// number alone, as the tensor maps of one batch of B*H heads do.  Maps of several batches want the head's number inside its batch,
+// also where the batches follow one another: theirs would end before a head past the first batch, whose rows would be loaded as
+// zeros and whose dK and dV would not be stored.
+constexpr bool bwd_dense(const BwdArgs& a) {
+    const long long row = kHeadDim, head = (long long)a.L * kHeadDim;
+    return a.heads_per_batch == a.n_heads && a.in_row == row && a.od_row == row && a.g_row == row && a.in_head == head && a.od_head == head &&
+           a.g_head == head;
+}
+constexpr BwdArgs bwd_layout_example(int heads_per_batch, int n_heads, int L, long long row, long long head, long long batch) {
+    BwdArgs a{};
+    a.heads_per_batch = heads_per_batch;
+    a.n_heads = n_heads;
+    a.L = L;
+    a.in_row = a.od_row = a.g_row = row;
+    a.in_head = a.od_head = a.g_head = head;
+    a.in_batch = a.od_batch = a.g_batch = batch;
+    return a;
+}
+static_assert(bwd_dense(bwd_layout_example(6, 6, 30, 64, 1920, 11520)) && !bwd_dense(bwd_layout_example(3, 6, 30, 64, 1920, 5760)) &&
+              !bwd_dense(bwd_layout_example(3, 6, 30, 576, 64, 17280)) && !bwd_dense(bwd_layout_example(6, 6, 30, 64, 1984, 11904)),
+              "one batch of dense heads; dense batches, the packed layout and heads apart are strided");
+
 size_t fwd_tc_smem_bytes();
 cudaError_t launch_selftest_wait(int* status, cudaStream_t stream);
 cudaError_t launch_bwd_tc(const CUtensorMap& q, const CUtensorMap& k, const CUtensorMap& v, const CUtensorMap& dout_map,
