@@ -433,7 +433,6 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     float x0, x1;
                     f32x2_split(ffma2(f32x2(__uint_as_float(b0[i]), __uint_as_float(b0[i + 1])), sl2_2, m_2), x0, x1);
                     const float p0 = ex2(x0), p1 = ex2(x1);
-                    
                     l_2 = fadd2(l_2, f32x2(p0, p1));
                     packed[i / 2] = pack_bf16(p0, p1);
                 }
@@ -441,10 +440,9 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 if (two) {
 #pragma unroll
                     for (int i = 0; i < 32; i += 2) {
-                    float x0, x1;
-                    f32x2_split(ffma2(f32x2(__uint_as_float(b1[i]), __uint_as_float(b1[i + 1])), sl2_2, m_2), x0, x1);
-                    const float p0 = ex2(x0), p1 = ex2(x1);
-                        
+                        float x0, x1;
+                        f32x2_split(ffma2(f32x2(__uint_as_float(b1[i]), __uint_as_float(b1[i + 1])), sl2_2, m_2), x0, x1);
+                        const float p0 = ex2(x0), p1 = ex2(x1);
                         l_2 = fadd2(l_2, f32x2(p0, p1));
                         packed[i / 2] = pack_bf16(p0, p1);
                     }
@@ -477,16 +475,14 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const uint32_t* src = i < 4 ? b0 + 8 * i : b1 + 8 * (i - 4);
-                    uint4 v4;
-                    uint32_t out4[4];
+                    uint32_t o4[4];
 #pragma unroll
                     for (int t = 0; t < 4; ++t) {
                         float o0, o1;
                         f32x2_split(fmul2(f32x2(__uint_as_float(src[2 * t]), __uint_as_float(src[2 * t + 1])), inv_2), o0, o1);
-                        out4[t] = pack_bf16(o0, o1);
+                        o4[t] = pack_bf16(o0, o1);
                     }
-                    v4 = make_uint4(out4[0], out4[1], out4[2], out4[3]);
-                    *reinterpret_cast<uint4*>(stage + lane * 128 + ((i ^ (lane & 7)) << 4)) = v4;
+                    *reinterpret_cast<uint4*>(stage + lane * 128 + ((i ^ (lane & 7)) << 4)) = make_uint4(o4[0], o4[1], o4[2], o4[3]);
                 }
                 __syncwarp();
                 // Two rounds at a time: a block runs this code once, so what it costs is largely the fetching of it (all eight
