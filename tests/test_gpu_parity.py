@@ -784,19 +784,27 @@ def test_last_query_tiles_with_one_to_four_softmax_warps(side):
     _no_device_error()
 
 
-@pytest.mark.parametrize("B, H", [(1, 1111), (101, 11)])
-def test_forward_in_groups_of_heads_with_a_smaller_last_group(B, H):
+@pytest.mark.parametrize("B, H, packed", [(1, 1111, False), (101, 11, True)])
+def test_forward_in_groups_of_heads_with_a_smaller_last_group(B, H, packed):
     """Q, K, V of 1111 heads are more than two L2s: three groups of heads, the last one smaller.  Every head's rows are those of a
-    call on that head alone, bit for bit."""
+    call on that head alone, bit for bit.  The contiguous call is one batch of 1111 heads; the packed one has 101 batches of 11, so
+    that a head of the smaller group has to be found in its batch too, and gives the contiguous call's bits for every head."""
     sides = (1, 2, 3, 4, 5, 6, 8, 10, 13, 16)
     L = sum(s * s for s in sides)
     g = torch.Generator(device="cuda").manual_seed(11)
     q, k, v = (torch.randn((B, H, L, 64), generator=g, device="cuda").to(torch.bfloat16) for _ in range(3))
-    out, lse = hmar.hmar_attn_fwd(q, k, v, sides, 0.125)
+    if packed:
+        out, lse = hmar.hmar_attn_fwd_packed(torch.stack([t.transpose(1, 2) for t in (q, k, v)], dim=2), sides, 0.125)
+        out = out.transpose(1, 2).contiguous()
+        out_c, lse_c = hmar.hmar_attn_fwd(q, k, v, sides, 0.125)
+        assert torch.equal(out, out_c) and torch.equal(lse, lse_c)
+    else:
+        out, lse = hmar.hmar_attn_fwd(q, k, v, sides, 0.125)
     flat = [t.view(B * H, L, 64) for t in (q, k, v, out)]
     for head in (0, 1, 369, 370, 371, 372, 740, 741, 742, 743, 1109, 1110):
         o1, l1 = hmar.hmar_attn_fwd(*(t[head].view(1, 1, L, 64) for t in flat[:3]), sides, 0.125)
         assert torch.equal(o1.view(L, 64), flat[3][head]) and torch.equal(l1.view(L), lse.view(B * H, L)[head]), head
+    _no_device_error()
 
 
 @pytest.mark.parametrize("noalloc", [False, True])
