@@ -241,8 +241,10 @@ int hmar_schedule_tiles_window(int n_scales, const int* side_lens, int window, i
 
 /* Share, in thousandths, of a head's backward steps (128 key rows x 128 query rows) that belong to full tiles:
  * 128 key rows that all see the tile's whole query range, which the backward kernel processes without mask code.
- * The backward picks its instantiation by it: side lists below 600 run the one that keeps a single, fully
- * masked variant of the softmax-gradient code (smaller code), the others the one with three variants.  Returns a negative hmar_status for a bad side list.  Host only. */
+ * The backward picks its instantiation by it: side lists below 500, or below 700 where their items go head by head (short items of
+ * tensors that exceed L2), run the one that keeps a single, fully masked variant of the softmax-gradient code (smaller code), the
+ * others the one with three variants.  The gradients carry the same bits (dq: to the order of its sums).  Returns a negative
+ * hmar_status for a bad side list.  Host only. */
 int hmar_schedule_bwd_full_tile_share(int n_scales, const int* side_lens, int window);
 
 /* The backward's work items in the order in which its persistent blocks take them, block by block: a backward over

@@ -227,8 +227,8 @@ __device__ __forceinline__ void softmax_grad_half(uint32_t lane_base, int cbase,
 // benchmarks run: the extra address arithmetic and code of the strided one cost it a tenth of its speed).
 // ONE_MASK: every tile goes through the variant of the softmax-gradient code with per-element bounds, so that the
 // block's code holds one variant instead of three.  It is the instantiation for side lists whose tiles are mostly
-// partial or packed (L = 680, 960 heads: whole backward 336 us, 400 with three variants); where most steps belong to full tiles
-// the plain variant's shorter arithmetic wins (share 700: 6 to 9 %).  See kOneMaskBelowPermille.
+// partial or packed (L = 680, 960 heads: whole backward 0.84 of the three variants' time); where most steps belong to full tiles
+// the plain variant's shorter arithmetic wins (share 700, class by class: 4 to 10 %).  See bwd_one_mask.
 template <bool STRIDED, bool ONE_MASK>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 hmar_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -928,13 +928,6 @@ static int sm_count() {
     return cached[dev];
 }
 
-// Side lists with fewer than this share (in thousandths) of their steps in full tiles run the one-variant
-// instantiation.  Whole backward, one variant / three: 0.84 at 421 (L = 680, 960 heads; 1.00 with 128), 0.83 at 481 (L = 774, 468
-// heads), 1.00 at 526 (L = 538, 50 heads), 1.02 at 548 (L = 788, 16 heads), 1.00 at 571 (L = 958, 84 heads), 1.02 at 607 (L = 594, 725
-// heads), 1.05 at 642 (L = 875, 30 heads), 1.06 to 1.09 from 690 to 731.  (Four scales of 15, 500: 1.02; twelve of 11, which have no
-// full tile, 1.04 before the masks were bits: their tiles are all cut short alike.)
-constexpr int kOneMaskBelowPermille = 600;
-
 template <bool STRIDED>
 static cudaError_t launch_bwd_tc_layout(const CUtensorMap& q, const CUtensorMap& k, const CUtensorMap& v, const CUtensorMap& dout_map,
                                         const CUtensorMap& dq_acc_map, const CUtensorMap& dk_map, const CUtensorMap& dv_map, const BwdArgs& args,
@@ -955,7 +948,7 @@ static cudaError_t launch_bwd_tc_layout(const CUtensorMap& q, const CUtensorMap&
         BwdArgs a = args;
         a.by_head = bwd_by_head(args.head_steps, args.n_work, n_rows);
         static SmemOptIn opt_in[2];
-        const bool one_mask = args.plain_permille < kOneMaskBelowPermille;
+        const bool one_mask = bwd_one_mask(args.plain_permille, a.by_head);
         auto kernel = one_mask ? hmar_bwd_tc_kernel<STRIDED, true> : hmar_bwd_tc_kernel<STRIDED, false>;
         cudaError_t e = opt_in[one_mask]((const void*)kernel, smem);
         if (e == cudaSuccess) e = launch_overlapped(kernel, grid, NUM_THREADS, smem, stream, q, k, v, dout_map, dq_acc_map, dk_map, dv_map, a);

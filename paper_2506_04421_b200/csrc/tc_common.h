@@ -105,6 +105,15 @@ inline bool bwd_by_head(int head_steps, int n_work, size_t n_rows) {
     return head_steps < 4 * n_work && n_rows * row_bytes > kL2Bytes + kL2Bytes / 4;
 }
 
+// Whether the backward runs the instantiation whose code holds one variant of the softmax-gradient code, with a bit per column, and
+// not three (none, rows only, columns).  It is the better one where few steps belong to full tiles, and the line lies higher where
+// the items go head by head: tiles of all kinds follow one another there, and with them the variants of the code.  Whole backward, one
+// variant / three.  Class by class, 25 000 to 190 000 rows: mean 0.94 (0.79 to 1.01) at shares of 330 to 400, 0.99 (0.83 to 1.04)
+// from 400 to 500, 1.02 (0.95 to 1.07; a single list of 500: 0.94) from 515 to 570, 1.05 (0.98 to 1.12) above.  Head by head, 230 000 to
+// 800 000 rows: 0.84 (0.74 to 0.95) up to 490, 0.93 (0.82 to 1.02) to 600, 0.94 (0.81 to 1.04) to 700, 0.98 (0.87 to 1.05) to
+// 900, 1.04 (1.01 to 1.07) above.  (L = 680, share 421: 0.84 with 960 heads, 1.00 with 128.)
+inline bool bwd_one_mask(int plain_permille, bool by_head) { return plain_permille < (by_head ? 700 : 500); }
+
 // The item that a block takes in a round: returns its tile and sets its head, or returns -1 where there are no more.
 // A head's tiles are ordered by cost; tiles of equal cost are one class.  The launch works class by class, head by head
 // inside a class (by_head: all tiles are one class), and the items are dealt to the blocks round by round, back and forth.
@@ -127,7 +136,7 @@ struct BwdArgs {
     const BwdWork* work;
     int n_work;
     int n_heads;             // B * H
-    int plain_permille;      // from bwd_plain_permille: picks the instantiation of the main kernel
+    int plain_permille;      // from bwd_plain_permille: picks the instantiation of the main kernel, see bwd_one_mask
     int head_steps;          // steps of all tiles of a head (from bwd_fill_classes)
     int by_head;             // set by the launcher (bwd_by_head)
     int L;

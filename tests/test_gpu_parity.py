@@ -906,6 +906,20 @@ def test_a_refused_launch_leaves_no_error_behind(name):
     _no_device_error()
 
 
+@pytest.mark.parametrize("sides, H", [((11, 16, 8), 522), ((16, 16, 9, 4, 13), 296)])
+def test_backward_head_by_head_and_class_by_class_give_the_same_bits(sides, H):
+    """Tensors over L2 whose items are short go head by head, and shares of full tiles from 500 to 700 then take the backward's
+    one-variant instantiation where a few of the same heads, class by class, take the other one (600 here; the second list, 761, takes
+    the one with three variants either way).  Against the oracle, and dK and dV bit for bit against the call on those heads alone."""
+    wl = _Wl(sides, B=1, H=H)
+    heads = _partition_heads(wl, 6)
+    dev, out, lse, grads = _check_sampled(wl, heads, hmar.HMAR_WINDOW_MARKOV, "markov", True, 6)
+    few = [t[:, heads].contiguous() for t in (dev["q"], dev["k"], dev["v"], out, lse, dev["dout"])]
+    _, dk, dv = hmar.hmar_attn_bwd(*few, wl.side_lens, wl.softmax_scale)
+    assert torch.equal(dk, grads[1][:, heads]) and torch.equal(dv, grads[2][:, heads])
+    _no_device_error()
+
+
 def test_edge_cases_through_the_checking_build():
     """The library compiled with -DHMAR_BOUNDS_CHECK compares every address its kernels form by their own
     arithmetic (plain loads and stores; TMA copies are clipped by the hardware) with the extent of its tensor and
