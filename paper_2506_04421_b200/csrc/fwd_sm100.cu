@@ -26,8 +26,11 @@
 //               without the redistribution the softmax warps spill and the kernel is 4 % slower)
 // TMEM columns: S/P [0,64), O [64,128).
 // Registers: the block starts with 64 per thread (four blocks per SM); the softmax warpgroup raises its
-// to 96 and the second warpgroup drops to 32 (setmaxnreg), the same total.  (88 and 40 leave spills in the softmax loop: L = 680
-// 960 heads 116.6 us against 115, L = 2240 384 heads 337.6 against 330; 104 and 24 spill in the other warps, 1 % slower.)
+// to 96 and the second warpgroup drops to 32 (setmaxnreg), the same total.  24 bytes are spilled then, 44 with 88 and 40 (L = 680
+// 960 heads 114.4 -> 115.6 us, inference step 13 -> 18 1536 heads 138.2 -> 140.2), 60 with 104 and 24 (1 % slower).
+// A time in these comments is that of the kernel in a row of some tens of launches, caches as the launch before leaves them, both sides
+// of a pair in turn on one GPU.  Pairs of different dates do not add up: a block of the step 13 -> 18 lives 26 500 clocks, and the
+// launch takes 123 us on a GPU that was idle before (SMs at 1.8 GHz inside the kernel) and 139 to 143 at the power limit (1.61 to 1.65).
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -95,13 +98,6 @@ __device__ __forceinline__ KvTile kv_tile(const FwdWork& w, int tiles0, int j) {
 
 // columns issued for a tile with n_valid keys (a multiple of 16)
 __device__ __forceinline__ int tile_cols(int n_valid) { return (n_valid + 15) & ~15; }
-
-// Maximum of three in one instruction (in pairs: L = 680 960 heads 115.2 -> 114 us, inference step 13 -> 18 1536 heads 131 -> 128.5).
-__device__ __forceinline__ float max3(float a, float b, float c) {
-    float d;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
 
 template <int N> __device__ __forceinline__ void reg_inc() {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
@@ -391,10 +387,10 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 }
                 float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};     // four chains of maxima, not one of 64
 #pragma unroll
-                for (int i = 0; i < 32; i += 2) mx4[i / 2 & 3] = max3(mx4[i / 2 & 3], __uint_as_float(b0[i]), __uint_as_float(b0[i + 1]));
+                for (int i = 0; i < 32; ++i) mx4[i & 3] = fmaxf(mx4[i & 3], __uint_as_float(b0[i]));
                 if (two) {
 #pragma unroll
-                    for (int i = 0; i < 32; i += 2) mx4[i / 2 & 3] = max3(mx4[i / 2 & 3], __uint_as_float(b1[i]), __uint_as_float(b1[i + 1]));
+                    for (int i = 0; i < 32; ++i) mx4[i & 3] = fmaxf(mx4[i & 3], __uint_as_float(b1[i]));
                 }
                 const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * sl2;     // softmax_scale > 0
 
@@ -423,8 +419,9 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 
                 // P = 2^(s * scale - m): fp32 row sum, bf16 P written over the S columns already read.  Pairs of logits share an
                 // instruction but for the exponential: with the exponentials' pipe 85 % busy while four blocks are in their loops,
-                // the issue slots between them count (with O / l in pairs too: L = 680 960 heads 118 -> 114.5 us, L = 2240 384 heads
-                // 341 -> 332, inference step 13 -> 18 1536 heads 135 -> 129.5, 24 -> 32 384 heads 226.7 -> 220).
+                // the issue slots between them count (one by one: L = 680 960 heads 114.1 -> 117.1 to 118.8 us, L = 2240 384 heads 2 to 8 %,
+                // inference step 13 -> 18 1536 heads 138 -> 141, 24 -> 32 384 heads 239 -> 245.5).  The compiler takes the maxima above by
+                // threes on its own, and O / l in pairs changes nothing.
                 uint32_t packed[16];
                 const uint64_t sl2_2 = f32x2(sl2, sl2), m_2 = f32x2(-m_sub, -m_sub);
                 uint64_t l_2 = f32x2(0.f, 0.f);
@@ -461,7 +458,6 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             if (ok) {
                 tc_fence_after();
                 const float inv = 1.f / l;
-                const uint64_t inv_2 = f32x2(inv, inv);
                 tmem_ld32(o_addr, b0);
                 tmem_ld32(o_addr + 32, b1);
                 tmem_ld_wait();
@@ -475,14 +471,12 @@ hmar_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const uint32_t* src = i < 4 ? b0 + 8 * i : b1 + 8 * (i - 4);
-                    uint32_t o4[4];
-#pragma unroll
-                    for (int t = 0; t < 4; ++t) {
-                        float o0, o1;
-                        f32x2_split(fmul2(f32x2(__uint_as_float(src[2 * t]), __uint_as_float(src[2 * t + 1])), inv_2), o0, o1);
-                        o4[t] = pack_bf16(o0, o1);
-                    }
-                    *reinterpret_cast<uint4*>(stage + lane * 128 + ((i ^ (lane & 7)) << 4)) = make_uint4(o4[0], o4[1], o4[2], o4[3]);
+                    uint4 v4;
+                    v4.x = pack_bf16(__uint_as_float(src[0]) * inv, __uint_as_float(src[1]) * inv);
+                    v4.y = pack_bf16(__uint_as_float(src[2]) * inv, __uint_as_float(src[3]) * inv);
+                    v4.z = pack_bf16(__uint_as_float(src[4]) * inv, __uint_as_float(src[5]) * inv);
+                    v4.w = pack_bf16(__uint_as_float(src[6]) * inv, __uint_as_float(src[7]) * inv);
+                    *reinterpret_cast<uint4*>(stage + lane * 128 + ((i ^ (lane & 7)) << 4)) = v4;
                 }
                 __syncwarp();
                 // Two rounds at a time: a block runs this code once, so what it costs is largely the fetching of it (all eight
