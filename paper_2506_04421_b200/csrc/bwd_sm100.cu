@@ -35,10 +35,11 @@
 // two warpgroups lower theirs (setmaxnreg) within the same total.
 // The SMs of a cluster share the instruction cache behind the small per-partition one, and this kernel's
 // speed depends on how much code it streams through it: changes that only add instructions (more unrolled
-// variants, code that never runs) have cost up to a tenth of the time, so variants are kept few.  (94 to 96 % of the
+// variants, code that never runs) have cost up to a tenth of the time, so variants are kept few.  (96 to 97 % of the
 // requests hit now, 67 to 92 % while each wait carried a timer and a report of its own.)
-// What bounds the steady loop is the 128-byte port of shared memory: per 128 x 128 step (2 830 clocks on average at L = 2240) the
-// tensor core takes 877 of its cycles, the LSU 990, the copies of Q and dO 256 and the copy engine's reading of staged dQ 256.
+// What bounds it at L = 2240 is the 128-byte port of shared memory: per 128 x 128 step (2 780 clocks on average, item ends included;
+// 2 450 in the steady loop) the tensor core takes 877 of its cycles, the LSU 961 (loads 326, stores 593, barriers 42),
+// the copies of Q and dO 256 and the copy engine's reading of staged dQ 256: 2 350, averages of a whole launch like the 2 780.
 // Hand-overs rearranged, more warps or more issuers leave that as it is, and none of them made the kernel faster.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -150,7 +151,7 @@ __device__ __forceinline__ void load_swizzled_row(const uint8_t* tile, int r, ui
 // P^T = 2^(S^T * scale * log2e - lse * log2e) and dS^T = P^T o (dP^T - delta) in fp32.
 // S^T and dP^T are read 16 key rows at a time in the layout in which a thread holds, of two rows, the
 // column pairs 8k + 2(t % 4) + {0, 1}: a thread then needs lse and delta of 16 columns only (eight 8-byte
-// loads each, one shared-memory wavefront per load; one key row per thread would need all 64 columns as
+// loads each, two shared-memory wavefronts per load, counted: 256 of a step's 326; one key row per thread would need all 64 columns as
 // broadcast loads, which were the largest share of the shared-memory traffic of the LSU).  A column pair
 // packs into one bf16x2: P^T goes back to TMEM over S^T and dS^T over dP^T with the matching store layout
 // (the 32 packed columns start at the half's first column, which this warp has already read for these
@@ -223,8 +224,9 @@ __device__ __forceinline__ void softmax_grad_half(uint32_t lane_base, int cbase,
 }
 
 // STRIDED: the bf16 tensors have the strides given in the arguments (packed projection layouts); otherwise they are
-// dense [BH, L, 64] and every address is formed with compile-time strides (the dense instantiation is the one the
-// benchmarks run: the extra address arithmetic and code of the strided one cost it a tenth of its speed).
+// dense [BH, L, 64] and every address is formed with compile-time strides.  Dense tensors through the strided one, whole
+// backward: L = 680 960 heads 381.6 -> 397.8 us, 128 heads 59.9 -> 60.6, 16 heads 16.6 -> 17.0, L = 2240 384 heads 829 -> 838; equal from
+// L = 1600 with 39 heads to L = 9451 with 48.  (9 % in an earlier form of the kernel.)
 // ONE_MASK: every tile goes through the variant of the softmax-gradient code with per-element bounds, so that the
 // block's code holds one variant instead of three.  It is the instantiation for side lists whose tiles are mostly
 // partial or packed (L = 680, 960 heads: whole backward 0.84 of the three variants' time); where most steps belong to full tiles

@@ -21,7 +21,7 @@ struct FwdWork {
 // Division of numbers below 2^31 by a number that the host knows: q = (hi(n * mul) + n) >> shift with mul = 2^32 * (2^shift / d - 1)
 // rounded up and shift = ceil(log2(d)) (Granlund and Montgomery, "Division by invariant integers using multiplication").
 // A division by a variable is some forty instructions, and every block of the forward began with three of them, in all of its
-// warps: 1 100 clocks of a block's 11 000 to 69 000.  L = 680 960 heads 127 -> 121 us, L = 2240 384 heads 346 -> 338, L = 384 128
+// warps: 1 100 clocks of a block's 11 000 to 69 000.  Kernel times, taken as fwd_sm100.cu says: L = 680 960 heads 127 -> 121 us, L = 2240 384 heads 346 -> 338, L = 384 128
 // heads 17.7 -> 16.6, inference step 13 -> 18 1536 heads 143 -> 139, 24 -> 32 384 heads 224 -> 219.5.
 struct FastDiv {
     uint32_t mul = 0, shift = 0;
